@@ -131,8 +131,8 @@ PE_API int pe_field(const int64_t* rho_fx, int32_t ncell, double dx, int32_t s_w
                     uint32_t* status, void* stream);
 
 /* pe_field with a boundary (PE_BOUNDARY_*). With PE_BOUNDARY_ABSORBING the equations at the
- * wall nodes use the mirror ghosts and twice the deposit, E is 0 on the walls, and the
- * Jacobian solve runs in FP64 (vacuum regions make it ill-conditioned for FP32).
+ * wall nodes use the mirror ghosts and twice the deposit, and E is 0 on the walls (vacuum
+ * regions make the Jacobian ill-conditioned: the solve takes more Newton updates there).
  * pe_field is pe_field_ex with PE_BOUNDARY_PERIODIC. */
 PE_API int pe_field_ex(const int64_t* rho_fx, int32_t ncell, double dx, int32_t s_w, int32_t mode,
                        int32_t boundary, double tol, int32_t maxit, double* phi, double* E, float* Ef,

@@ -95,15 +95,12 @@ struct pe_batch {
     int block, priv;  // particle launch shape: threads per block, shared-memory deposit window
     int nitems;
     int max_ncell, max_nb;
-    // Field-solve groups, one launch each: (cluster size G) x (FP32 | FP64 Jacobian solve; FP64
-    // only for bounded grids with kWallsJacobianFP64). The batch sizes clusters for throughput
-    // (newton_batch_cluster_size), so its solves can differ from a lone context's in the last
-    // bits (the same equations, another partition of the linear solve); both converge to the
-    // Newton tolerance.
+    // Field-solve groups, one launch each: the realisations of one grid size. The batch sizes
+    // clusters for throughput (newton_batch_cluster_size), so its solves can differ from a lone
+    // context's in the last bits (the same equations, another partition of the linear solve);
+    // both converge to the Newton tolerance.
     struct FieldGroup {
-        int G;
-        bool fp64;
-        int maxn;
+        int ncell;
         std::vector<int> ids;
     };
     std::vector<FieldGroup> fgroups;
@@ -205,7 +202,7 @@ static int field_all(pe_batch* b, bool extrap)
         const int n = (int)fg.ids.size();
         cudaStream_t s = fork ? b->side[k] : b->stream;
         if (fork && cudaStreamWaitEvent(s, b->ev_fork, 0) != cudaSuccess) return PE_ECUDA;
-        PE_TRY(launch_newton_batch(base + field_desc_size() * o, n, fg.G, fg.maxn, fg.fp64, extrap, s));
+        PE_TRY(launch_newton_batch(base + field_desc_size() * o, n, fg.ncell, extrap, s));
         if (fork && cudaEventRecord(b->ev_join[k], s) != cudaSuccess) return PE_ECUDA;
         o += (size_t)n;
     }
@@ -294,22 +291,19 @@ extern "C" PE_API int pe_batch_create(pe_ctx* const* ctxs, int32_t n, void* scra
         so += 2 * (int64_t)x->nb;
         if (x->nb > b->max_nb) b->max_nb = x->nb;
         if (x->cfg.ncell > b->max_ncell) b->max_ncell = x->cfg.ncell;
-        const int G = newton_batch_cluster_size(x->cfg.ncell);
-        if (G < 1) {
+        if (newton_batch_cluster_size(x->cfg.ncell) < 1) {
             cudaEventDestroy(b->ev_in);
             cudaEventDestroy(b->ev_out);
             delete b;
             return PE_EINVAL;
         }
-        const bool fp64 = x->walls != 0 && kWallsJacobianFP64;
         bool placed = false;
         for (auto& fg : b->fgroups)
-            if (fg.G == G && fg.fp64 == fp64) {
+            if (fg.ncell == x->cfg.ncell) {
                 fg.ids.push_back(r);
-                if (x->cfg.ncell > fg.maxn) fg.maxn = x->cfg.ncell;
                 placed = true;
             }
-        if (!placed) b->fgroups.push_back({G, fp64, x->cfg.ncell, {r}});
+        if (!placed) b->fgroups.push_back({x->cfg.ncell, {r}});
     }
     int rc = PE_OK;
     if (cudaEventCreateWithFlags(&b->ev_fork, cudaEventDisableTiming) != cudaSuccess) rc = PE_ECUDA;

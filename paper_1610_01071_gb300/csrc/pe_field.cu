@@ -18,50 +18,94 @@ namespace cg = cooperative_groups;
 
 namespace pe {
 
-constexpr int kClusterMinCells = 512;  // grids at least this large use the multi-SM solver
-
 // ---------------------------------------------------------------------------------
-// Production solver: one thread-block cluster of G blocks (G = 1 for small grids, up to
-// 16 for large ones, one block per SM); block g owns the B = ncell / G nodes
-// [g B, (g+1) B), one node per thread.
+// Solver: one thread-block cluster of G blocks (G = 1 for small grids, up to 16 for large ones,
+// one block per SM); block g owns the B = ncell / G nodes [g B, (g+1) B), one node per thread.
+//
+// What bounds it: latency. An FP64 instruction (a conversion to or from FP64 among them) holds
+// its scheduler's FP64 pipe for 64-76 cycles whatever is independent around it (measured: 76
+// cycles per warp instruction with one warp on each of the SM's four schedulers, 152 with two,
+// 304 with four), so the time is the number of FP64 instructions per node times the warps per
+// scheduler, plus the exchanges between warps and blocks. Hence
+//  - FP64 only where the result needs it: the potential, its residual, exp(phi). Conversions
+//    between FP32, FP64 and the fixed-point charge are integer operations (bits of the formats);
+//    the convergence test runs in FP32;
+//  - exp(phi) is evaluated once and then carried multiplicatively, exp(phi + x) = exp(phi) exp(x),
+//    with a Taylor polynomial whose degree follows the largest update;
+//  - one block barrier and one cluster barrier per linear solve: every warp solves the block's
+//    and the cluster's separator systems itself instead of waiting for one warp's result. The
+//    second exchange of an iteration (largest update) runs behind the FP64 update.
+// One solve of a time loop (two updates; the walls' about seven) takes 7.1 us on 128 nodes (15.1
+// us before these points), 10.4 on 1024 (18.0), 12.8 on 4096 (23.3) and 37 on 8192 with walls (60).
 //
 // Precision: phi, exp(phi), the Newton residual and the update are FP64; the Jacobian
-// correction J d = -F is solved in FP32 on periodic grids. This is Newton's method with an
-// inexact linear solve (mixed-precision iterative refinement): the FP64 residual drives the
-// iteration, so it converges to the FP64 solution of the discrete equation, while the
-// FP32 solve only bounds the final contraction rate (~ cond(J) 2^-24 per iteration).
-// Bounded grids with vacuum regions have exp(phi) ~ 1e-6 there and cond(J) ~ 1e7: the FP32
-// solve still contracts, but slowly (7 Newton iterations instead of 3 on an 8192-node slab from
-// a warm start); it remains the faster solve (kWallsJacobianFP64 selects the FP64 elimination,
-// template parameter T).
-// On this GPU a dependent FP64 instruction costs ~100 cycles and the FP64 pipe retires
-// ~2 lanes per cycle per SM, so FP64 is used only for per-node work, spread over many
-// warps and SMs, and kept off the serial chains of the tridiagonal elimination.
+// correction J d = -F is solved in FP32. This is Newton's method with an inexact linear solve
+// (mixed-precision iterative refinement): the FP64 residual drives the iteration, so it converges
+// to the FP64 solution of the discrete equation, while the FP32 solve only bounds the final
+// contraction rate (~ cond(J) 2^-24 per iteration). Bounded grids with vacuum regions have
+// exp(phi) ~ 1e-6 there and cond(J) ~ 1e7: the FP32 solve still contracts, but slowly (7 Newton
+// iterations instead of 2 on an 8192-node slab from a warm start); an FP64 elimination needs 3,
+// but each costs several times as much.
 //
 // Linear solve (nested separators, scalar tridiagonal systems only): the last row of every
 // warp is a separator, and the last row of every block is a separator of the cluster. Each
 // warp solves its other rows (its interior) by parallel cyclic reduction with register
 // shuffles, with the couplings to the two separators around it moved to two extra right-hand
 // sides (x = y - g S_left - h S_right). Substituting the interiors next to a separator into
-// its row leaves a scalar tridiagonal system over the separators: one warp of the block solves
-// the block's warp separators in terms of the two block separators around them, and one warp
-// of every block solves the cyclic system of the cluster's block separators, whose rows every
-// block pushes into every other block's shared memory before the cluster barrier. exp(phi) is
-// evaluated once per solve and then carried multiplicatively, exp(phi + s d) = exp(phi)
-// exp(s d), with a Taylor polynomial.
+// its row leaves a scalar tridiagonal system over the separators: every warp solves the block's
+// warp separators in terms of the two block separators around them, and the cyclic system of the
+// cluster's block separators, whose rows every block pushes into every other block's shared
+// memory before the cluster barrier.
 //
-// Stopping: besides max |update| < tol, the iteration stops before a linear solve when the
-// residual already bounds the next update below tol. The Jacobian J = L + diag(g'(phi)) has
-// L symmetric with zero row sums and non-positive off-diagonals (periodic or mirror-wall
-// rows), so J is an M-matrix with row sums g'(phi_j) and ||J^-1||_inf <= 1 / min_j g'(phi_j):
-// the next Newton update is at most max|F| / min g' in every component.
+// Stopping, besides max |update| < tol: J = L + diag(g'(phi)) has L symmetric with zero row sums
+// and non-positive off-diagonals (periodic or mirror-wall rows), so J is an M-matrix with row
+// sums g'(phi_j) and ||J^-1||_inf <= 1 / min_j g'(phi_j): the next update is at most max|F| /
+// min g' in every component. Before a linear solve |F| is the FP64 residual; after one, the
+// residual that the update leaves is bounded in FP32 as |r - J x| + g x^2 (1/2 + |x|) plus the
+// rounding of that evaluation, which ends the usual solve after its second update without a
+// third residual and reduction only to learn that it has converged.
 
+constexpr int kClusterMinCells = 512;   // grids at least this large use the multi-SM solver
 constexpr int kClusterMax = 16;
 constexpr int kNewtonMaxThreads = 512;  // nodes (threads) per block: 16 blocks cover the largest grid
+constexpr int kNewtonMaxWarps = kNewtonMaxThreads / 32;
+
+// Conversions on the integer pipe (their FP64-pipe instructions hold the pipe as long as an FMA).
+// FP64 to FP32, round to nearest even; magnitudes below FP32's normal range give 0, those of
+// 2^127 and above infinity.
+__device__ __forceinline__ float f32_of(double v)
+{
+    const uint32_t hi = (uint32_t)__double2hiint(v), lo = (uint32_t)__double2loint(v);
+    const uint32_t mag = hi & 0x7FFFFFFFu, sign = hi & 0x80000000u;
+    uint32_t b = __funnelshift_l(lo, mag - (896u << 20), 3);
+    b += ((lo & 0x1FFFFFFFu) + 0x0FFFFFFFu + (b & 1u)) >> 29;
+    if (mag < 0x38100000u) b = 0u;
+    if (mag >= 0x47E00000u) b = (mag > 0x7FF00000u || (mag == 0x7FF00000u && lo)) ? 0x7FC00000u : 0x7F800000u;
+    return __uint_as_float(b | sign);
+}
+
+// FP32 to FP64 (exact); subnormal numbers give 0.
+__device__ __forceinline__ double f64_of(float x)
+{
+    const uint32_t b = __float_as_uint(x), mag = b & 0x7FFFFFFFu, sign = b & 0x80000000u;
+    const uint32_t hi = mag >= 0x7F800000u ? 0x7FF00000u | ((mag & 0x007FFFFFu) >> 3) : (mag >> 3) + (896u << 20);
+    return mag < 0x00800000u ? 0.0 : __hiloint2double((int)(hi | sign), (int)(mag << 29));
+}
+
+// v 2^-shift, round to nearest even: the fixed-point charge as a density.
+__device__ __forceinline__ double fixed_to_double(long long v, int shift)
+{
+    const unsigned long long u = v < 0 ? 0ull - (unsigned long long)v : (unsigned long long)v;
+    const int lz = __clzll((long long)u);
+    const unsigned long long m = u << (lz & 63);  // the leading bit at bit 63: 53 bits and 11 below them
+    const unsigned long long r = (m >> 11) + (((m & 0x7FFull) + 0x3FFull + ((m >> 11) & 1ull)) >> 11);
+    // r holds the implicit bit (and may have carried into the next power of two)
+    const unsigned long long bits = ((unsigned long long)(1085 - lz - shift) << 52) + r;
+    return u == 0ull ? 0.0 : __longlong_as_double((long long)(bits | ((unsigned long long)v & (1ull << 63))));
+}
 
 // exp(x) for |x| <= 2^-5 by its Taylor polynomial to degree 8 (relative error < 1e-18),
-// evaluated by Estrin's scheme: a dependent FP64 operation costs ~100 cycles here, and the
-// scheme's dependency depth is 5 instead of the 9 of Horner's rule.
+// evaluated by Estrin's scheme.
 __device__ __forceinline__ double exp_small(double x)
 {
     const double x2 = x * x, x4 = x2 * x2;
@@ -71,49 +115,46 @@ __device__ __forceinline__ double exp_small(double x)
     return fma(x4, fma(x4, 1.0 / 40320.0, hi), lo);
 }
 
-// exp(x) for |x| <= 2^-10 to degree 4 (relative error < 1e-17), dependency depth 3.
+// exp(x) for |x| <= 2^-10 to degree 4 (relative error < 1e-17).
 __device__ __forceinline__ double exp_tiny(double x)
 {
     const double x2 = x * x;
     return fma(x2, fma(x2, 1.0 / 24.0, fma(x, 1.0 / 6.0, 0.5)), 1.0 + x);
 }
 
-// Reciprocal for the elimination (and the 2x2 inverses of the boundary system): the fast FP32
-// reciprocal (__fdividef, within 2 ulp for the diagonal magnitudes that occur here), or in
-// FP64 two Newton-Raphson steps r <- r (2 - x r) from it (each step squares the relative
-// error, 2^-22 -> 2^-44 -> 2^-88), which avoids the long division sequences on the
-// reductions' serial chains. The FP32 solve is the inexact linear solve of a Newton
-// iteration whose residual is FP64, so a 2-ulp reciprocal only changes its contraction rate.
+// Reciprocal of the elimination: the fast FP32 reciprocal (__fdividef, within 2 ulp for the
+// diagonal magnitudes that occur here). The FP32 solve is the inexact linear solve of a Newton
+// iteration whose residual is FP64, so this only changes its contraction rate.
 __device__ __forceinline__ float recip(float x) { return __fdividef(1.0f, x); }
-__device__ __forceinline__ double recip(double x)
+
+// Warp maximum / minimum of non-negative floats by their bits (a NaN counts as the largest).
+__device__ __forceinline__ float warp_max_bits(uint32_t v)
 {
-    double r = (double)__fdividef(1.0f, (float)x);
-    r = r * fma(-x, r, 2.0);
-    return r * fma(-x, r, 2.0);
+    return __uint_as_float(__reduce_max_sync(0xFFFFFFFFu, v));
+}
+__device__ __forceinline__ float warp_min_bits(float v)
+{
+    return __uint_as_float(__reduce_min_sync(0xFFFFFFFFu, __float_as_uint(v)));
 }
 
 // Parallel cyclic reduction of a scalar tridiagonal system held by lanes 0 .. n-1 of the
 // calling warp (n a power of two, <= 32; all 32 lanes call it; a lane without a row holds the
 // identity row). Row k: a x_{k-1} + b x_k + c x_{k+1} = r (three right-hand sides r0, r1,
-// r2). cyclic: rows couple to (k +- 1) mod n; else the chain ends at 0 and n - 1. Returns
-// x_k for each right-hand side (after the last step of a cyclic system its remaining
-// couplings reach the row itself and are folded into the diagonal).
-template <typename T>
-__device__ __forceinline__ void warp_scalar_pcr(T a, T b, T c, T r0, T r1, T r2, int n, bool cyclic, T& x0, T& x1,
-                                                T& x2)
+// r2); the chain ends at 0 and n - 1. Returns x_k for each right-hand side.
+__device__ __forceinline__ void warp_chain_pcr(float a, float b, float c, float r0, float r1, float r2, int n, float& x0,
+                                               float& x1, float& x2)
 {
     const int k = threadIdx.x & 31;
     for (int s = 1; s < n; s <<= 1) {
-        const int km = (k - s + n) % n, kp = (k + s) % n;
-        const T am = __shfl_sync(0xFFFFFFFFu, a, km), bm = __shfl_sync(0xFFFFFFFFu, b, km);
-        const T cm = __shfl_sync(0xFFFFFFFFu, c, km), q0m = __shfl_sync(0xFFFFFFFFu, r0, km);
-        const T q1m = __shfl_sync(0xFFFFFFFFu, r1, km), q2m = __shfl_sync(0xFFFFFFFFu, r2, km);
-        const T ap = __shfl_sync(0xFFFFFFFFu, a, kp), bp = __shfl_sync(0xFFFFFFFFu, b, kp);
-        const T cp = __shfl_sync(0xFFFFFFFFu, c, kp), q0p = __shfl_sync(0xFFFFFFFFu, r0, kp);
-        const T q1p = __shfl_sync(0xFFFFFFFFu, r1, kp), q2p = __shfl_sync(0xFFFFFFFFu, r2, kp);
-        const bool hm = k < n && (cyclic || k >= s), hp = k < n && (cyclic || k + s < n);
-        const T al = hm ? a * recip(bm) : T(0);
-        const T ga = hp ? c * recip(bp) : T(0);
+        const int km = (k - s) & (n - 1), kp = (k + s) & (n - 1);
+        const float am = __shfl_sync(0xFFFFFFFFu, a, km), bm = __shfl_sync(0xFFFFFFFFu, b, km);
+        const float cm = __shfl_sync(0xFFFFFFFFu, c, km), q0m = __shfl_sync(0xFFFFFFFFu, r0, km);
+        const float q1m = __shfl_sync(0xFFFFFFFFu, r1, km), q2m = __shfl_sync(0xFFFFFFFFu, r2, km);
+        const float ap = __shfl_sync(0xFFFFFFFFu, a, kp), bp = __shfl_sync(0xFFFFFFFFu, b, kp);
+        const float cp = __shfl_sync(0xFFFFFFFFu, c, kp), q0p = __shfl_sync(0xFFFFFFFFu, r0, kp);
+        const float q1p = __shfl_sync(0xFFFFFFFFu, r1, kp), q2p = __shfl_sync(0xFFFFFFFFu, r2, kp);
+        const float al = (k < n && k >= s) ? a * recip(bm) : 0.0f;
+        const float ga = (k + s < n) ? c * recip(bp) : 0.0f;
         a = -al * am;
         c = -ga * cp;
         b = b - al * cm - ga * ap;
@@ -121,48 +162,51 @@ __device__ __forceinline__ void warp_scalar_pcr(T a, T b, T c, T r0, T r1, T r2,
         r1 = r1 - al * q1m - ga * q1p;
         r2 = r2 - al * q2m - ga * q2p;
     }
-    const T bt = cyclic ? a + b + c : b;
-    const T rb = recip(bt);
+    const float rb = recip(b);
     x0 = r0 * rb;
     x1 = r1 * rb;
     x2 = r2 * rb;
 }
 
-// Parameters of one field solve (one realisation).
-struct FieldDesc {
-    const long long* rho;
-    double* phi;
-    double* E;
-    float* Ef;
-    int* diag;
-    uint32_t* status;
-    double dx, nscale, tol;
-    int ncell, mode, maxit, walls;  // walls: 1 for a bounded grid
-    // Newton start: phi_prev (may be null) keeps the solution before the current one; with
-    // extrap the start is the linear extrapolation 2 phi - phi_prev (solves one fine step apart)
-    double* phi_prev;
-    int extrap, pad2;
-};
+// The same for a cyclic system (rows couple to (k +- 1) mod n) with one right-hand side, lane k
+// holding row k mod n; returns x_{k mod n} on every lane (after the last step the remaining
+// couplings reach the row itself and are folded into the diagonal).
+__device__ __forceinline__ float warp_cyclic(float a, float b, float c, float r, int n)
+{
+    const int k = threadIdx.x & 31;
+    for (int s = 1; s < n; s <<= 1) {
+        const int km = (k - s) & (n - 1), kp = (k + s) & (n - 1);
+        const float am = __shfl_sync(0xFFFFFFFFu, a, km), bm = __shfl_sync(0xFFFFFFFFu, b, km);
+        const float cm = __shfl_sync(0xFFFFFFFFu, c, km), rm = __shfl_sync(0xFFFFFFFFu, r, km);
+        const float ap = __shfl_sync(0xFFFFFFFFu, a, kp), bp = __shfl_sync(0xFFFFFFFFu, b, kp);
+        const float cp = __shfl_sync(0xFFFFFFFFu, c, kp), rp = __shfl_sync(0xFFFFFFFFu, r, kp);
+        const float al = a * recip(bm), ga = c * recip(bp);
+        a = -al * am;
+        c = -ga * cp;
+        b = b - al * cm - ga * ap;
+        r = r - al * rm - ga * rp;
+    }
+    return r * recip(a + b + c);
+}
 
 // Parallel cyclic reduction of the 32 rows held by the calling warp (one per lane; a lane
 // without a row holds the identity row). Row i: a x_{i-1} + b x_i + c x_{i+1} = d, with the
 // couplings to rows outside the warp already moved to the columns gc (left) and hc (right).
-// On return every row is decoupled: b x_i = d - gc X_left - hc X_right.
-template <typename T>
-__device__ __forceinline__ void warp_pcr(T& a, T& b, T& c, T& d, T& gc, T& hc)
+// On return every row is decoupled: x_i = d - gc X_left - hc X_right.
+__device__ __forceinline__ void warp_pcr(float a, float b, float c, float& d, float& gc, float& hc)
 {
     const int lane = threadIdx.x & 31;
-    T rb = recip(b);
+    float rb = recip(b);
 #pragma unroll
     for (int s = 1; s < 32; s <<= 1) {
-        const T am = __shfl_up_sync(0xFFFFFFFFu, a, s), cm = __shfl_up_sync(0xFFFFFFFFu, c, s);
-        const T dm = __shfl_up_sync(0xFFFFFFFFu, d, s), gm = __shfl_up_sync(0xFFFFFFFFu, gc, s);
-        const T hm = __shfl_up_sync(0xFFFFFFFFu, hc, s), rm = __shfl_up_sync(0xFFFFFFFFu, rb, s);
-        const T ap = __shfl_down_sync(0xFFFFFFFFu, a, s), cp = __shfl_down_sync(0xFFFFFFFFu, c, s);
-        const T dp = __shfl_down_sync(0xFFFFFFFFu, d, s), gp = __shfl_down_sync(0xFFFFFFFFu, gc, s);
-        const T hp = __shfl_down_sync(0xFFFFFFFFu, hc, s), rp = __shfl_down_sync(0xFFFFFFFFu, rb, s);
-        const T al = (lane >= s) ? a * rm : T(0);
-        const T ga = (lane + s < 32) ? c * rp : T(0);
+        const float am = __shfl_up_sync(0xFFFFFFFFu, a, s), cm = __shfl_up_sync(0xFFFFFFFFu, c, s);
+        const float dm = __shfl_up_sync(0xFFFFFFFFu, d, s), gm = __shfl_up_sync(0xFFFFFFFFu, gc, s);
+        const float hm = __shfl_up_sync(0xFFFFFFFFu, hc, s), rm = __shfl_up_sync(0xFFFFFFFFu, rb, s);
+        const float ap = __shfl_down_sync(0xFFFFFFFFu, a, s), cp = __shfl_down_sync(0xFFFFFFFFu, c, s);
+        const float dp = __shfl_down_sync(0xFFFFFFFFu, d, s), gp = __shfl_down_sync(0xFFFFFFFFu, gc, s);
+        const float hp = __shfl_down_sync(0xFFFFFFFFu, hc, s), rp = __shfl_down_sync(0xFFFFFFFFu, rb, s);
+        const float al = (lane >= s) ? a * rm : 0.0f;
+        const float ga = (lane + s < 32) ? c * rp : 0.0f;
         a = -al * am;
         c = -ga * cp;
         b = b - al * cm - ga * ap;
@@ -176,326 +220,266 @@ __device__ __forceinline__ void warp_pcr(T& a, T& b, T& c, T& d, T& gc, T& hc)
     hc *= rb;
 }
 
-// Values every block pushes into every block's shared memory before the first cluster barrier
-// of a Newton iteration (slot k holds block k's): its first interior row and its last interior
-// row in terms of the block separators around it (x = y - g s_{k-1} - h s_k), its separator
-// row (a, b, c, d of row s_k), and its residual bound (max |F|, min g').
-constexpr int kPush = 12;
+// Parameters of one field solve (one realisation).
+struct FieldDesc {
+    const long long* rho;
+    double* phi;
+    double* E;
+    float* Ef;
+    int* diag;
+    uint32_t* status;
+    double inv_dx2, half_inv_dx;    // 1 / dx^2, 1 / (2 dx)
+    float tol;
+    int shift;                      // density = rho 2^-shift
+    int ncell, mode, maxit, walls;  // walls: 1 for a bounded grid
+    // Newton start: phi_prev (may be null) keeps the solution before the current one; with
+    // extrap the start is the linear extrapolation 2 phi - phi_prev (solves one fine step apart)
+    double* phi_prev;
+    int extrap, pad;
+};
 
-// A block's first interior row from its pushed values, given the separators around the block
-// (the owner and its left neighbour evaluate this same function, so the neighbour's halo stays
-// bit-identical to the owner's node).
-template <typename T>
-__device__ __forceinline__ T edge_row(const T* r, T s_left, T s_right)
+// A unit's (a warp's, a block's) rows as its neighbours see them: its first row and its last
+// interior row in terms of the separators around it (x = y - g s_left - h s_right) and the row of
+// its own separator (a, b, c, d), with its largest |F| and its smallest g'.
+struct UnitRow {
+    float4 first;  // y, g, h, max |F|
+    float4 last;   // y, g, h, min g'
+    float4 sep;    // a, b, c, d
+};
+
+// Double-buffered by iteration parity: a warp or block may write the next iteration's rows
+// while another still reads these (it cannot write the one after that before every warp has
+// passed the barrier in between).
+struct NewtonShared {
+    UnitRow warp[2][kNewtonMaxWarps];                // this block's warps
+    UnitRow block[2][kClusterMax];                   // rows pushed by every block of the cluster
+    float2 upd[2][kClusterMax * kNewtonMaxWarps];    // every warp's largest |update| and the bound of
+                                                     // the residual it leaves
+};
+
+// A unit's first row given the separators around it (the owner and its left neighbour evaluate
+// this same function, so the neighbour's halo stays bit-identical to the owner's node).
+__device__ __forceinline__ float edge_row(const float4& f, float s_left, float s_right)
 {
-    return r[0] - r[1] * s_left - r[2] * s_right;
+    return f.x - f.y * s_left - f.z * s_right;
 }
 
-// Solver body for the realisation of this cluster: B = ncell / G nodes per block, one per
-// thread; threads at or beyond B (a batched launch sized for a larger grid) only take
-// part in the barriers. T is the precision of the linear solve.
-template <typename T>
+// Solver body for the realisation of this cluster: B = ncell / G nodes per block, one per thread
+// (on grids below 32 nodes the block's one warp has lanes without a node).
 __device__ __forceinline__ void newton_body(const FieldDesc& d, cg::cluster_group& cluster)
 {
-    extern __shared__ double sh[];
-    const int G = (int)cluster.num_blocks();
-    const int g = (int)cluster.block_rank();
-    const int ncell = d.ncell;
-    const int B = ncell / G;
+    __shared__ NewtonShared sh;
+    const int G = (int)cluster.num_blocks(), g = (int)cluster.block_rank();
+    const int ncell = d.ncell, mask = ncell - 1, B = ncell / G;
     const int i = threadIdx.x, lane = i & 31, w = i >> 5;
-    const int W = (B + 31) >> 5;  // warps holding rows
+    const int W = (B + 31) >> 5;  // warps
     const bool act = i < B;
-    const long long* rho = d.rho;
-    double* phi = d.phi;
-    const double dx = d.dx, nscale = d.nscale, tol = d.tol;
-    const int mode = d.mode, maxit = d.maxit;
-    double* ph = sh;                              // [B + 2] phi with the halo
-    T* recv = reinterpret_cast<T*>(ph + B + 2);   // [G][kPush] rows pushed by every block
-    T* recvm = recv + kPush * G;                  // [G] every block's max |update|
-    T* wedge = recvm + G;                         // [W][8]: warp w's first interior row (y, g, h),
-                                                  // last interior row (y, g, h), max|F|, min g'
-    T* wsep = wedge + 8 * W;                      // [W][4]: warp w's separator row (a, b, c, d)
-    T* lev2 = wsep + 4 * W;                       // [W][3]: S_w = Y - Gc s_{k-1} - Hc s_k
-    T* svals = lev2 + 3 * W;                      // [G]: every block separator s_k
-    T* wmax = svals + G;                          // [32]: per-warp max |update|
-    T* flag = wmax + 32;                          // [1]: converged by the residual bound
-
-    const int mask = ncell - 1;
     const int j = g * B + (act ? i : 0);
-    const bool walls = d.walls != 0;
+    const bool walls = d.walls != 0, boltz = d.mode == PE_POISSON_BOLTZMANN;
     const bool wl = walls && j == 0, wr = walls && j == ncell - 1;  // this thread's node is a wall
-    const double inv_dx2 = 1.0 / (dx * dx);
-    const T o = (T)(-inv_dx2);
-    const bool boltz = (mode == PE_POISSON_BOLTZMANN);
-    const double nj = act ? (double)__ldg(rho + j) * nscale * ((wl || wr) ? 2.0 : 1.0) : 0.0;
-    // Newton start: phi, or with extrap the extrapolation 2 phi - phi_prev of the last two
-    // solutions. Nothing is written to phi or phi_prev before the first cluster barrier, so the
-    // halo nodes below (the neighbouring blocks' boundary nodes) are read unchanged and
-    // extrapolated here with the owners' arithmetic.
-    const bool hist = d.phi_prev != nullptr, ex = hist && d.extrap;
-    const double p_old = act ? phi[j] : 0.0;
-    double pj = (act && ex) ? 2.0 * p_old - d.phi_prev[j] : p_old;
-    double gj = boltz ? exp(pj) : 1.0 + pj;
-    // Halo ph[0], ph[B + 1]: read once and then advanced here with the same damped updates their
-    // owners apply (values of the reduced systems, known to every block), so they stay
-    // bit-identical to the owners' values. Only threads 0 and B - 1 read and write them.
-    if (act && (i == 0 || i == B - 1)) {
-        const int h = (i == 0) ? ((g * B - 1) & mask) : ((g * B + B) & mask);
-        const double v = phi[h];
-        ph[i == 0 ? 0 : B + 1] = ex ? 2.0 * v - d.phi_prev[h] : v;
-    }
-    bool hist_written = false;
+    const double inv_dx2 = d.inv_dx2, diag0 = 2.0 * inv_dx2;
+    const float inv = f32_of(inv_dx2), o = -inv;
     const int sep = (w == W - 1) ? ((B - 1) & 31) : 31;  // this warp's separator lane
+    // the couplings of this row: mirror ghosts double a wall row's one coupling
+    const float lo = wl ? 0.0f : (wr ? 2.0f * o : o), up = wr ? 0.0f : (wl ? 2.0f * o : o);
+    if (G > 1) asm volatile("barrier.cluster.arrive.relaxed.aligned;" ::: "memory");
+
+    // Newton start: phi, or with extrap the extrapolation 2 phi - phi_prev of the last two
+    // solutions. phi and phi_prev are written after the iteration only, so the halo nodes below (the
+    // neighbouring warps' edge nodes, on the first and the separator lane) are read unchanged
+    // and extrapolated here with the owners' arithmetic; later they are advanced here with the
+    // updates their owners apply (values of the reduced systems, known to every warp), so they
+    // stay bit-identical to the owners' values.
+    const bool hist = d.phi_prev != nullptr, ex = hist && d.extrap;
+    auto start = [&](int node) { return ex ? 2.0 * d.phi[node] - d.phi_prev[node] : d.phi[node]; };
+    const long long q = __ldg(d.rho + j);
+    double p = start(j);
+    double halo = start(lane == 0 ? ((j - 1) & mask) : ((j + 1) & mask));
+    // density; a wall node's is twice its deposit
+    const double nj = fixed_to_double(q, d.shift - ((wl || wr) ? 1 : 0));
+    double gj = boltz ? exp(p) : 1.0 + p;
+    if (G > 1) asm volatile("barrier.cluster.wait.acquire.aligned;" ::: "memory");  // every block has started
 
     int it = 0;
     bool converged = false;
-    for (it = 0; it < maxit; ++it) {
-        // ---- FP64 residual with the halo from the neighbouring blocks (mirror ghosts at walls)
-        if (act) ph[i + 1] = pj;
-        __syncthreads();
-        T a = T(0), b = T(1), c = T(0), rhs = T(0), gc = T(0), hc = T(0);
-        float fabs_r = 0.f, gmin = 3.0e38f;
-        T sa = T(0), sb = T(1), sc = T(0), sd = T(0);  // the separator's row (lane sep)
-        if (act) {
-            const double pl = wl ? ph[i + 2] : ph[i], pr = wr ? ph[i] : ph[i + 2];
-            const double lap = (pl - 2.0 * pj + pr) * inv_dx2;
-            const double r = lap - gj + nj;  // -F_j
-            fabs_r = (float)fabs(r);
-            gmin = boltz ? (float)gj : 1.0f;
-            const T lo = wr ? T(2) * o : o, up = wl ? T(2) * o : o;  // mirror ghosts double a wall row's coupling
-            const T bd = (T)(2.0 * inv_dx2 + (boltz ? gj : 1.0));
-            if (lane == sep) {  // separator: an identity row in the warp's reduction
-                sa = wl ? T(0) : lo;
-                sb = bd;
-                sc = wr ? T(0) : up;
-                sd = (T)r;
-            } else {
-                b = bd;
-                rhs = (T)r;
-                // couplings to the separators around the interior become extra right-hand sides
-                if (lane == 0) gc = wl ? T(0) : lo;
-                else a = lo;
-                if (lane == sep - 1) hc = wr ? T(0) : up;
-                else c = up;
-            }
-        }
+    for (it = 0; it < d.maxit; ++it) {
+        const int par = it & 1;
+        // ---- FP64 residual (mirror ghosts at walls)
+        double pl = __shfl_up_sync(0xFFFFFFFFu, p, 1), pr = __shfl_down_sync(0xFFFFFFFFu, p, 1);
+        if (lane == 0) pl = halo;
+        if (lane == sep) pr = halo;
+        if (wl) pl = pr;
+        if (wr) pr = pl;
+        const float r = f32_of(fma(fma(-2.0, p, pl) + pr, inv_dx2, -gj) + nj);  // -F_j
+        const float bd = f32_of(diag0 + (boltz ? gj : 1.0));
+        const float gf = boltz ? f32_of(gj) : 1.0f;
+        const float fw = warp_max_bits(act ? __float_as_uint(fabsf(r)) : 0u);
+        const float gw = warp_min_bits(act ? gf : 3.0e38f);
         // ---- warp interiors: x = rhs - gc S_left - hc S_right
+        float a = 0.0f, b = 1.0f, c = 0.0f, rhs = 0.0f, gc = 0.0f, hc = 0.0f;
+        if (act && lane != sep) {  // the separator holds an identity row in the warp's reduction
+            b = bd;
+            rhs = r;
+            // couplings to the separators around the interior become extra right-hand sides
+            if (lane == 0) gc = lo;
+            else a = lo;
+            if (lane == sep - 1) hc = up;
+            else c = up;
+        }
         warp_pcr(a, b, c, rhs, gc, hc);
-        float fr = fabs_r, gm = gmin;
-#pragma unroll
-        for (int off = 16; off > 0; off >>= 1) {
-            fr = fmaxf(fr, __shfl_xor_sync(0xFFFFFFFFu, fr, off));
-            gm = fminf(gm, __shfl_xor_sync(0xFFFFFFFFu, gm, off));
-        }
-        if (w < W) {
-            T* e = wedge + 8 * w;
-            if (lane == 0) {
-                e[0] = rhs;
-                e[1] = gc;
-                e[2] = hc;
-                e[6] = (T)fr;
-                e[7] = (T)gm;
-            }
-            if (lane == sep - 1) {
-                e[3] = rhs;
-                e[4] = gc;
-                e[5] = hc;
-            }
-            if (lane == sep) {
-                wsep[4 * w] = sa;
-                wsep[4 * w + 1] = sb;
-                wsep[4 * w + 2] = sc;
-                wsep[4 * w + 3] = sd;
-            }
-        }
+        UnitRow* mine = &sh.warp[par][w];
+        if (lane == 0) mine->first = make_float4(rhs, gc, hc, fw);
+        if (lane == sep - 1) mine->last = make_float4(rhs, gc, hc, gw);
+        if (lane == sep) mine->sep = make_float4(lo, bd, up, r);
         __syncthreads();
-        // ---- warp 0: the block's warp separators S_0 .. S_{W-2} in terms of the block
-        // separators s_{k-1} (left) and s_k (right), then the block's rows for the cluster system
-        if (w == 0) {
-            // row q = lane < W - 1: separator of warp q, between warp q's last interior row and
-            // warp q+1's first interior row
-            T la = T(0), lb = T(1), lc = T(0), r0 = T(0), r1 = T(0), r2 = T(0);
-            if (lane < W - 1) {
-                const T* ep = wedge + 8 * lane;        // warp q
-                const T* en = wedge + 8 * (lane + 1);  // warp q + 1
-                const T* sr = wsep + 4 * lane;
-                la = -sr[0] * ep[4];
-                lb = sr[1] - sr[0] * ep[5] - sr[2] * en[1];
-                lc = -sr[2] * en[2];
-                r0 = sr[3] - sr[0] * ep[3] - sr[2] * en[0];
-                if (lane == 0) {  // S_{-1} = s_{k-1}
-                    r1 = la;
-                    la = T(0);
+        // ---- the block's warp separators S_0 .. S_{W-2} in terms of the block separators s_{k-1}
+        // (left) and s_k (right): row q = lane < W - 1 lies between warp q's last interior row and
+        // warp q + 1's first row
+        const UnitRow* wrow = sh.warp[par];
+        float la = 0.0f, lb = 1.0f, lc = 0.0f, r0 = 0.0f, r1 = 0.0f, r2 = 0.0f;
+        uint32_t fl = 0u;
+        float gl = 3.0e38f;
+        if (lane < W) {
+            fl = __float_as_uint(wrow[lane].first.w);
+            gl = wrow[lane].last.w;
+        }
+        if (lane < W - 1) {
+            const float4 ep = wrow[lane].last, sr = wrow[lane].sep, en = wrow[lane + 1].first;
+            la = -sr.x * ep.y;
+            lb = sr.y - sr.x * ep.z - sr.z * en.y;
+            lc = -sr.z * en.z;
+            r0 = sr.w - sr.x * ep.x - sr.z * en.x;
+            if (lane == 0) {  // S_{-1} = s_{k-1}
+                r1 = la;
+                la = 0.0f;
+            }
+            if (lane == W - 2) {  // S_{W-1} = s_k
+                r2 = lc;
+                lc = 0.0f;
+            }
+        }
+        float Y, Gc, Hc;
+        warp_chain_pcr(la, lb, lc, r0, r1, r2, W, Y, Gc, Hc);
+        // the block's first row (warp 0) and last interior row (warp W - 1) in terms of s_{k-1}, s_k
+        const float4 e0 = wrow[0].first, eL = wrow[W - 1].last;
+        UnitRow own;
+        own.sep = wrow[W - 1].sep;
+        const float fbk = warp_max_bits(fl), gbk = warp_min_bits(gl);  // residual bound of the block
+        if (W > 1) {  // first row: x = y - g s_{k-1} - h S_0; last row: x = y - g S_{W-2} - h s_k
+            const float Y0 = __shfl_sync(0xFFFFFFFFu, Y, 0), G0 = __shfl_sync(0xFFFFFFFFu, Gc, 0);
+            const float H0 = __shfl_sync(0xFFFFFFFFu, Hc, 0), YL = __shfl_sync(0xFFFFFFFFu, Y, W - 2);
+            const float GL = __shfl_sync(0xFFFFFFFFu, Gc, W - 2), HL = __shfl_sync(0xFFFFFFFFu, Hc, W - 2);
+            own.first = make_float4(e0.x - e0.z * Y0, e0.y - e0.z * G0, -e0.z * H0, fbk);
+            own.last = make_float4(eL.x - eL.y * YL, -eL.y * GL, eL.z - eL.y * HL, gbk);
+        } else {
+            own.first = make_float4(e0.x, e0.y, e0.z, fbk);
+            own.last = make_float4(eL.x, eL.y, eL.z, gbk);
+        }
+        // ---- the cyclic system of the block separators s_0 .. s_{G-1}, and the residual bound
+        UnitRow rk = own;
+        float4 nf = own.first;  // the next block's first row
+        if (G > 1) {
+            for (int t = w; t < G; t += W)  // the block's warps share the pushes (they hold the same rows)
+                if (lane < 3) {
+                    float4* dst = reinterpret_cast<float4*>(cluster.map_shared_rank(&sh.block[par][g], t));
+                    dst[lane] = lane == 0 ? own.first : (lane == 1 ? own.last : own.sep);
                 }
-                if (lane == W - 2) {  // S_{W-1} = s_k
-                    r2 = lc;
-                    lc = T(0);
-                }
-            }
-            T Y = T(0), Gc = T(0), Hc = T(0);
-            warp_scalar_pcr(la, lb, lc, r0, r1, r2, W, false, Y, Gc, Hc);
-            if (lane < W - 1) {
-                lev2[3 * lane] = Y;
-                lev2[3 * lane + 1] = Gc;
-                lev2[3 * lane + 2] = Hc;
-            }
-            // the block's first interior row (warp 0, lane 0) and last interior row (warp W-1,
-            // lane sep-1), each in terms of s_{k-1} and s_k
-            const T* e0 = wedge;
-            const T* eL = wedge + 8 * (W - 1);
-            const T Y0 = __shfl_sync(0xFFFFFFFFu, Y, 0), G0 = __shfl_sync(0xFFFFFFFFu, Gc, 0),
-                    H0 = __shfl_sync(0xFFFFFFFFu, Hc, 0);
-            const int ql = W >= 2 ? W - 2 : 0;
-            const T YL = __shfl_sync(0xFFFFFFFFu, Y, ql), GL = __shfl_sync(0xFFFFFFFFu, Gc, ql),
-                    HL = __shfl_sync(0xFFFFFFFFu, Hc, ql);
-            T row[kPush];
-            if (W > 1) {  // first row: x = y - g s_{k-1} - h S_0; last row: x = y - g S_{W-2} - h s_k
-                row[0] = e0[0] - e0[2] * Y0;
-                row[1] = e0[1] - e0[2] * G0;
-                row[2] = -e0[2] * H0;
-                row[3] = eL[3] - eL[4] * YL;
-                row[4] = -eL[4] * GL;
-                row[5] = eL[5] - eL[4] * HL;
-            } else {
-                row[0] = e0[0];
-                row[1] = e0[1];
-                row[2] = e0[2];
-                row[3] = eL[3];
-                row[4] = eL[4];
-                row[5] = eL[5];
-            }
-            const T* sL = wsep + 4 * (W - 1);  // the block separator s_k
-            row[6] = sL[0];
-            row[7] = sL[1];
-            row[8] = sL[2];
-            row[9] = sL[3];
-            // residual bound of the block
-            T fb = lane < W ? wedge[8 * lane + 6] : T(0), gb = lane < W ? wedge[8 * lane + 7] : T(3.0e38f);
-#pragma unroll
-            for (int off = 16; off > 0; off >>= 1) {
-                const T f2 = __shfl_xor_sync(0xFFFFFFFFu, fb, off), g2 = __shfl_xor_sync(0xFFFFFFFFu, gb, off);
-                fb = f2 > fb ? f2 : fb;
-                gb = g2 < gb ? g2 : gb;
-            }
-            row[10] = fb;
-            row[11] = gb;
-            if (lane < G) {  // lane r pushes the block's rows into block r's shared memory
-                T* dst = cluster.map_shared_rank(recv, lane) + kPush * g;
-#pragma unroll
-                for (int c2 = 0; c2 < kPush; ++c2) dst[c2] = row[c2];
-            }
+            cluster.sync();  // every block's pushed rows are visible in every block
+            rk = sh.block[par][lane & (G - 1)];
+            nf = sh.block[par][(lane + 1) & (G - 1)].first;
         }
-        cluster.sync();  // #1: every block's pushed rows are visible in every block
-        if (hist && !hist_written) {  // every block has read its halo: the history may move on
-            if (act) d.phi_prev[j] = p_old;
-            hist_written = true;
-        }
-        // ---- warp 0: the cyclic system of the block separators s_0 .. s_{G-1}, and the residual bound
-        if (w == 0) {
-            T la = T(0), lb = T(1), lc = T(0), r0 = T(0);
-            T fb = T(0), gb = T(3.0e38f);
-            if (lane < G) {
-                // row of s_k: a x_last(k) + b s_k + c x_first(k+1) = d
-                const T* rk = recv + kPush * lane;
-                const T* rn = recv + kPush * ((lane + 1) % G);
-                la = -rk[6] * rk[4];
-                lb = rk[7] - rk[6] * rk[5] - rk[8] * rn[1];
-                lc = -rk[8] * rn[2];
-                r0 = rk[9] - rk[6] * rk[3] - rk[8] * rn[0];
-                fb = rk[10];
-                gb = rk[11];
-            }
-#pragma unroll
-            for (int off = 16; off > 0; off >>= 1) {
-                const T f2 = __shfl_xor_sync(0xFFFFFFFFu, fb, off), g2 = __shfl_xor_sync(0xFFFFFFFFu, gb, off);
-                fb = f2 > fb ? f2 : fb;
-                gb = g2 < gb ? g2 : gb;
-            }
-            T sk, u1, u2;
-            warp_scalar_pcr(la, lb, lc, r0, T(0), T(0), G, true, sk, u1, u2);
-            if (lane < G) svals[lane] = sk;
-            // the residual bounds the next update below tol: phi is converged (the same decision
-            // in every block: the same pushed values reduced in the same order)
-            if (lane == 0) flag[0] = (it > 0 && (double)fb < tol * (double)gb) ? T(1) : T(0);
-        }
-        __syncthreads();
-        if (flag[0] != T(0)) {
+        const float fb = warp_max_bits(__float_as_uint(rk.first.w)), gb = warp_min_bits(rk.last.w);
+        // the residual bounds the next update below tol: phi is converged (the same decision in
+        // every warp: the same pushed values)
+        if (it > 0 && fb < d.tol * gb) {
             converged = true;
             break;
         }
-        const T Sl = svals[(g - 1 + G) % G], Sr = svals[g];  // s_{k-1}, s_k
-        // ---- back substitution: the warp's separators, then its row
-        T dlt = T(0);
+        // row of s_k: a x_last(k) + b s_k + c x_first(k+1) = d
+        const float sk = warp_cyclic(-rk.sep.x * rk.last.y, rk.sep.y - rk.sep.x * rk.last.z - rk.sep.z * nf.y,
+                                     -rk.sep.z * nf.z, rk.sep.w - rk.sep.x * rk.last.x - rk.sep.z * nf.x, G);
+        const float Sl = __shfl_sync(0xFFFFFFFFu, sk, (g - 1) & (G - 1)), Sr = __shfl_sync(0xFFFFFFFFu, sk, g);
+        const float Sn = __shfl_sync(0xFFFFFFFFu, sk, (g + 1) & (G - 1));  // s_{k-1}, s_k, s_{k+1}
+        // ---- back substitution: the warp's separators, then its rows
+        const float Sq = lane < W - 1 ? Y - Gc * Sl - Hc * Sr : Sr;  // S_lane
+        const float S0 = __shfl_sync(0xFFFFFFFFu, Sq, (w - 1) & 31), Sw_r = __shfl_sync(0xFFFFFFFFu, Sq, w);
+        const float S2 = __shfl_sync(0xFFFFFFFFu, Sq, w + 1 < W ? w + 1 : w);
+        const float Sw_l = w == 0 ? Sl : S0;
+        float x = 0.0f;
         if (act) {
-            const T Sw_l = (w == 0) ? Sl : lev2[3 * (w - 1)] - lev2[3 * (w - 1) + 1] * Sl - lev2[3 * (w - 1) + 2] * Sr;
-            const T Sw_r = (w == W - 1) ? Sr : lev2[3 * w] - lev2[3 * w + 1] * Sl - lev2[3 * w + 2] * Sr;
-            if (lane == sep) dlt = Sw_r;
-            else if (i == 0)  // the block's first row: the form the left neighbour uses for its halo
-                dlt = edge_row(recv + kPush * g, Sl, Sr);
-            else
-                dlt = rhs - gc * Sw_l - hc * Sw_r;
+            if (lane == sep) x = Sw_r;
+            else if (i == 0) x = edge_row(own.first, Sl, Sr);  // the form the left neighbour uses for its halo
+            else x = rhs - gc * Sw_l - hc * Sw_r;
         }
-        // ---- global max |update| (damping and convergence): pushed to every block
-        T mloc = dlt < T(0) ? -dlt : dlt;
-#pragma unroll
-        for (int off = 16; off > 0; off >>= 1) {
-            const T oth = __shfl_xor_sync(0xFFFFFFFFu, mloc, off);
-            mloc = oth > mloc ? oth : mloc;
+        // the updates of the halo nodes: the left neighbour's separator, the right neighbour's first row
+        float4 right = wrow[w + 1 < W ? w + 1 : w].first;
+        if (w + 1 == W) right = G > 1 ? sh.block[par][(g + 1) & (G - 1)].first : own.first;
+        const float x_next = w + 1 < W ? edge_row(right, Sw_r, S2) : edge_row(right, Sr, Sn);
+        const float mw = warp_max_bits(__float_as_uint(fabsf(x)));  // the warp's largest |update|
+        // ---- exchange of the largest update (damping, convergence) and of the bound of the
+        // residual it leaves; the FP64 update runs while the exchange is under way
+        float xl = __shfl_up_sync(0xFFFFFFFFu, x, 1), xr = __shfl_down_sync(0xFFFFFFFFu, x, 1);
+        if (lane == 0) xl = Sw_l;
+        if (lane == sep) xr = x_next;
+        if (wl) xl = xr;
+        if (wr) xr = xl;
+        const float Jx = inv * ((x - xl) + (x - xr)) + gf * x;
+        const float ax = fabsf(x), big = fmaxf(ax, fmaxf(fabsf(xl), fabsf(xr)));
+        // rounding of r, Jx, g and their difference: a few 2^-24 of the terms
+        const float e = fabsf(r - Jx) + 2e-6f * ((4.0f * inv + gf) * big + fabsf(r)) +
+                        (boltz ? gf * ax * ax * (0.5f + ax) : 0.0f);
+        const float2 v = make_float2(mw, warp_max_bits(act ? __float_as_uint(e) : 0u));
+        if (G > 1) {
+            if (lane < G) *cluster.map_shared_rank(&sh.upd[par][g * W + w], lane) = v;
+            asm volatile("barrier.cluster.arrive.release.aligned;" ::: "memory");
+        } else if (lane == 0) {
+            sh.upd[par][w] = v;
         }
-        if (lane == 0) wmax[w] = mloc;
-        __syncthreads();
-        if (w == 0) {
-            T v = (lane < ((int)(blockDim.x + 31) >> 5)) ? wmax[lane] : T(0);
-#pragma unroll
-            for (int off = 16; off > 0; off >>= 1) {
-                const T oth = __shfl_xor_sync(0xFFFFFFFFu, v, off);
-                v = oth > v ? oth : v;
+        // the undamped update, and exp(phi) carried with the small-update polynomial
+        const double x1 = f64_of(x), xh = f64_of(lane == 0 ? Sw_l : x_next);
+        double pn = p + x1, hn = halo + xh, gn = boltz ? gj * exp_tiny(x1) : 1.0 + pn;
+        if (G > 1) asm volatile("barrier.cluster.wait.acquire.aligned;" ::: "memory");
+        else __syncthreads();
+        uint32_t mb = 0u, rb = 0u;
+        for (int k = lane; k < G * W; k += 32) {
+            const float2 t = sh.upd[par][k];
+            mb = max(mb, __float_as_uint(t.x));
+            rb = max(rb, __float_as_uint(t.y));
+        }
+        const float m = warp_max_bits(mb), rm = warp_max_bits(rb);
+        // min g' after the update is at least (1 - m) gb
+        const bool done = m < d.tol || (m <= 0.0078125f && rm < 0.99f * d.tol * gb);
+        if (!done && !(m <= 0.0009765625f)) {  // 2^-10: the polynomial's degree follows the largest update
+            double xs = x1;
+            if (m > 2.0f) {  // damped
+                const double scale = 2.0 / (double)m;
+                xs = scale * x1;
+                pn = p + xs;
+                hn = halo + scale * xh;
             }
-            v = __shfl_sync(0xFFFFFFFFu, v, 0);
-            if (lane < G) cluster.map_shared_rank(recvm, lane)[g] = v;
+            if (boltz) gn = (fabs(xs) <= 0.03125) ? gj * exp_small(xs) : exp(pn);
+            else gn = 1.0 + pn;
         }
-        // #2: every block's maximum is visible; the pushed rows are no longer read. The next
-        // iteration pushes again only after its barrier #1, which every block reaches after
-        // reading these.
-        cluster.sync();
-        T mm = T(0);
-        for (int k = 0; k < G; ++k) mm = recvm[k] > mm ? recvm[k] : mm;
-        const double m = (double)mm;
-        const double scale = (m > 2.0) ? 2.0 / m : 1.0;
-        const double x = act ? scale * (double)dlt : 0.0;
-        pj += x;
-        if (act) phi[j] = pj;
-        if (act && i == 0) ph[0] += scale * (double)Sl;  // the previous block's last node is s_{k-1}
-        if (act && i == B - 1) {  // the next block's first row, as its owner computes it
-            ph[B + 1] += scale * (double)edge_row(recv + kPush * ((g + 1) % G), Sr, svals[(g + 1) % G]);
-        }
-        if (boltz) {  // |x| <= scale m for every node: the degree follows the cluster-wide bound
-            if (scale * m <= 0.0009765625)
-                gj *= exp_tiny(x);
-            else
-                gj = (fabs(x) <= 0.03125) ? gj * exp_small(x) : exp(pj);
-        } else {
-            gj = 1.0 + pj;
-        }
-        if (m < tol) {
+        p = pn;
+        halo = hn;
+        gj = gn;
+        if (done) {
             converged = true;
             ++it;
             break;
         }
     }
-    if (hist && !hist_written) {  // no iteration ran (maxit 0): the start is the solution
-        cluster.sync();           // every block has read its halo
-        if (act) {
-            d.phi_prev[j] = p_old;
-            phi[j] = pj;
-        }
-    }
-    if (act) ph[i + 1] = pj;
-    __syncthreads();
+    if (d.maxit < 1 && G > 1) cluster.sync();  // no exchange ran: every block has read its halo
+    if (d.maxit < 1) __syncthreads();
+    double pl = __shfl_up_sync(0xFFFFFFFFu, p, 1), pr = __shfl_down_sync(0xFFFFFFFFu, p, 1);
+    if (lane == 0) pl = halo;
+    if (lane == sep) pr = halo;
     if (act) {
-        const double e = (wl || wr) ? 0.0 : -(ph[i + 2] - ph[i]) * (0.5 / dx);
+        const double e = (wl || wr) ? 0.0 : (pl - pr) * d.half_inv_dx;
+        if (hist) d.phi_prev[j] = d.phi[j];
+        d.phi[j] = p;
         d.E[j] = e;
-        d.Ef[j] = (float)e;
+        d.Ef[j] = f32_of(e);
     }
     if (g == 0 && i == 0) {
         if (d.diag) {
@@ -506,35 +490,32 @@ __device__ __forceinline__ void newton_body(const FieldDesc& d, cg::cluster_grou
         }
         if (!converged) raise_flag(d.status, PE_FLAG_NOCONV);
     }
-    cluster.sync();  // no block leaves while another may still push into it
 }
 
-template <typename T>
 __global__ void __launch_bounds__(kNewtonMaxThreads, 1) k_newton_cluster(FieldDesc d)
 {
     cg::cluster_group cluster = cg::this_cluster();
-    newton_body<T>(d, cluster);
+    newton_body(d, cluster);
 }
 
 // One cluster per realisation: cluster c solves descs[c]; extrap applies to every realisation.
-template <typename T>
 __global__ void __launch_bounds__(kNewtonMaxThreads, 1) k_newton_batch(const FieldDesc* descs, int extrap)
 {
     cg::cluster_group cluster = cg::this_cluster();
     FieldDesc d = descs[blockIdx.x / cluster.num_blocks()];
     d.extrap = extrap;
-    newton_body<T>(d, cluster);
+    newton_body(d, cluster);
 }
 
-static int cluster_size_for(int ncell)
+// Largest cluster (<= 16, a power of two) the device accepts for these kernels.
+static int cluster_limit()
 {
-    // largest cluster (<= 16) the device accepts for this kernel; 0 if none
     static int cached[64] = {0};
     int dev = 0;
-    if (cudaGetDevice(&dev) != cudaSuccess || dev < 0 || dev >= 64) return 0;
+    if (cudaGetDevice(&dev) != cudaSuccess || dev < 0 || dev >= 64) return 1;
     if (!cached[dev]) {
-        cudaFuncSetAttribute((const void*)k_newton_cluster<float>, cudaFuncAttributeNonPortableClusterSizeAllowed, 1);
-        cudaFuncSetAttribute((const void*)k_newton_cluster<double>, cudaFuncAttributeNonPortableClusterSizeAllowed, 1);
+        cudaFuncSetAttribute((const void*)k_newton_cluster, cudaFuncAttributeNonPortableClusterSizeAllowed, 1);
+        cudaFuncSetAttribute((const void*)k_newton_batch, cudaFuncAttributeNonPortableClusterSizeAllowed, 1);
         cudaLaunchConfig_t cfg = {};
         cudaLaunchAttribute attr[1];
         attr[0].id = cudaLaunchAttributeClusterDimension;
@@ -542,70 +523,30 @@ static int cluster_size_for(int ncell)
         attr[0].val.clusterDim.y = 1;
         attr[0].val.clusterDim.z = 1;
         cfg.gridDim = dim3(kClusterMax);
-        cfg.blockDim = dim3(512);
-        cfg.dynamicSmemBytes = 16 * 1024;
+        cfg.blockDim = dim3(kNewtonMaxThreads);
         cfg.attrs = attr;
         cfg.numAttrs = 1;
         int size = 0;
-        if (cudaOccupancyMaxPotentialClusterSize(&size, (const void*)k_newton_cluster<float>, &cfg) != cudaSuccess)
-            size = 8;
+        if (cudaOccupancyMaxPotentialClusterSize(&size, (const void*)k_newton_cluster, &cfg) != cudaSuccess) size = 8;
         cudaGetLastError();
         int p = 1;
         while (p * 2 <= size && p * 2 <= kClusterMax) p *= 2;
         cached[dev] = p;
     }
-    int G = cached[dev];
-    while (G > 1 && ncell / G < 32) G >>= 1;  // at least 32 nodes per block
+    return cached[dev];
+}
+
+// Cluster size of a lone solve: as many blocks as the device clusters, at least 32 nodes each (the
+// FP64 work is spread over the SMs), one block for the grids below kClusterMinCells.
+static int cluster_size_for(int ncell)
+{
+    const int gmax = cluster_limit();
+    int G = gmax;
+    while (G > 1 && ncell / G < 32) G >>= 1;
     if (ncell < kClusterMinCells) G = 1;
     while (ncell / G > kNewtonMaxThreads) G <<= 1;  // at most kNewtonMaxThreads nodes (threads) per block
-    return G <= kClusterMax ? G : 0;
+    return G <= gmax ? G : 0;
 }
-
-size_t newton_smem_bytes(int B, int G, bool fp64)
-{
-    const size_t t = fp64 ? sizeof(double) : sizeof(float);
-    const size_t W = ((size_t)B + 31) / 32;
-    return sizeof(double) * ((size_t)B + 2) + t * ((kPush + 2) * (size_t)G + 15 * W + 33) + 16;
-}
-
-static cudaLaunchConfig_t cluster_config(cudaLaunchAttribute* attr, int G, int nclusters, int block, size_t smem,
-                                         cudaStream_t s)
-{
-    cudaLaunchConfig_t cfg = {};
-    attr[0].id = cudaLaunchAttributeClusterDimension;
-    attr[0].val.clusterDim.x = G;
-    attr[0].val.clusterDim.y = 1;
-    attr[0].val.clusterDim.z = 1;
-    cfg.gridDim = dim3(G * nclusters);
-    cfg.blockDim = dim3(block);
-    cfg.dynamicSmemBytes = smem;
-    cfg.stream = s;
-    cfg.attrs = attr;
-    cfg.numAttrs = 1;
-    return cfg;
-}
-
-static int launch_newton_cluster(int G, const long long* rho, int ncell, double dx, double nscale, int mode,
-                                 int walls, double tol, int maxit, double* phi, double* E, float* Ef, int* diag,
-                                 uint32_t* status, double* phi_prev, int extrap, cudaStream_t s)
-{
-    const int B = ncell / G;  // one node per thread
-    if (B > kNewtonMaxThreads || B < 2) return PE_EINVAL;
-    const bool fp64 = walls != 0 && kWallsJacobianFP64;
-    const size_t smem = newton_smem_bytes(B, G, fp64);
-    const void* k = fp64 ? (const void*)k_newton_cluster<double> : (const void*)k_newton_cluster<float>;
-    if (ensure_smem(k, smem) != PE_OK) return PE_ECUDA;
-    FieldDesc d{rho, phi, E, Ef, diag, status, dx, nscale, tol, ncell, mode, maxit, walls ? 1 : 0, phi_prev,
-                extrap ? 1 : 0, 0};
-    cudaLaunchAttribute attr[1];
-    cudaLaunchConfig_t cfg = cluster_config(attr, G, 1, B, smem, s);
-    const cudaError_t e = fp64 ? cudaLaunchKernelEx(&cfg, k_newton_cluster<double>, d)
-                               : cudaLaunchKernelEx(&cfg, k_newton_cluster<float>, d);
-    if (e != cudaSuccess) return PE_ECUDA;
-    return launch_status();
-}
-
-int newton_cluster_size(int ncell) { return cluster_size_for(ncell); }
 
 // Cluster size of a realisation's solve inside a batched launch: as few blocks as hold the grid
 // at kNewtonMaxThreads nodes each. A lone solve spreads its nodes over up to 16 SMs to cut the
@@ -613,37 +554,55 @@ int newton_cluster_size(int ncell) { return cluster_size_for(ncell); }
 // 16 for small grids left most of them waiting for SMs in later waves.
 int newton_batch_cluster_size(int ncell)
 {
-    const int gmax = cluster_size_for(kNewtonMaxThreads * kClusterMax);  // the device's largest
+    const int gmax = cluster_limit();
     int G = 1;
     while (ncell / G > kNewtonMaxThreads) G <<= 1;
     return G <= gmax ? G : 0;
 }
 
-// Batched field solves: descs[R] on the device, every grid with the same cluster size G;
-// fp64: the linear solves run in FP64 (bounded grids with kWallsJacobianFP64).
-int launch_newton_batch(const void* descs, int R, int G, int max_ncell, bool fp64, bool extrap, cudaStream_t s)
+static cudaLaunchConfig_t cluster_config(cudaLaunchAttribute* attr, int G, int nclusters, int B, cudaStream_t s)
 {
-    const int B = max_ncell / G;
-    if (B > kNewtonMaxThreads || B < 2 || R < 1) return PE_EINVAL;
-    const size_t smem = newton_smem_bytes(B, G, fp64);
-    const void* k = fp64 ? (const void*)k_newton_batch<double> : (const void*)k_newton_batch<float>;
-    if (ensure_smem(k, smem) != PE_OK) return PE_ECUDA;
-    static bool nonportable[2][64] = {{false}};
-    int dev = 0;
-    if (cudaGetDevice(&dev) != cudaSuccess || dev < 0 || dev >= 64) return PE_ECUDA;
-    if (G > 8 && !nonportable[fp64][dev]) {
-        if (cudaFuncSetAttribute(k, cudaFuncAttributeNonPortableClusterSizeAllowed, 1) != cudaSuccess)
-            return PE_ECUDA;
-        nonportable[fp64][dev] = true;
-    }
+    cudaLaunchConfig_t cfg = {};
+    attr[0].id = cudaLaunchAttributeClusterDimension;
+    attr[0].val.clusterDim.x = G;
+    attr[0].val.clusterDim.y = 1;
+    attr[0].val.clusterDim.z = 1;
+    cfg.gridDim = dim3(G * nclusters);
+    cfg.blockDim = dim3(B < 32 ? 32 : B);
+    cfg.stream = s;
+    cfg.attrs = attr;
+    cfg.numAttrs = 1;
+    return cfg;
+}
+
+static int launch_newton_cluster(int G, const FieldDesc& d, cudaStream_t s)
+{
+    const int B = d.ncell / G;  // one node per thread
+    if (B > kNewtonMaxThreads || B < 2) return PE_EINVAL;
     cudaLaunchAttribute attr[1];
-    cudaLaunchConfig_t cfg = cluster_config(attr, G, R, B, smem, s);
-    const FieldDesc* dd = static_cast<const FieldDesc*>(descs);
-    const int ex = extrap ? 1 : 0;
-    const cudaError_t e = fp64 ? cudaLaunchKernelEx(&cfg, k_newton_batch<double>, dd, ex)
-                               : cudaLaunchKernelEx(&cfg, k_newton_batch<float>, dd, ex);
-    if (e != cudaSuccess) return PE_ECUDA;
+    cudaLaunchConfig_t cfg = cluster_config(attr, G, 1, B, s);
+    if (cudaLaunchKernelEx(&cfg, k_newton_cluster, d) != cudaSuccess) return PE_ECUDA;
     return launch_status();
+}
+
+// Batched field solves: descs[R] on the device, every grid of ncell nodes.
+int launch_newton_batch(const void* descs, int R, int ncell, bool extrap, cudaStream_t s)
+{
+    const int G = newton_batch_cluster_size(ncell);
+    if (G < 1 || R < 1) return PE_EINVAL;
+    cudaLaunchAttribute attr[1];
+    cudaLaunchConfig_t cfg = cluster_config(attr, G, R, ncell / G, s);
+    if (cudaLaunchKernelEx(&cfg, k_newton_batch, static_cast<const FieldDesc*>(descs), extrap ? 1 : 0) != cudaSuccess)
+        return PE_ECUDA;
+    return launch_status();
+}
+
+static FieldDesc field_desc(const int64_t* rho, int ncell, double dx, int s_w, int mode, int walls, double tol, int maxit,
+                            double* phi, double* E, float* Ef, int32_t* diag, uint32_t* status, double* phi_prev,
+                            int extrap)
+{
+    return FieldDesc{reinterpret_cast<const long long*>(rho), phi, E, Ef, diag, status, 1.0 / (dx * dx), 0.5 / dx,
+                     (float)tol, s_w + 24, ncell, mode, maxit, walls ? 1 : 0, phi_prev, extrap ? 1 : 0, 0};
 }
 
 size_t field_desc_size() { return sizeof(FieldDesc); }
@@ -651,8 +610,7 @@ size_t field_desc_size() { return sizeof(FieldDesc); }
 void make_field_desc(void* out, const int64_t* rho, int ncell, double dx, int s_w, int mode, int walls, double tol,
                      int maxit, double* phi, double* E, float* Ef, int32_t* diag, uint32_t* status, double* phi_prev)
 {
-    FieldDesc d{reinterpret_cast<const long long*>(rho), phi, E, Ef, diag, status, dx, ldexp(1.0, -(s_w + 24)), tol,
-                ncell, mode, maxit, walls ? 1 : 0, phi_prev, 0, 0};
+    const FieldDesc d = field_desc(rho, ncell, dx, s_w, mode, walls, tol, maxit, phi, E, Ef, diag, status, phi_prev, 0);
     memcpy(out, &d, sizeof(d));
 }
 
@@ -670,13 +628,12 @@ int field_solve_history(const int64_t* rho_fx, int ncell, double dx, int s_w, in
     if (!is_pow2(ncell) || ncell < 8 || !rho_fx || !phi || !E || !Ef || !(dx > 0.0) || maxit < 0) return PE_EINVAL;
     if (mode != PE_POISSON_BOLTZMANN && mode != PE_POISSON_LINEARIZED) return PE_EINVAL;
     if (boundary != PE_BOUNDARY_PERIODIC && boundary != PE_BOUNDARY_ABSORBING) return PE_EINVAL;
-    const double nscale = ldexp(1.0, -(s_w + 24));
     if (ncell > kFullGridMax) return PE_EINVAL;
     const int G = cluster_size_for(ncell);
     if (G < 1) return PE_EINVAL;
-    return launch_newton_cluster(G, reinterpret_cast<const long long*>(rho_fx), ncell, dx, nscale, mode,
-                                 boundary == PE_BOUNDARY_ABSORBING, tol, maxit, phi, E, Ef, diag, status, phi_prev,
-                                 extrap, s);
+    const FieldDesc d = field_desc(rho_fx, ncell, dx, s_w, mode, boundary == PE_BOUNDARY_ABSORBING, tol, maxit, phi, E, Ef,
+                                   diag, status, phi_prev, extrap);
+    return launch_newton_cluster(G, d, s);
 }
 }  // namespace pe
 

@@ -39,15 +39,14 @@ int ensure_smem(const void* kernel, size_t smem);
 // Resident blocks per SM for (kernel, block, smem) on the current device (cached).
 int blocks_per_sm(const void* kernel, int block, size_t smem);
 
-// Batched field solves (pe_field.cu): descriptor size, descriptor builder, cluster size
-// used for a grid of ncell nodes, and the launch over R realisations of one cluster size.
+// Batched field solves (pe_field.cu): descriptor size, descriptor builder, the cluster size of a
+// realisation's solve (0: the grid does not fit), the launch over R realisations of one grid size.
 size_t field_desc_size();
 void make_field_desc(void* out, const int64_t* rho, int ncell, double dx, int s_w, int mode, int walls, double tol,
                      int maxit, double* phi, double* E, float* Ef, int32_t* diag, uint32_t* status,
                      double* phi_prev);
-int newton_cluster_size(int ncell);
 int newton_batch_cluster_size(int ncell);
-int launch_newton_batch(const void* descs, int R, int G, int max_ncell, bool fp64, bool extrap, cudaStream_t s);
+int launch_newton_batch(const void* descs, int R, int ncell, bool extrap, cudaStream_t s);
 // Single field solve whose Newton start may extrapolate the solution history (context path).
 int field_solve_history(const int64_t* rho_fx, int ncell, double dx, int s_w, int mode, int boundary, double tol,
                         int maxit, double* phi, double* E, float* Ef, int32_t* diag, uint32_t* status,
@@ -108,11 +107,6 @@ constexpr int kFullGridMax = 8192;     // largest grid the context API accepts
 constexpr int kRhoWindowNodes = 1024;  // charge deposit: window around the block's cells
 constexpr int kWindowNodes = 4096;     // restriction samples: window (co-moving spread)
 constexpr int kWindowNodesE = 1024;    // the same with the second moment (three rows in shared memory)
-// Bounded grids (vacuum regions, exp(phi) ~ 1e-6, cond(J) ~ 1e7) slow the FP32 Jacobian solve's
-// contraction: about 7 Newton updates instead of 3 on the 8192-node slab from a warm start. Each
-// FP32 update costs so much less than an FP64 one that the field solve is still faster (56 against
-// 125 us on the slab), so the FP64 elimination stays compiled but unused (true selects it).
-constexpr bool kWallsJacobianFP64 = false;
 // TMA tensor map of a K-major BF16 GEMM operand: rows x K elements, row stride ld elements,
 // box {64, box_rows}, 128-byte swizzle, zero fill (pe_tc.cu).
 int tc_operand_map(::CUtensorMap_st* map, const void* base, int64_t rows, int64_t K, int64_t ld, int box_rows);

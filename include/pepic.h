@@ -889,8 +889,7 @@ enum pe_mlp_buffer {
     PE_MLP_ADAM_M,      /* f32[nparams] first moments */
     PE_MLP_ADAM_V,      /* f32[nparams] second moments */
     PE_MLP_NORM,        /* f32[4][dmax] mu_in, sd_in, mu_out, sd_out; statistics scratch; step, loss */
-    PE_MLP_WORK,        /* batch workspace for max_batch rows: activations and gradients, and their
-                           transposes (the weight-gradient GEMMs contract over the batch) */
+    PE_MLP_WORK,        /* batch workspace for max_batch rows: activations and gradients */
     PE_MLP_NBUF
 };
 typedef struct pe_mlp_layout {

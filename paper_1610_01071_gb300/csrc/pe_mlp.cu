@@ -1,12 +1,19 @@
 // Learned coarse-derivative surrogate: a multilayer perceptron c -> dc/dt trained on the
 // least-squares slopes that resolved bursts measure (Section 3.3, Eq. (leastsquares)),
 // with BF16 tensor-core GEMMs accumulating in FP32, GELU hidden layers, MSE loss and
-// Adam. Every layer's forward, data-gradient and weight-gradient product is one launch of
-// the tcgen05 GEMM of pe_tc.cuh (TMEM accumulator, TMA-staged operands) with the bias,
-// activation, loss or GELU' factor fused into its epilogue. That kernel takes both operands
-// with K contiguous, so the products that contract over another index read transposed
-// copies kept alongside: the BF16 weights' transposes (rewritten with the mirror by Adam),
-// and the activations' and gradients' transposes (written by the epilogues that produce them).
+// Adam. Every product runs on the tcgen05 tile of pe_tc.cuh (TMEM accumulator, TMA-staged operands)
+// with the bias, activation, loss or GELU' factor fused into its epilogue: one launch per layer
+// forward and per data gradient, one launch for all weight gradients. The weight gradients
+// contract over the batch and read the row-major activations and gradients as they are
+// (operands with M and N contiguous); the data gradients read the BF16 weights' transposes
+// (rewritten with the mirror by Adam).
+//
+// What bounds a training step: the chain of its launches. Each product of the usual widths (512,
+// batch 2048) is under 1 us of tensor-core time, so the work around it sets the time: a step
+// of 512-512-512-512-512 at batch 2048 took 266 us in 25 launches (epilogues writing every row
+// in 4-byte pieces and a second time transposed, an Adam kernel finding each weight's place with
+// 64-bit divisions) and takes 95 us in 10, each started under its predecessor's tail
+// (programmatic dependent launch).
 //
 // Storage (caller-owned arena, see pe_mlp_layout_for): FP32 master parameters (the flat
 // vector W_1 [d1][d0], b_1, W_2, ...), their BF16 mirror and its per-layer transposes used by
@@ -34,7 +41,7 @@ namespace {
 constexpr int kNormBlocks = 64;    // row blocks of the z-score statistics
 constexpr int kLossSlots = 4096;
 
-enum Epi { kEpiHidden = 0, kEpiOutInfer = 1, kEpiOutTrain = 2, kEpiDgrad = 3, kEpiWgrad = 4 };
+enum Epi { kEpiHidden = 0, kEpiHiddenInfer = 1, kEpiOutInfer = 2, kEpiOutTrain = 3, kEpiDgrad = 4, kEpiWgrad = 5 };
 
 __device__ __forceinline__ float warp_sum_f(float v)
 {
@@ -64,69 +71,80 @@ struct GemmArgs {
     float gscale;          // train: 2 / (B D)
 };
 
-// Epilogue of the tensor-core GEMM for row m, columns n0 .. n0 + 31 of C = A B^T (FP32 from
-// TMEM): the bias + GELU of a hidden layer (Z, Aout and its transpose AoutT), the
-// de-normalised output (inference), the loss and output gradient (training; Y optional, G and
-// its transpose), the data gradient times GELU'(Z) (G and its transpose), or the FP32 weight
-// gradient. Rows beyond M are not stored. finish() folds the training loss of the block into
-// loss_part[block] (every thread calls it).
+__device__ __forceinline__ uint32_t bf16_pair(float a, float b)
+{
+    const __nv_bfloat162 p = __floats2bfloat162_rn(a, b);
+    return *reinterpret_cast<const uint32_t*>(&p);
+}
+
+// Epilogue of the tensor-core GEMM for row m, columns n0 .. n0 + 31 of C (FP32 from TMEM): the
+// bias + GELU of a hidden layer (Aout, and Z in training), the de-normalised output (inference),
+// the loss and output gradient (training), the data gradient times GELU'(Z), or the FP32 weight
+// gradient. Rows beyond M are not stored. A lane holds a whole row piece, so rows go to memory in
+// 32-byte vectors (every arena row is 128-byte aligned). finish() folds the training loss of
+// the block into loss_part[block] (every thread calls it).
 template <int EPI>
 struct TcEpi {
     GemmArgs g;
-    __nv_bfloat16* AoutT;  // transposed BF16 output [N][ldT]
-    int ldT;
     float lsum;
 
     __device__ __forceinline__ void operator()(int m, int n0, const float* v)
     {
         if (m >= g.M) return;
         const size_t o = (size_t)m * g.N + n0;
-        if (EPI == kEpiWgrad) {
-            float4* d = reinterpret_cast<float4*>(g.Y + o);
+        uint32_t r[8], a[8];
 #pragma unroll
-            for (int j = 0; j < 8; ++j) d[j] = make_float4(v[4 * j], v[4 * j + 1], v[4 * j + 2], v[4 * j + 3]);
-            return;
-        }
+        for (int j0 = 0; j0 < 32; j0 += 16) {
 #pragma unroll
-        for (int j = 0; j < 32; j += 2) {
-            const int n = n0 + j;
-            float v0 = v[j], v1 = v[j + 1];
-            if (EPI == kEpiHidden) {
-                v0 += g.bias[n];
-                v1 += g.bias[n + 1];
-                *reinterpret_cast<float2*>(g.Z + o + j) = make_float2(v0, v1);
-                const __nv_bfloat162 a = __floats2bfloat162_rn(gelu_f(v0), gelu_f(v1));
-                *reinterpret_cast<__nv_bfloat162*>(g.Aout + o + j) = a;
-                AoutT[(size_t)n * ldT + m] = a.x;
-                AoutT[(size_t)(n + 1) * ldT + m] = a.y;
-            } else if (EPI == kEpiOutInfer) {
-                v0 += g.bias[n];
-                v1 += g.bias[n + 1];
-                const float y0 = fmaf(v0, g.sd[n], g.mu[n]), y1 = fmaf(v1, g.sd[n + 1], g.mu[n + 1]);
-                if (g.Y64) {
-                    g.Y64[o + j] = (double)y0;
-                    g.Y64[o + j + 1] = (double)y1;
+            for (int q = 0; q < 16; q += 8) {
+                const int j = j0 + q;
+                if (EPI == kEpiWgrad) {
+#pragma unroll
+                    for (int k = 0; k < 8; ++k) r[k] = __float_as_uint(v[j + k]);
+                    tc::st_global32(g.Y + o + j, r);
+                } else if (EPI == kEpiOutInfer) {
+#pragma unroll
+                    for (int k = 0; k < 8; k += 2) {
+                        const int n = n0 + j + k;
+                        const float v0 = v[j + k] + g.bias[n], v1 = v[j + k + 1] + g.bias[n + 1];
+                        const float y0 = fmaf(v0, g.sd[n], g.mu[n]), y1 = fmaf(v1, g.sd[n + 1], g.mu[n + 1]);
+                        if (g.Y64) {
+                            g.Y64[o + j + k] = (double)y0;
+                            g.Y64[o + j + k + 1] = (double)y1;
+                        } else {
+                            *reinterpret_cast<float2*>(g.Y + o + j + k) = make_float2(y0, y1);
+                        }
+                    }
                 } else {
-                    *reinterpret_cast<float2*>(g.Y + o + j) = make_float2(y0, y1);
+                    float b[8], x[8];
+                    if (EPI == kEpiDgrad) tc::ld_global32(g.Z + o + j, r);
+                    else if (EPI == kEpiOutTrain) tc::ld_global32(g.T + o + j, r);
+                    if (EPI != kEpiDgrad) {  // the same address in every lane
+                        const float4 b0 = *reinterpret_cast<const float4*>(g.bias + n0 + j);
+                        const float4 b1 = *reinterpret_cast<const float4*>(g.bias + n0 + j + 4);
+                        b[0] = b0.x, b[1] = b0.y, b[2] = b0.z, b[3] = b0.w;
+                        b[4] = b1.x, b[5] = b1.y, b[6] = b1.z, b[7] = b1.w;
+                    }
+#pragma unroll
+                    for (int k = 0; k < 8; ++k) {
+                        if (EPI == kEpiHidden || EPI == kEpiHiddenInfer) {
+                            const float z = v[j + k] + b[k];
+                            r[k] = __float_as_uint(z);
+                            x[k] = gelu_f(z);
+                        } else if (EPI == kEpiOutTrain) {
+                            const float d = (v[j + k] + b[k]) - __uint_as_float(r[k]);
+                            lsum = fmaf(d, d, lsum);
+                            x[k] = g.gscale * d;
+                        } else {
+                            x[k] = v[j + k] * gelu_grad_f(__uint_as_float(r[k]));
+                        }
+                    }
+                    if (EPI == kEpiHidden) tc::st_global32(g.Z + o + j, r);
+#pragma unroll
+                    for (int k = 0; k < 8; k += 2) a[q / 2 + k / 2] = bf16_pair(x[k], x[k + 1]);
                 }
-            } else if (EPI == kEpiOutTrain) {
-                v0 += g.bias[n];
-                v1 += g.bias[n + 1];
-                const float2 t = *reinterpret_cast<const float2*>(g.T + o + j);
-                const float d0 = v0 - t.x, d1 = v1 - t.y;
-                lsum = fmaf(d0, d0, fmaf(d1, d1, lsum));
-                if (g.Y) *reinterpret_cast<float2*>(g.Y + o + j) = make_float2(v0, v1);
-                const __nv_bfloat162 gr = __floats2bfloat162_rn(g.gscale * d0, g.gscale * d1);
-                *reinterpret_cast<__nv_bfloat162*>(g.Aout + o + j) = gr;
-                AoutT[(size_t)n * ldT + m] = gr.x;
-                AoutT[(size_t)(n + 1) * ldT + m] = gr.y;
-            } else if (EPI == kEpiDgrad) {
-                const float2 z = *reinterpret_cast<const float2*>(g.Z + o + j);
-                const __nv_bfloat162 gr = __floats2bfloat162_rn(v0 * gelu_grad_f(z.x), v1 * gelu_grad_f(z.y));
-                *reinterpret_cast<__nv_bfloat162*>(g.Aout + o + j) = gr;
-                AoutT[(size_t)n * ldT + m] = gr.x;
-                AoutT[(size_t)(n + 1) * ldT + m] = gr.y;
             }
+            if (EPI != kEpiWgrad && EPI != kEpiOutInfer) tc::st_global32(g.Aout + o + j0, a);
         }
     }
 
@@ -144,6 +162,122 @@ struct TcEpi {
         }
     }
 };
+
+// Layer of a small batch (at most kSmallBatch rows; the gated macro step evaluates one): the
+// product with its roles exchanged, C^T[n][b] = sum_k W[n][k] x[b][k], 128 outputs per block as the
+// MMA's rows and the batch as its 32 columns. A thread then finishes one output, where the other
+// form leaves the whole epilogue of a row to two lanes of the block. The weights are loaded before
+// the wait for the previous layer. Same sums as the other form (the accumulation runs over k in
+// the same order).
+constexpr int kSmallBatch = 32;
+constexpr int kSmallStages = 8;  // K = 512 in flight at once
+constexpr int kSmallABytes = 128 * tc::kBK * 2, kSmallBBytes = kSmallBatch * tc::kBK * 2;
+constexpr int kSmallStageBytes = kSmallABytes + kSmallBBytes;
+constexpr int kSmallSmem = kSmallStages * kSmallStageBytes + 1024 + 8 * (2 * kSmallStages + 1) + 16;
+
+template <bool LAST>
+__global__ void __launch_bounds__(128, 1) k_mlp_small(const __grid_constant__ CUtensorMap tw,
+                                                      const __grid_constant__ CUtensorMap tx, GemmArgs g,
+                                                      uint32_t* status)
+{
+    using namespace tc;
+    extern __shared__ uint8_t smem_raw[];
+    uint8_t* smem = reinterpret_cast<uint8_t*>((reinterpret_cast<uintptr_t>(smem_raw) + 1023) & ~uintptr_t(1023));
+    uint64_t* full = reinterpret_cast<uint64_t*>(smem + kSmallStages * kSmallStageBytes);
+    uint64_t* empty = full + kSmallStages;
+    uint64_t* done = empty + kSmallStages;
+    uint32_t* tmem_slot = reinterpret_cast<uint32_t*>(done + 1);
+    __shared__ int s_fail;
+    const int tid = threadIdx.x, warp = tid >> 5, lane = tid & 31;
+    const int n0 = (int)blockIdx.x * 128;
+    const int ktiles = (g.K + kBK - 1) / kBK, pro = ktiles < kSmallStages ? ktiles : kSmallStages;
+    if (tid == 0) {
+        for (int s = 0; s < kSmallStages; ++s) {
+            mbar_init(&full[s], 1);
+            mbar_init(&empty[s], 1);
+        }
+        mbar_init(done, 1);
+        fence_mbar_init();
+        s_fail = 0;
+        for (int t = 0; t < pro; ++t) {
+            mbar_expect_tx(&full[t], kSmallStageBytes);
+            tma_load_2d(smem + t * kSmallStageBytes, &tw, &full[t], t * kBK, n0);
+        }
+    }
+    if (warp == 0) tmem_alloc(tmem_slot, 32);
+    tc_fence_before();
+    __syncthreads();
+    tc_fence_after();
+    const uint32_t tmem = *tmem_slot;
+    grid_release();
+    grid_wait();
+    if (tid == 0) {
+        for (int t = 0; t < pro; ++t)
+            tma_load_2d(smem + t * kSmallStageBytes + kSmallABytes, &tx, &full[t], t * kBK, 0);
+        int issued = pro, consumed = 0;
+        bool ok = true;
+        for (int kt = 0; kt < ktiles; ++kt) {
+            const int s = kt % kSmallStages;
+            if (!mbar_wait(&full[s], (uint32_t)((kt / kSmallStages) & 1))) {
+                ok = false;
+                break;
+            }
+            consumed = kt + 1;
+            tc_fence_after();
+            const uint32_t a0 = saddr(smem + s * kSmallStageBytes), b0 = a0 + kSmallABytes;
+#pragma unroll
+            for (int k = 0; k < kBK / 16; ++k)
+                umma_bf16(tmem, sw128_desc(a0 + 32 * k), sw128_desc(b0 + 32 * k), idesc_bf16(128, kSmallBatch),
+                          (kt | k) ? 1u : 0u);
+            umma_commit(&empty[s]);
+            const int t = kt - 1 + kSmallStages;
+            if (kt >= 1 && t < ktiles) {
+                const int q = (kt - 1) % kSmallStages;
+                if (!mbar_wait(&empty[q], (uint32_t)(((kt - 1) / kSmallStages) & 1))) {
+                    ok = false;
+                    break;
+                }
+                mbar_expect_tx(&full[q], kSmallStageBytes);
+                tma_load_2d(smem + q * kSmallStageBytes, &tw, &full[q], t * kBK, n0);
+                tma_load_2d(smem + q * kSmallStageBytes + kSmallABytes, &tx, &full[q], t * kBK, 0);
+                ++issued;
+            }
+        }
+        umma_commit(done);
+        if (!ok) {
+            s_fail = 1;
+            for (int t = consumed; t < issued; ++t)
+                mbar_wait(&full[t % kSmallStages], (uint32_t)((t / kSmallStages) & 1));
+        }
+    }
+    __syncthreads();
+    bool ok = mbar_wait(done, 0u) && !s_fail;
+    ok = __all_sync(0xFFFFFFFFu, ok);
+    if (!ok && lane == 0) atomicOr(status, PE_FLAG_TIMEOUT);
+    tc_fence_after();
+    if (ok) {
+        const int n = n0 + warp * 32 + lane;
+        float v[32];
+        tmem_ld32(tmem + ((uint32_t)(warp * 32) << 16), v);
+        if (n < g.N) {
+            const float bias = g.bias[n];
+            const float sd = LAST ? g.sd[n] : 0.0f, mu = LAST ? g.mu[n] : 0.0f;
+#pragma unroll
+            for (int b = 0; b < 32; ++b) {
+                if (b < g.M) {
+                    const float z = v[b] + bias;
+                    const size_t o = (size_t)b * g.N + n;
+                    if (!LAST) g.Aout[o] = __float2bfloat16_rn(gelu_f(z));
+                    else if (g.Y64) g.Y64[o] = (double)fmaf(z, sd, mu);
+                    else g.Y[o] = fmaf(z, sd, mu);
+                }
+            }
+        }
+    }
+    tc_fence_before();
+    __syncthreads();
+    if (warp == 0) tmem_dealloc(tmem, 32);
+}
 
 // ------------------------------------------------------------------ small kernels
 
@@ -271,102 +405,236 @@ __global__ void k_norm_final(const double* __restrict__ part, int nparts, int D,
     for (int k = threadIdx.x; k < D; k += blockDim.x) out32[k] = (float)fmax(acc64[D + k], smax);
 }
 
-// Batch rows and translation shifts for a training step, from the splitmix64 sequence of
-// (seed, step): row = (h >> 32) npairs >> 32, shift = (h mod 2^32) P >> 32.
-__global__ void k_sample_rows(uint64_t seed, const int64_t* __restrict__ step, int B, int64_t npairs, int P,
-                              int32_t* __restrict__ rows, int32_t* __restrict__ shifts)
-{
-    const int i = blockIdx.x * blockDim.x + threadIdx.x;
-    if (i >= B) return;
-    const uint64_t h = splitmix64_seq(seed, (uint64_t)(*step) * (uint64_t)B + (uint64_t)i);
-    rows[i] = (int32_t)(((h >> 32) * (uint64_t)npairs) >> 32);
-    shifts[i] = P > 0 ? (int32_t)(((h & 0xFFFFFFFFull) * (uint64_t)P) >> 32) : 0;
-}
-
-// Normalised BF16 inputs (and FP32 targets) of a batch: x'[k] = x[src(k)] with the
-// circular shift s inside each block of P components, src(k) = b P + (j - s) mod P.
+// Normalised BF16 inputs (and FP32 targets) of a batch, one row per block: x'[k] = x[src(k)] with
+// the circular shift s inside each block of P components, src(k) = b P + (j - s) mod P. The row
+// and shift come from rows (shift 0), or, drawing a training batch (step not null), from the
+// splitmix64 sequence of (seed, step): row = (h >> 32) npairs >> 32, shift = (h mod 2^32) P >> 32;
+// else block i takes row i.
 template <typename T>
-__global__ void k_prep(const T* __restrict__ X, const float* __restrict__ Y, int B, int D, int Dout,
-                       const int32_t* __restrict__ rows, const int32_t* __restrict__ shifts, int P,
-                       const float* __restrict__ mu, const float* __restrict__ sd, const float* __restrict__ mu_o,
-                       const float* __restrict__ sd_o, __nv_bfloat16* __restrict__ xz, __nv_bfloat16* __restrict__ xzT,
-                       int ldT, float* __restrict__ tz)
+__global__ void __launch_bounds__(128) k_prep(const T* __restrict__ X, const float* __restrict__ Y, int B, int D,
+                                              int Dout, const int32_t* __restrict__ rows,
+                                              const int64_t* __restrict__ step, uint64_t seed, int64_t npairs, int P,
+                                              const float* __restrict__ mu, const float* __restrict__ sd,
+                                              const float* __restrict__ mu_o, const float* __restrict__ sd_o,
+                                              __nv_bfloat16* __restrict__ xz, float* __restrict__ tz)
 {
-    const int i = blockIdx.y;
-    if (i >= B) return;
-    const int64_t r = rows ? rows[i] : i;
-    const int s = shifts ? shifts[i] : 0;
-    for (int k = blockIdx.x * blockDim.x + threadIdx.x; k < max(D, Dout); k += gridDim.x * blockDim.x) {
-        int src = k;
-        if (P > 0) {
-            const int j = k % P;
-            src = k - j + (j - s + P) % P;
-        }
-        if (k < D) {
-            const float x = (float)X[r * D + src];
-            const __nv_bfloat16 b = __float2bfloat16_rn((x - mu[k]) / sd[k]);
-            xz[(size_t)i * D + k] = b;
-            if (xzT) xzT[(size_t)k * ldT + i] = b;
-        }
-        if (Y && k < Dout) tz[(size_t)i * Dout + k] = (Y[r * Dout + src] - mu_o[k]) / sd_o[k];
+    tc::grid_release();
+    tc::grid_wait();
+    const int i = blockIdx.x;
+    int64_t r = rows ? rows[i] : i;
+    int s = 0;
+    if (step) {
+        const uint64_t h = splitmix64_seq(seed, (uint64_t)(*step) * (uint64_t)B + (uint64_t)i);
+        r = (int32_t)(((h >> 32) * (uint64_t)npairs) >> 32);
+        s = P > 0 ? (int32_t)(((h & 0xFFFFFFFFull) * (uint64_t)P) >> 32) : 0;
     }
+    auto source = [&](int k) {
+        if (P <= 0) return k;
+        const int j = k % P;
+        return k - j + (j >= s ? j - s : j - s + P);
+    };
+    // dims are multiples of 64: pairs of components, one 4-byte store each
+    for (int k = 2 * threadIdx.x; k < D; k += 2 * blockDim.x) {
+        const float x0 = (float)X[r * D + source(k)], x1 = (float)X[r * D + source(k + 1)];
+        reinterpret_cast<uint32_t*>(xz + (size_t)i * D)[k >> 1] =
+            bf16_pair((x0 - mu[k]) / sd[k], (x1 - mu[k + 1]) / sd[k + 1]);
+    }
+    if (Y)
+        for (int k = threadIdx.x; k < Dout; k += blockDim.x)
+            tz[(size_t)i * Dout + k] = (Y[r * Dout + source(k)] - mu_o[k]) / sd_o[k];
 }
 
-// Bias gradient db[n] = sum_m G[m][n] from the transposed gradient GT [N][ldT] (row n holds
-// G[0..M)[n] contiguously): one warp per n, lanes over m, FP32 partial sums folded in a
-// fixed order (reproducible).
-__global__ void k_bias_grad(const __nv_bfloat16* __restrict__ GT, int ldT, int M, int N, float* __restrict__ db)
+// Bias correction of Adam step t = *step + 1 into c[2], and the step counter advanced. The decay
+// rates come in FP64 (0.999 is not a float); one thread, once per step: the FP64 powers cost
+// microseconds on every thread that forms them.
+__device__ __forceinline__ void adam_begin(int64_t* step, float* c, double b1, double b2)
 {
-    const int n = blockIdx.x * (blockDim.x >> 5) + (threadIdx.x >> 5), lane = threadIdx.x & 31;
-    if (n >= N) return;
-    const __nv_bfloat16* row = GT + (size_t)n * ldT;
-    float s = 0.0f;
-    for (int m = lane; m < M; m += 32) s += __bfloat162float(row[m]);
-    s = warp_sum_f(s);
-    if (lane == 0) db[n] = s;
+    const int64_t t = *step + 1;
+    c[0] = (float)(1.0 / (1.0 - pow(b1, (double)t)));
+    c[1] = (float)(1.0 / (1.0 - pow(b2, (double)t)));
+    *step = t;
 }
 
-__global__ void k_loss_final(const float* __restrict__ part, int n, float* __restrict__ out, float scale)
+__global__ void k_adam_begin(int64_t* step, float* c, double b1, double b2)
 {
+    if (threadIdx.x == 0 && blockIdx.x == 0) adam_begin(step, c, b1, b2);
+}
+
+// All weight and bias gradients of the network and the loss, one launch: they depend only on the
+// forward and data-gradient passes, so the layers' tiles fill the GPU together (32 tiles of a
+// 512 x 512 layer alone leave four fifths of it idle for the length of a batch's reduction).
+// Blocks, in this order: per layer the tiles of dW_l [d_{l+1}][d_l] = G_l^T act_{l-1} (contraction
+// over the batch, operands row-major), then per layer the 64-column blocks of db_l, then one
+// block for the loss and, in a training step (adam), Adam's bias corrections.
+struct WgradArgs {
+    CUtensorMap a[PE_MLP_MAX_LAYERS], b[PE_MLP_MAX_LAYERS];  // G_l, act_{l-1}: dims {d, B}, boxes {64, 64}
+    const __nv_bfloat16* G[PE_MLP_MAX_LAYERS];
+    float* dW[PE_MLP_MAX_LAYERS];
+    float* db[PE_MLP_MAX_LAYERS];
+    int tile0[PE_MLP_MAX_LAYERS + 1], bias0[PE_MLP_MAX_LAYERS + 1];  // first block of each layer's tiles / columns
+    int M[PE_MLP_MAX_LAYERS], N[PE_MLP_MAX_LAYERS];
+    int L, B;
+    const float* loss_part;
+    int nloss;
+    float loss_scale;
+    float* loss;
+    int adam;
+    int64_t* step;
+    float* corr;
+    double b1, b2;
+};
+
+// Bias gradient db[n] = sum_m G[m][n] of 64 columns: 32 running sums per column (rows m = l mod 32,
+// FP32, in row order), folded pairwise (l with l + 16, then + 8, ...): a fixed order.
+__device__ __forceinline__ void bias_grad_block(const __nv_bfloat16* G, int B, int N, int n0, float* db, float* red)
+{
+    const int warp = threadIdx.x >> 5, lane = threadIdx.x & 31;
+    const uint32_t* G2 = reinterpret_cast<const uint32_t*>(G + n0) + lane;  // columns n0 + 2 lane, + 1
+    float s0[4], s1[4];
+#pragma unroll
+    for (int k = 0; k < 4; ++k) s0[k] = s1[k] = 0.0f;
+#pragma unroll 4
+    for (int m = 4 * warp; m < B; m += 32) {  // B a multiple of 32
+        uint32_t u[4];
+#pragma unroll
+        for (int k = 0; k < 4; ++k) u[k] = __ldg(G2 + (size_t)(m + k) * (N / 2));
+#pragma unroll
+        for (int k = 0; k < 4; ++k) {
+            s0[k] += __uint_as_float(u[k] << 16);
+            s1[k] += __uint_as_float(u[k] & 0xFFFF0000u);
+        }
+    }
+#pragma unroll
+    for (int k = 0; k < 4; ++k) {
+        red[(4 * warp + k) * 64 + 2 * lane] = s0[k];
+        red[(4 * warp + k) * 64 + 2 * lane + 1] = s1[k];
+    }
+    __syncthreads();
+    for (int h = 16; h > 0; h >>= 1) {
+        for (int t = threadIdx.x; t < h * 64; t += blockDim.x) red[t] += red[t + h * 64];
+        __syncthreads();
+    }
+    if (threadIdx.x < 64) db[n0 + threadIdx.x] = red[threadIdx.x];
+}
+
+__global__ void __launch_bounds__(tc::kThreads, 1) k_mlp_wgrad(const __grid_constant__ WgradArgs w, uint32_t* status)
+{
+    extern __shared__ uint8_t smem_raw[];
+    const int blk = blockIdx.x, L = w.L;
+    if (blk < w.tile0[L]) {
+        int l = 0;
+        while (blk >= w.tile0[l + 1]) ++l;
+        const int t = blk - w.tile0[l], nx = w.N[l] / 64;
+        TcEpi<kEpiWgrad> e{};
+        e.g.M = w.M[l];
+        e.g.N = w.N[l];
+        e.g.Y = w.dW[l];
+        tc::gemm_tile<64, true>(&w.a[l], &w.b[l], (t / nx) * tc::kBM, (t % nx) * 64, w.B, e, status);
+        return;
+    }
+    tc::grid_release();
+    tc::grid_wait();
+    if (blk < w.bias0[L]) {
+        int l = 0;
+        while (blk >= w.bias0[l + 1]) ++l;
+        bias_grad_block(w.G[l], w.B, w.M[l], 64 * (blk - w.bias0[l]), w.db[l], reinterpret_cast<float*>(smem_raw));
+        return;
+    }
     __shared__ double red[32];
     double s = 0.0;
-    for (int i = threadIdx.x; i < n; i += blockDim.x) s += (double)part[i];
+    for (int i = threadIdx.x; i < w.nloss; i += blockDim.x) s += (double)w.loss_part[i];
     s = warp_sum(s);
     if ((threadIdx.x & 31) == 0) red[threadIdx.x >> 5] = s;
     __syncthreads();
     if (threadIdx.x == 0) {
         double t = 0.0;
-        for (int w = 0; w < (int)(blockDim.x >> 5); ++w) t += red[w];
-        *out = (float)(t * scale);
+        for (int k = 0; k < (int)(blockDim.x >> 5); ++k) t += red[k];
+        *w.loss = (float)(t * w.loss_scale);
+        if (w.adam) adam_begin(w.step, w.corr, w.b1, w.b2);
     }
 }
 
-// Adam with bias correction; the step counter lives on the device (graph replays
-// advance it). theta, m, v FP32; the BF16 mirror is rewritten. The decay rates and their
-// complements come in FP64 (0.999 is not a float) and the bias corrections are formed in
-// FP64 once per thread.
-__global__ void k_adam(float* __restrict__ p, __nv_bfloat16* __restrict__ pb, __nv_bfloat16* __restrict__ pbT,
-                       WeightTable wt, const float* __restrict__ grad, float* __restrict__ m, float* __restrict__ v,
-                       int64_t n, int64_t* __restrict__ step, float lr, double b1, double b2, float eps)
+// Adam with bias correction (corr: adam_begin's factors; the step counter lives on the device, so
+// graph replays advance it). theta, m, v FP32; the BF16 mirror and its transposes are rewritten.
+// The decay rates and their complements come in FP64 (0.999 is not a float). Bound by memory (32
+// bytes per parameter; L2 holds the arrays of the usual networks): a block takes a 64 x 64 tile of
+// one layer's weights, so that the mirror's transpose leaves through shared memory in rows of 128
+// bytes; the last blocks take the biases. (One thread per parameter at any index, with the
+// transposed store at a stride and 64-bit divisions to find it: 51 us for 10^6 parameters, 9 us
+// now.)
+__global__ void __launch_bounds__(256) k_adam(float* __restrict__ p, __nv_bfloat16* __restrict__ pb,
+                                              __nv_bfloat16* __restrict__ pbT, WeightTable wt,
+                                              const float* __restrict__ grad, float* __restrict__ m,
+                                              float* __restrict__ v, const float* __restrict__ corr, float lr, double b1,
+                                              double b2, float eps)
 {
-    const int64_t t = *step + 1;
-    const float c1 = (float)(1.0 / (1.0 - pow(b1, (double)t))), c2 = (float)(1.0 / (1.0 - pow(b2, (double)t)));
+    __shared__ __nv_bfloat16 tile[64][66];
+    tc::grid_release();
+    tc::grid_wait();
+    const float c1 = corr[0], c2 = corr[1];
     const float fb1 = (float)b1, fb2 = (float)b2, ob1 = (float)(1.0 - b1), ob2 = (float)(1.0 - b2);
-    for (int64_t i = (int64_t)blockIdx.x * blockDim.x + threadIdx.x; i < n; i += (int64_t)gridDim.x * blockDim.x) {
-        const float gi = grad[i];
-        const float mi = fmaf(fb1, m[i], ob1 * gi);
-        const float vi = fmaf(fb2, v[i], ob2 * gi * gi);
-        m[i] = mi;
-        v[i] = vi;
-        const float w = p[i] - lr * (mi * c1) / (sqrtf(vi * c2) + eps);
-        p[i] = w;
-        put_bf16(wt, i, w, pb, pbT);
+    auto update = [&](float& w, float& mi, float& vi, float gi) {
+        mi = fmaf(fb1, mi, ob1 * gi);
+        vi = fmaf(fb2, vi, ob2 * gi * gi);
+        w = w - lr * (mi * c1) / (sqrtf(vi * c2) + eps);
+    };
+    int blk = blockIdx.x, l = 0;
+    for (; l < wt.L; ++l) {
+        const int n = (wt.rows[l] / 64) * (wt.cols[l] / 64);
+        if (blk < n) break;
+        blk -= n;
     }
-}
-
-__global__ void k_step_advance(int64_t* step)
-{
-    if (threadIdx.x == 0 && blockIdx.x == 0) *step += 1;
+    if (l == wt.L) {  // biases, 256 per block
+        for (l = 0; l < wt.L; ++l) {
+            const int n = (wt.rows[l] + 255) / 256;
+            if (blk < n) break;
+            blk -= n;
+        }
+        const int k = 256 * blk + threadIdx.x;
+        if (l < wt.L && k < wt.rows[l]) {
+            const int64_t i = wt.off[l] + (int64_t)wt.rows[l] * wt.cols[l] + k;
+            float w = p[i], mi = m[i], vi = v[i];
+            update(w, mi, vi, grad[i]);
+            m[i] = mi;
+            v[i] = vi;
+            p[i] = w;
+            pb[i] = __float2bfloat16_rn(w);
+        }
+        return;
+    }
+    const int rows = wt.rows[l], cols = wt.cols[l], nx = cols / 64;
+    const int r0 = 64 * (blk / nx), c0 = 64 * (blk % nx);
+    const int tr = threadIdx.x >> 4, tc4 = 4 * (threadIdx.x & 15);
+#pragma unroll
+    for (int q = 0; q < 4; ++q) {
+        const int r = tr + 16 * q;
+        const int64_t i = wt.off[l] + (int64_t)(r0 + r) * cols + c0 + tc4;
+        float4 w4 = *reinterpret_cast<const float4*>(p + i), m4 = *reinterpret_cast<const float4*>(m + i);
+        float4 v4 = *reinterpret_cast<const float4*>(v + i);
+        const float4 g4 = *reinterpret_cast<const float4*>(grad + i);
+        update(w4.x, m4.x, v4.x, g4.x);
+        update(w4.y, m4.y, v4.y, g4.y);
+        update(w4.z, m4.z, v4.z, g4.z);
+        update(w4.w, m4.w, v4.w, g4.w);
+        *reinterpret_cast<float4*>(p + i) = w4;
+        *reinterpret_cast<float4*>(m + i) = m4;
+        *reinterpret_cast<float4*>(v + i) = v4;
+        const uint2 b = make_uint2(bf16_pair(w4.x, w4.y), bf16_pair(w4.z, w4.w));
+        *reinterpret_cast<uint2*>(pb + i) = b;
+        uint32_t* t = reinterpret_cast<uint32_t*>(&tile[r][tc4]);
+        t[0] = b.x;
+        t[1] = b.y;
+    }
+    __syncthreads();
+    // transpose: column c of the tile is a row piece of 64 elements, four threads per column
+    const int c = threadIdx.x >> 2, k0 = 16 * (threadIdx.x & 3);
+    uint32_t o[8];
+#pragma unroll
+    for (int k = 0; k < 8; ++k) {
+        const __nv_bfloat162 t2 = __halves2bfloat162(tile[k0 + 2 * k][c], tile[k0 + 2 * k + 1][c]);
+        o[k] = *reinterpret_cast<const uint32_t*>(&t2);
+    }
+    tc::st_global32(pbT + wt.off[l] + (int64_t)(c0 + c) * rows + r0 + k0, o);
 }
 
 }  // namespace
@@ -395,19 +663,13 @@ struct pe_mlp {
     double* normpart;   // [kNormBlocks][dmax]
     int64_t* step;      // Adam step counter (device)
     float* loss;        // last training loss (device)
+    float* corr;        // [2] bias corrections of the current Adam step (device)
     float* loss_part;   // [kLossSlots]
-    int32_t* rows;
-    int32_t* shifts;
     __nv_bfloat16* xz;  // [Bm][d0]
     float* z[PE_MLP_MAX_LAYERS];
     __nv_bfloat16* a[PE_MLP_MAX_LAYERS];
-    float* y;           // [Bm][dL]
     float* tz;          // [Bm][dL]
-    __nv_bfloat16* g[2];
-    int ldT;             // row stride of the transposed batch arrays (max_batch rounded up to 64)
-    __nv_bfloat16* xzT;  // [d0][ldT]
-    __nv_bfloat16* aT[PE_MLP_MAX_LAYERS];  // [d_{l+1}][ldT]
-    __nv_bfloat16* gT[2];                  // [dmax][ldT]
+    __nv_bfloat16* g[PE_MLP_MAX_LAYERS];  // [Bm][d_{l+1}] gradient at layer l's output
     uint32_t* status;    // device status word (PE_FLAG_TIMEOUT from the GEMM's bounded waits)
     int shift_period;   // period used by the statistics (for reference)
 };
@@ -427,13 +689,10 @@ int check_dims(int32_t nlayers, const int32_t* dims, int32_t max_batch)
 }
 
 struct WorkPlan {
-    size_t rows, shifts, xz, z[PE_MLP_MAX_LAYERS], a[PE_MLP_MAX_LAYERS], y, tz, g0, g1, xzT, aT[PE_MLP_MAX_LAYERS],
-        gT0, gT1, total;
+    size_t xz, z[PE_MLP_MAX_LAYERS], a[PE_MLP_MAX_LAYERS], tz, g[PE_MLP_MAX_LAYERS], total;
 };
 
-int ld_transposed(int Bm) { return (Bm + 63) & ~63; }
-
-WorkPlan plan_work(int L, const int32_t* dims, int Bm, int dmax)
+WorkPlan plan_work(int L, const int32_t* dims, int Bm)
 {
     WorkPlan w;
     size_t o = 0;
@@ -442,29 +701,38 @@ WorkPlan plan_work(int L, const int32_t* dims, int Bm, int dmax)
         o += al256(bytes);
         return at;
     };
-    w.rows = take(4 * (size_t)Bm);
-    w.shifts = take(4 * (size_t)Bm);
     w.xz = take(2 * (size_t)Bm * dims[0]);
     for (int l = 0; l + 1 < L; ++l) {
         w.z[l] = take(4 * (size_t)Bm * dims[l + 1]);
         w.a[l] = take(2 * (size_t)Bm * dims[l + 1]);
     }
-    w.y = take(4 * (size_t)Bm * dims[L]);
     w.tz = take(4 * (size_t)Bm * dims[L]);
-    w.g0 = take(2 * (size_t)Bm * dmax);
-    w.g1 = take(2 * (size_t)Bm * dmax);
-    const size_t ldT = (size_t)ld_transposed(Bm);
-    w.xzT = take(2 * ldT * dims[0]);
-    for (int l = 0; l + 1 < L; ++l) w.aT[l] = take(2 * ldT * dims[l + 1]);
-    w.gT0 = take(2 * ldT * dmax);
-    w.gT1 = take(2 * ldT * dmax);
+    for (int l = 0; l < L; ++l) w.g[l] = take(2 * (size_t)Bm * dims[l + 1]);
     w.total = o;
     return w;
 }
 
+// Launch with the programmatic-dependence attribute: the kernel may start while its predecessor on
+// the stream drains (it waits with grid_wait before touching anything a predecessor wrote).
+template <class... P, class... A>
+int launch_dependent(void (*kernel)(P...), dim3 grid, int block, size_t smem, cudaStream_t s, A... args)
+{
+    if (ensure_smem((const void*)kernel, smem) != PE_OK) return PE_ECUDA;
+    cudaLaunchAttribute attr[1];
+    attr[0].id = cudaLaunchAttributeProgrammaticStreamSerialization;
+    attr[0].val.programmaticStreamSerializationAllowed = 1;
+    cudaLaunchConfig_t cfg = {};
+    cfg.gridDim = grid;
+    cfg.blockDim = dim3(block);
+    cfg.dynamicSmemBytes = smem;
+    cfg.stream = s;
+    cfg.attrs = attr;
+    cfg.numAttrs = 1;
+    return cudaLaunchKernelEx(&cfg, kernel, P(args)...) == cudaSuccess ? PE_OK : PE_ECUDA;
+}
+
 // C[M][N] = A[M][K] B[N][K]^T on the tensor cores with the epilogue EPI; A and B stored
-// with K contiguous (row strides lda, ldb). AoutT/ldT: transposed BF16 copy of the output.
-// Returns the number of tiles (one loss partial each).
+// with K contiguous (row strides lda, ldb).
 // Tile width: 128 columns, or 64 when N needs it or when 128-wide tiles would leave SMs idle.
 int tile_n(int N, int M)
 {
@@ -473,27 +741,29 @@ int tile_n(int N, int M)
 }
 
 template <int EPI>
-int tc_gemm(pe_mlp* h, const GemmArgs& g, __nv_bfloat16* AoutT, cudaStream_t s, int* tiles)
+int tc_gemm(pe_mlp* h, const GemmArgs& g, cudaStream_t s)
 {
     const int bn = tile_n(g.N, g.M);
     CUtensorMap ma, mb;
     PE_TRY(tc_operand_map(&ma, g.A, g.M, g.K, g.lda, tc::kBM));
     PE_TRY(tc_operand_map(&mb, g.B, g.N, g.K, g.ldb, bn));
-    TcEpi<EPI> e{g, AoutT, h->ldT, 0.0f};
-    dim3 grid(g.N / bn, (g.M + tc::kBM - 1) / tc::kBM);
-    if (tiles) *tiles = (int)(grid.x * grid.y);
-    if (bn == 128) {
-        const void* k = (const void*)tc::k_tc_gemm<128, TcEpi<EPI>>;
-        if (ensure_smem(k, tc::TileCfg<128>::kSmemBytes) != PE_OK) return PE_ECUDA;
-        tc::k_tc_gemm<128, TcEpi<EPI>><<<grid, tc::kThreads, tc::TileCfg<128>::kSmemBytes, s>>>(ma, mb, g.M, g.K, e,
-                                                                                               h->status);
-    } else {
-        const void* k = (const void*)tc::k_tc_gemm<64, TcEpi<EPI>>;
-        if (ensure_smem(k, tc::TileCfg<64>::kSmemBytes) != PE_OK) return PE_ECUDA;
-        tc::k_tc_gemm<64, TcEpi<EPI>><<<grid, tc::kThreads, tc::TileCfg<64>::kSmemBytes, s>>>(ma, mb, g.M, g.K, e,
-                                                                                             h->status);
-    }
-    return PE_OK;
+    TcEpi<EPI> e{g, 0.0f};
+    const dim3 grid(g.N / bn, (g.M + tc::kBM - 1) / tc::kBM);
+    if (bn == 128)
+        return launch_dependent(tc::k_tc_gemm<128, TcEpi<EPI>>, grid, tc::kThreads, tc::TileCfg<128>::kSmemBytes, s, ma, mb,
+                                g.K, e, h->status);
+    return launch_dependent(tc::k_tc_gemm<64, TcEpi<EPI>>, grid, tc::kThreads, tc::TileCfg<64>::kSmemBytes, s, ma, mb, g.K,
+                            e, h->status);
+}
+
+// One layer of a small batch (inference): the product with its roles exchanged.
+template <bool LAST>
+int small_layer(pe_mlp* h, const GemmArgs& g, cudaStream_t s)
+{
+    CUtensorMap mw, mx;
+    PE_TRY(tc_operand_map(&mw, g.B, g.N, g.K, g.ldb, 128));
+    PE_TRY(tc_operand_map(&mx, g.A, g.M, g.K, g.lda, kSmallBatch));
+    return launch_dependent(k_mlp_small<LAST>, dim3((g.N + 127) / 128), 128, kSmallSmem, s, mw, mx, g, h->status);
 }
 
 // Loss partials of the output layer's GEMM (one per tile).
@@ -501,12 +771,14 @@ int loss_tiles(int Dout, int B) { return (Dout / tile_n(Dout, B)) * ((B + tc::kB
 
 GemmArgs args0() { GemmArgs g; memset(&g, 0, sizeof(g)); return g; }
 
-// Forward through every layer from h->xz (rows B). mode 0: inference, output into
-// y32 / y64 de-normalised; mode 1: training, output compared with h->tz.
+// Forward through every layer from h->xz (rows B). Inference: output into y32 / y64
+// de-normalised; training: output compared with h->tz.
 int forward(pe_mlp* h, int B, int train, float* y32, double* y64, int* launches)
 {
     cudaStream_t s = h->stream;
     const __nv_bfloat16* in = h->xz;
+    // batches of up to 32 rows: one 128-row tile of the usual form would be mostly padding
+    const bool small = !train && B <= kSmallBatch;
     for (int l = 0; l < h->L; ++l) {
         GemmArgs g = args0();
         g.A = in;
@@ -520,50 +792,39 @@ int forward(pe_mlp* h, int B, int train, float* y32, double* y64, int* launches)
         if (l + 1 < h->L) {
             g.Z = h->z[l];
             g.Aout = h->a[l];
-            PE_TRY(tc_gemm<kEpiHidden>(h, g, h->aT[l], s, nullptr));
+            if (small) PE_TRY(small_layer<false>(h, g, s));
+            else if (train) PE_TRY(tc_gemm<kEpiHidden>(h, g, s));
+            else PE_TRY(tc_gemm<kEpiHiddenInfer>(h, g, s));
             in = h->a[l];
         } else if (!train) {
             g.Y = y32;
             g.Y64 = y64;
             g.mu = h->norm + 2 * h->dmax;
             g.sd = h->norm + 3 * h->dmax;
-            PE_TRY(tc_gemm<kEpiOutInfer>(h, g, nullptr, s, nullptr));
+            if (small) PE_TRY(small_layer<true>(h, g, s));
+            else PE_TRY(tc_gemm<kEpiOutInfer>(h, g, s));
         } else {
             g.T = h->tz;
-            g.Y = h->y;
-            g.Aout = h->g[(h->L - 1) & 1];
+            g.Aout = h->g[l];
             g.loss_part = h->loss_part;
             g.gscale = 2.0f / ((float)B * (float)g.N);
-            PE_TRY(tc_gemm<kEpiOutTrain>(h, g, h->gT[(h->L - 1) & 1], s, nullptr));
+            PE_TRY(tc_gemm<kEpiOutTrain>(h, g, s));
         }
         ++*launches;
     }
     return PE_OK;
 }
 
-// Backward from the output gradient in g[(L-1)&1]: weight and bias gradients of every
-// layer into h->grad, data gradients (times GELU') down to layer 1.
-int backward(pe_mlp* h, int B, int* launches)
+// Backward from the output gradient in g[L-1]: data gradients (times GELU') down to layer 1, then
+// the weight and bias gradients of every layer into h->grad, the loss, and with adam the bias
+// corrections of the step.
+int backward(pe_mlp* h, int B, bool adam, double b1, double b2, int* launches)
 {
     cudaStream_t s = h->stream;
-    for (int l = h->L - 1; l >= 0; --l) {
-        const __nv_bfloat16* gl = h->g[l & 1];
-        GemmArgs w = args0();  // dW_l [d_{l+1}][d_l] = G_l^T act_{l-1}: both transposes, K = batch
-        w.A = h->gT[l & 1];
-        w.B = l ? h->aT[l - 1] : h->xzT;
-        w.M = h->dims[l + 1];
-        w.N = h->dims[l];
-        w.K = B;
-        w.lda = h->ldT;
-        w.ldb = h->ldT;
-        w.Y = h->grad + h->w_off[l];
-        PE_TRY(tc_gemm<kEpiWgrad>(h, w, nullptr, s, nullptr));
-        k_bias_grad<<<(h->dims[l + 1] + 7) / 8, 256, 0, s>>>(h->gT[l & 1], h->ldT, B, h->dims[l + 1],
-                                                             h->grad + h->b_off[l]);
-        *launches += 2;
-        if (l == 0) break;
+    const int L = h->L, Dout = h->dims[L];
+    for (int l = L - 1; l > 0; --l) {
         GemmArgs d = args0();  // G_{l-1} = (G_l W_l) * GELU'(z_{l-1}): W_l read as its transpose
-        d.A = gl;
+        d.A = h->g[l];
         d.B = h->pbT + h->w_off[l];
         d.M = B;
         d.N = h->dims[l];
@@ -571,27 +832,66 @@ int backward(pe_mlp* h, int B, int* launches)
         d.lda = h->dims[l + 1];
         d.ldb = h->dims[l + 1];
         d.Z = h->z[l - 1];
-        d.Aout = h->g[(l - 1) & 1];
-        PE_TRY(tc_gemm<kEpiDgrad>(h, d, h->gT[(l - 1) & 1], s, nullptr));
+        d.Aout = h->g[l - 1];
+        PE_TRY(tc_gemm<kEpiDgrad>(h, d, s));
         ++*launches;
     }
+    WgradArgs w;
+    memset(&w, 0, sizeof(w));
+    w.L = L;
+    w.B = B;
+    int blk = 0;
+    for (int l = 0; l < L; ++l) {
+        w.M[l] = h->dims[l + 1];
+        w.N[l] = h->dims[l];
+        w.G[l] = h->g[l];
+        w.dW[l] = h->grad + h->w_off[l];
+        w.db[l] = h->grad + h->b_off[l];
+        w.tile0[l] = blk;
+        blk += (w.N[l] / 64) * ((w.M[l] + tc::kBM - 1) / tc::kBM);
+        PE_TRY(tc_operand_map(&w.a[l], h->g[l], B, w.M[l], w.M[l], 64));
+        PE_TRY(tc_operand_map(&w.b[l], l ? h->a[l - 1] : h->xz, B, w.N[l], w.N[l], 64));
+    }
+    w.tile0[L] = blk;
+    for (int l = 0; l < L; ++l) {
+        w.bias0[l] = blk;
+        blk += w.M[l] / 64;
+    }
+    w.bias0[L] = blk;
+    w.loss_part = h->loss_part;
+    w.nloss = loss_tiles(Dout, B);
+    w.loss_scale = 1.0f / ((float)B * (float)Dout);
+    w.loss = h->loss;
+    w.adam = adam ? 1 : 0;
+    w.step = h->step;
+    w.corr = h->corr;
+    w.b1 = b1;
+    w.b2 = b2;
+    PE_TRY(launch_dependent(k_mlp_wgrad, dim3(blk + 1), tc::kThreads, tc::TileCfg<64>::kSmemBytes, s, w, h->status));
+    ++*launches;
     return PE_OK;
 }
 
-int grad_pass(pe_mlp* h, const float* X, const float* Y, int64_t npairs, const int32_t* rows, const int32_t* shifts,
-              int B, int P, int* launches)
+// Gradients of the batch rows[0..B) (B pairs from row 0 when null), or, with draw, of the batch of
+// the current step of the sequence of seed.
+int grad_pass(pe_mlp* h, const float* X, const float* Y, int64_t npairs, const int32_t* rows, bool draw, uint64_t seed,
+              int B, int P, double b1, double b2, int* launches)
 {
-    cudaStream_t s = h->stream;
-    const int D = h->dims[0], Dout = h->dims[h->L];
-    dim3 pg((std::max(D, Dout) + 255) / 256, B);
-    k_prep<float><<<pg, 256, 0, s>>>(X, Y, B, D, Dout, rows, shifts, P, h->norm, h->norm + h->dmax,
-                                     h->norm + 2 * h->dmax, h->norm + 3 * h->dmax, h->xz, h->xzT, h->ldT, h->tz);
+    PE_TRY(launch_dependent(k_prep<float>, dim3(B), 128, 0, h->stream, X, Y, B, h->dims[0], h->dims[h->L], rows,
+                            draw ? h->step : nullptr, seed, npairs, P, h->norm, h->norm + h->dmax,
+                            h->norm + 2 * h->dmax, h->norm + 3 * h->dmax, h->xz, h->tz));
     ++*launches;
     PE_TRY(forward(h, B, 1, nullptr, nullptr, launches));
-    const int nblk = loss_tiles(Dout, B);
-    k_loss_final<<<1, 256, 0, s>>>(h->loss_part, nblk, h->loss, 1.0f / ((float)B * (float)Dout));
-    ++*launches;
-    return backward(h, B, launches);
+    return backward(h, B, draw, b1, b2, launches);
+}
+
+int adam_update(pe_mlp* h, float lr, double b1, double b2, float eps)
+{
+    int blk = 0;
+    for (int l = 0; l < h->L; ++l)
+        blk += (h->dims[l] / 64) * (h->dims[l + 1] / 64) + (h->dims[l + 1] + 255) / 256;
+    return launch_dependent(k_adam, dim3(blk), 256, 0, h->stream, h->p, h->pb, h->pbT, h->wt, h->grad, h->am, h->av,
+                            h->corr, lr, b1, b2, eps);
 }
 
 }  // namespace
@@ -613,7 +913,7 @@ extern "C" PE_API int pe_mlp_layout_for(int32_t nlayers, const int32_t* dims, in
     out->bytes[PE_MLP_ADAM_V] = 4 * (size_t)np;
     out->bytes[PE_MLP_NORM] = 4 * 4 * (size_t)dmax + 8 * 2 * (size_t)dmax + 8 * (size_t)kNormBlocks * dmax + 256 +
                               4 * (size_t)kLossSlots;
-    out->bytes[PE_MLP_WORK] = plan_work(nlayers, dims, max_batch, dmax).total;
+    out->bytes[PE_MLP_WORK] = plan_work(nlayers, dims, max_batch).total;
     size_t off = 0;
     for (int b = 0; b < PE_MLP_NBUF; ++b) {
         out->offset[b] = off;
@@ -673,25 +973,17 @@ extern "C" PE_API int pe_mlp_create(int32_t nlayers, const int32_t* dims, int32_
     h->step = (int64_t*)nb;
     h->loss = (float*)(nb + 8);
     h->status = (uint32_t*)(nb + 16);
+    h->corr = (float*)(nb + 24);
     h->loss_part = (float*)(nb + 256);
-    const WorkPlan w = plan_work(nlayers, dims, max_batch, h->dmax);
+    const WorkPlan w = plan_work(nlayers, dims, max_batch);
     char* wb = h->arena + lay.offset[PE_MLP_WORK];
-    h->rows = (int32_t*)(wb + w.rows);
-    h->shifts = (int32_t*)(wb + w.shifts);
     h->xz = (__nv_bfloat16*)(wb + w.xz);
     for (int l = 0; l + 1 < nlayers; ++l) {
         h->z[l] = (float*)(wb + w.z[l]);
         h->a[l] = (__nv_bfloat16*)(wb + w.a[l]);
     }
-    h->y = (float*)(wb + w.y);
     h->tz = (float*)(wb + w.tz);
-    h->g[0] = (__nv_bfloat16*)(wb + w.g0);
-    h->g[1] = (__nv_bfloat16*)(wb + w.g1);
-    h->ldT = ld_transposed(max_batch);
-    h->xzT = (__nv_bfloat16*)(wb + w.xzT);
-    for (int l = 0; l + 1 < nlayers; ++l) h->aT[l] = (__nv_bfloat16*)(wb + w.aT[l]);
-    h->gT[0] = (__nv_bfloat16*)(wb + w.gT0);
-    h->gT[1] = (__nv_bfloat16*)(wb + w.gT1);
+    for (int l = 0; l < nlayers; ++l) h->g[l] = (__nv_bfloat16*)(wb + w.g[l]);
     *out = h;
     return PE_OK;
 }
@@ -751,13 +1043,16 @@ extern "C" PE_API int pe_mlp_forward(pe_mlp* h, const void* x, int32_t x_is_f64,
     if (!h || !x || !y || B < 1 || B > h->max_batch) return PE_EINVAL;
     cudaStream_t s = h->stream;
     const int D = h->dims[0];
-    dim3 pg((D + 255) / 256, B);
+    const int32_t* no_rows = nullptr;
+    const int64_t* no_step = nullptr;
+    const float* no_f = nullptr;
+    float* no_t = nullptr;
     if (x_is_f64)
-        k_prep<double><<<pg, 256, 0, s>>>((const double*)x, nullptr, B, D, 0, nullptr, nullptr, 0, h->norm,
-                                          h->norm + h->dmax, nullptr, nullptr, h->xz, nullptr, h->ldT, nullptr);
+        PE_TRY(launch_dependent(k_prep<double>, dim3(B), 128, 0, s, (const double*)x, no_f, B, D, 0, no_rows, no_step,
+                                uint64_t(0), int64_t(0), 0, h->norm, h->norm + h->dmax, no_f, no_f, h->xz, no_t));
     else
-        k_prep<float><<<pg, 256, 0, s>>>((const float*)x, nullptr, B, D, 0, nullptr, nullptr, 0, h->norm,
-                                         h->norm + h->dmax, nullptr, nullptr, h->xz, nullptr, h->ldT, nullptr);
+        PE_TRY(launch_dependent(k_prep<float>, dim3(B), 128, 0, s, (const float*)x, no_f, B, D, 0, no_rows, no_step,
+                                uint64_t(0), int64_t(0), 0, h->norm, h->norm + h->dmax, no_f, no_f, h->xz, no_t));
     int launches = 1;
     PE_TRY(forward(h, B, 0, y_is_f64 ? nullptr : (float*)y, y_is_f64 ? (double*)y : nullptr, &launches));
     return launch_status(launches);
@@ -769,7 +1064,7 @@ extern "C" PE_API int pe_mlp_grad(pe_mlp* h, const float* X, const float* Y, int
     if (!h || !X || !Y || B < 32 || B % 32 || B > h->max_batch || (!rows && npairs < B)) return PE_EINVAL;
     if (loss_tiles(h->dims[h->L], B) > kLossSlots) return PE_EINVAL;
     int launches = 0;
-    PE_TRY(grad_pass(h, X, Y, npairs, rows, nullptr, B, 0, &launches));
+    PE_TRY(grad_pass(h, X, Y, npairs, rows, false, 0, B, 0, 0.0, 0.0, &launches));
     if (loss && cudaMemcpyAsync(loss, h->loss, 4, cudaMemcpyDeviceToDevice, h->stream) != cudaSuccess) return PE_ECUDA;
     return launch_status(launches);
 }
@@ -779,9 +1074,8 @@ extern "C" PE_API int pe_mlp_adam(pe_mlp* h, double lr, double beta1, double bet
     if (!h || !(lr >= 0.0) || !(beta1 >= 0.0 && beta1 < 1.0) || !(beta2 >= 0.0 && beta2 < 1.0) || !(eps > 0.0))
         return PE_EINVAL;
     cudaStream_t s = h->stream;
-    k_adam<<<2 * sm_count(), 256, 0, s>>>(h->p, h->pb, h->pbT, h->wt, h->grad, h->am, h->av, h->nparams, h->step,
-                                          (float)lr, beta1, beta2, (float)eps);
-    k_step_advance<<<1, 32, 0, s>>>(h->step);
+    k_adam_begin<<<1, 32, 0, s>>>(h->step, h->corr, beta1, beta2);
+    PE_TRY(adam_update(h, (float)lr, beta1, beta2, (float)eps));
     return launch_status(2);
 }
 
@@ -795,15 +1089,12 @@ extern "C" PE_API int pe_mlp_train(pe_mlp* h, const float* X, const float* Y, in
     if (shift_period < 0 || (shift_period > 0 && (D % shift_period || Dout % shift_period))) return PE_EINVAL;
     if (loss_tiles(Dout, B) > kLossSlots) return PE_EINVAL;
     cudaStream_t s = h->stream;
-    const int nsm = sm_count();  // cached before any capture
-    int launches = 0;
+    (void)sm_count();  // cached before any capture
+    int launches = 0, rc = PE_OK;
     auto one_step = [&]() {
-        k_sample_rows<<<(B + 255) / 256, 256, 0, s>>>(seed, h->step, B, npairs, shift_period, h->rows, h->shifts);
-        grad_pass(h, X, Y, npairs, h->rows, h->shifts, B, shift_period, &launches);
-        k_adam<<<2 * nsm, 256, 0, s>>>(h->p, h->pb, h->pbT, h->wt, h->grad, h->am, h->av, h->nparams, h->step, lr,
-                                       0.9, 0.999, 1e-8f);
-        k_step_advance<<<1, 32, 0, s>>>(h->step);
-        launches += 3;
+        if (rc == PE_OK) rc = grad_pass(h, X, Y, npairs, nullptr, true, seed, B, shift_period, 0.9, 0.999, &launches);
+        if (rc == PE_OK) rc = adam_update(h, lr, 0.9, 0.999, 1e-8f);
+        ++launches;
     };
     // One step captured as a graph and replayed (the step counter on the device advances the
     // sampling and the bias correction); on the legacy default stream the steps run eagerly.
@@ -812,12 +1103,13 @@ extern "C" PE_API int pe_mlp_train(pe_mlp* h, const float* X, const float* Y, in
     bool captured = false;
     if (s != nullptr && nsteps > 1 && cudaStreamBeginCapture(s, cudaStreamCaptureModeThreadLocal) == cudaSuccess) {
         one_step();
-        if (cudaStreamEndCapture(s, &graph) == cudaSuccess && graph &&
+        if (cudaStreamEndCapture(s, &graph) == cudaSuccess && graph && rc == PE_OK &&
             cudaGraphInstantiate(&exec, graph, 0) == cudaSuccess)
             captured = true;
         else
             cudaGetLastError();
     }
+    rc = PE_OK;
     const int per_step = launches;
     if (captured) {
         for (int i = 0; i < nsteps; ++i)
@@ -832,7 +1124,8 @@ extern "C" PE_API int pe_mlp_train(pe_mlp* h, const float* X, const float* Y, in
     } else {
         if (graph) cudaGraphDestroy(graph);
         launches = 0;
-        for (int i = 0; i < nsteps; ++i) one_step();
+        for (int i = 0; i < nsteps && rc == PE_OK; ++i) one_step();
+        if (rc != PE_OK) return rc;
         if (cudaGetLastError() != cudaSuccess) return PE_ECUDA;
         note_launches(launches);
     }

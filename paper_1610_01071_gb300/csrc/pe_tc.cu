@@ -62,7 +62,7 @@ int launch_plain(const CUtensorMap& ma, const CUtensorMap& mb, int M, int N, int
     const void* k = (const void*)tc::k_tc_gemm<BN, EpiStoreF32>;
     if (ensure_smem(k, tc::TileCfg<BN>::kSmemBytes) != PE_OK) return PE_ECUDA;
     dim3 grid(N / BN, (M + tc::kBM - 1) / tc::kBM);
-    tc::k_tc_gemm<BN, EpiStoreF32><<<grid, tc::kThreads, tc::TileCfg<BN>::kSmemBytes, s>>>(ma, mb, M, K, epi, status);
+    tc::k_tc_gemm<BN, EpiStoreF32><<<grid, tc::kThreads, tc::TileCfg<BN>::kSmemBytes, s>>>(ma, mb, K, epi, status);
     return launch_status();
 }
 }  // namespace

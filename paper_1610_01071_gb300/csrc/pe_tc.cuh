@@ -1,13 +1,16 @@
 // Blackwell tensor-core GEMM building blocks (sm_100 family, compiled for sm_103a): mbarriers,
 // TMA tile loads with the 128-byte swizzle, tcgen05.mma with the accumulator in tensor memory
-// (TMEM), and a single-CTA kernel C[M][N] = A[M][K] B[N][K]^T for BF16 operands stored with K
-// contiguous, FP32 accumulation, and an epilogue functor applied to each row of the tile.
+// (TMEM), and one tile of C[M][N] = sum_k A(m, k) B(n, k) by one block, FP32 accumulation, with an
+// epilogue functor applied to each row of the tile. Both operands are BF16, stored either with K
+// contiguous (A[M][K], B[N][K]) or with M and N contiguous (A[K][M], B[K][N]).
 //
 // Tile: 128 rows (the MMA's M) x BN columns (64 or 128) x 64 K per stage (one 128-byte swizzle
 // row of BF16), four stages. One thread issues the TMA loads and the MMAs (kind::f16, K = 16
 // per instruction, four per stage); a stage is reloaded once the MMAs that read it have
-// signalled its empty barrier (tcgen05.commit). After the last MMA the four warps read their
-// 32 TMEM lanes (tile rows) 32 columns at a time (tcgen05.ld 32x32b.x32).
+// signalled its empty barrier (tcgen05.commit). After the last MMA the eight warps read the
+// accumulator 32 columns at a time (tcgen05.ld 32x32b.x32): warp w the TMEM lanes (tile rows) of
+// its quarter w mod 4, the left half of the columns for w < 4 and the right half for w >= 4. With
+// four warps the epilogue (its transcendental functions and stores) took longer than the products.
 //
 // Every wait on an mbarrier is bounded by a clock budget (about one second); on expiry the
 // kernel sets PE_FLAG_TIMEOUT in the status word, skips the remaining MMAs and the epilogue,
@@ -26,7 +29,7 @@ namespace tc {
 constexpr int kBM = 128;       // tile rows = MMA M
 constexpr int kBK = 64;        // K per stage: 64 BF16 = one 128-byte swizzle row
 constexpr int kStages = 4;
-constexpr int kThreads = 128;  // four warps: one per 32 TMEM lanes in the epilogue
+constexpr int kThreads = 256;  // eight warps: two per 32 TMEM lanes in the epilogue
 constexpr long long kWaitBudget = 2000000000LL;  // clock cycles (about one second)
 
 template <int BN>
@@ -112,10 +115,42 @@ __device__ __forceinline__ uint64_t sw128_desc(uint32_t addr)
            ((uint64_t)1 << 46) | ((uint64_t)2 << 61);
 }
 
-// Instruction descriptor of kind::f16: FP32 accumulator, BF16 A and B, both K-major, M x N.
-__host__ __device__ constexpr uint32_t idesc_bf16(int M, int N)
+// The same for an operand tile with M (or N) contiguous: slabs of 64 elements (128 bytes) along M,
+// each 64 K rows of 128 bytes (8 KB, the leading byte offset), groups of 8 K rows 1024 bytes apart.
+__device__ __forceinline__ uint64_t sw128_desc_mn(uint32_t addr)
 {
-    return (1u << 4) | (1u << 7) | (1u << 10) | ((uint32_t)(N >> 3) << 17) | ((uint32_t)(M >> 4) << 24);
+    return (uint64_t)((addr >> 4) & 0x3FFFu) | ((uint64_t)(8192 >> 4) << 16) | ((uint64_t)(1024 >> 4) << 32) |
+           ((uint64_t)1 << 46) | ((uint64_t)2 << 61);
+}
+
+// Instruction descriptor of kind::f16: FP32 accumulator, BF16 A and B, M x N; both operands K-major,
+// or (mn) both with M / N contiguous.
+__host__ __device__ constexpr uint32_t idesc_bf16(int M, int N, bool mn = false)
+{
+    return (1u << 4) | (1u << 7) | (1u << 10) | (mn ? (1u << 15) | (1u << 16) : 0u) | ((uint32_t)(N >> 3) << 17) |
+           ((uint32_t)(M >> 4) << 24);
+}
+
+// Programmatic dependent launch: waits until the kernels this one depends on have completed and
+// their writes are visible (returns at once in a launch without the attribute), and lets the
+// dependent launch start its prologue.
+__device__ __forceinline__ void grid_wait() { asm volatile("griddepcontrol.wait;" ::: "memory"); }
+__device__ __forceinline__ void grid_release() { asm volatile("griddepcontrol.launch_dependents;" ::: "memory"); }
+
+// 32-byte global accesses (one full sector per lane): rows are written one lane each, so narrower
+// ones would touch every sector several times. 32-byte aligned addresses.
+__device__ __forceinline__ void st_global32(void* p, const uint32_t* r)
+{
+    asm volatile("st.global.v8.b32 [%0], {%1, %2, %3, %4, %5, %6, %7, %8};" ::"l"(p), "r"(r[0]), "r"(r[1]), "r"(r[2]),
+                 "r"(r[3]), "r"(r[4]), "r"(r[5]), "r"(r[6]), "r"(r[7])
+                 : "memory");
+}
+__device__ __forceinline__ void ld_global32(const void* p, uint32_t* r)
+{
+    asm volatile("ld.global.v8.b32 {%0, %1, %2, %3, %4, %5, %6, %7}, [%8];"
+                 : "=r"(r[0]), "=r"(r[1]), "=r"(r[2]), "=r"(r[3]), "=r"(r[4]), "=r"(r[5]), "=r"(r[6]), "=r"(r[7])
+                 : "l"(p)
+                 : "memory");
 }
 
 __device__ __forceinline__ void umma_bf16(uint32_t tmem_d, uint64_t adesc, uint64_t bdesc, uint32_t idesc,
@@ -164,53 +199,67 @@ __device__ __forceinline__ void tmem_ld32(uint32_t taddr, float* v)
     for (int j = 0; j < 32; ++j) v[j] = __uint_as_float(r[j]);
 }
 
-// C tile (blockIdx.y, blockIdx.x) of A[M][K] B[N][K]^T; ta / tb: tensor maps of A (dims {K, M},
-// box {64, 128}) and B (dims {K, N}, box {64, BN}), 128-byte swizzle, zero fill beyond the
-// extents (ragged M and K). epi(row, col0, v) receives 32 columns col0.. of one row (the row
-// may be >= M: the functor checks); every thread then calls epi.finish() (block-wide
-// reductions of the epilogue). N % BN == 0.
-template <int BN, class Epi>
-__global__ void __launch_bounds__(kThreads, 1)
-    k_tc_gemm(const __grid_constant__ CUtensorMap ta, const __grid_constant__ CUtensorMap tb, int M, int K, Epi epi,
-              uint32_t* status)
+// Barriers and the TMEM address of a block's tile, after the operand stages in shared memory.
+struct TileShared {
+    uint64_t* full;
+    uint64_t* empty;
+    uint64_t* done;
+    uint32_t* tmem_slot;
+};
+
+// The C tile at (m0, n0) over K: ta / tb are the tensor maps of A and B with 128-byte swizzle and
+// zero fill beyond the extents (ragged M and K): K-major dims {K, M} box {64, 128} and dims {K, N}
+// box {64, BN}; MN: dims {M, K} and {N, K}, boxes {64, 64}. epi(row, col0, v) receives 32 columns
+// col0.. of one row (the row may be >= M: the functor checks); every thread then calls
+// epi.finish() (block-wide reductions of the epilogue). All threads of the block call it.
+template <int BN, bool MN, class Epi>
+__device__ __forceinline__ void gemm_tile(const CUtensorMap* ta, const CUtensorMap* tb, int m0, int n0, int K, Epi& epi,
+                                          uint32_t* status)
 {
     using Cfg = TileCfg<BN>;
     extern __shared__ uint8_t smem_raw[];
     uint8_t* smem = reinterpret_cast<uint8_t*>((reinterpret_cast<uintptr_t>(smem_raw) + 1023) & ~uintptr_t(1023));
-    uint64_t* full = reinterpret_cast<uint64_t*>(smem + kStages * Cfg::kStageBytes);
-    uint64_t* empty = full + kStages;
-    uint64_t* done = empty + kStages;
-    uint32_t* tmem_slot = reinterpret_cast<uint32_t*>(done + 1);
+    TileShared b;
+    b.full = reinterpret_cast<uint64_t*>(smem + kStages * Cfg::kStageBytes);
+    b.empty = b.full + kStages;
+    b.done = b.empty + kStages;
+    b.tmem_slot = reinterpret_cast<uint32_t*>(b.done + 1);
     __shared__ int s_fail;
 
     const int tid = threadIdx.x, warp = tid >> 5, lane = tid & 31;
-    const int m0 = blockIdx.y * kBM, n0 = blockIdx.x * BN;
     const int ktiles = (K + kBK - 1) / kBK;
-    constexpr uint32_t idesc = idesc_bf16(kBM, BN);
-    (void)M;
+    constexpr uint32_t idesc = idesc_bf16(kBM, BN, MN);
 
     if (tid == 0) {
         for (int s = 0; s < kStages; ++s) {
-            mbar_init(&full[s], 1);
-            mbar_init(&empty[s], 1);
+            mbar_init(&b.full[s], 1);
+            mbar_init(&b.empty[s], 1);
         }
-        mbar_init(done, 1);
+        mbar_init(b.done, 1);
         fence_mbar_init();
         s_fail = 0;
     }
-    if (warp == 0) tmem_alloc(tmem_slot, BN);
+    if (warp == 0) tmem_alloc(b.tmem_slot, BN);
     tc_fence_before();
     __syncthreads();
     tc_fence_after();
-    const uint32_t tmem = *tmem_slot;
+    const uint32_t tmem = *b.tmem_slot;
+    grid_release();
+    grid_wait();
 
     if (tid == 0) {
         auto load = [&](int t) {
             const int s = t % kStages;
             uint8_t* a = smem + s * Cfg::kStageBytes;
-            mbar_expect_tx(&full[s], Cfg::kStageBytes);
-            tma_load_2d(a, &ta, &full[s], t * kBK, m0);
-            tma_load_2d(a + Cfg::kABytes, &tb, &full[s], t * kBK, n0);
+            mbar_expect_tx(&b.full[s], Cfg::kStageBytes);
+            if (MN) {
+                for (int q = 0; q < kBM; q += 64) tma_load_2d(a + q * kBK * 2, ta, &b.full[s], m0 + q, t * kBK);
+                for (int q = 0; q < BN; q += 64)
+                    tma_load_2d(a + Cfg::kABytes + q * kBK * 2, tb, &b.full[s], n0 + q, t * kBK);
+            } else {
+                tma_load_2d(a, ta, &b.full[s], t * kBK, m0);
+                tma_load_2d(a + Cfg::kABytes, tb, &b.full[s], t * kBK, n0);
+            }
         };
         const int pro = ktiles < kStages ? ktiles : kStages;
         for (int t = 0; t < pro; ++t) load(t);
@@ -218,7 +267,7 @@ __global__ void __launch_bounds__(kThreads, 1)
         bool ok = true;
         for (int kt = 0; kt < ktiles; ++kt) {
             const int s = kt % kStages;
-            if (!mbar_wait(&full[s], (uint32_t)((kt / kStages) & 1))) {
+            if (!mbar_wait(&b.full[s], (uint32_t)((kt / kStages) & 1))) {
                 ok = false;
                 break;
             }
@@ -226,13 +275,17 @@ __global__ void __launch_bounds__(kThreads, 1)
             tc_fence_after();
             const uint32_t a0 = saddr(smem + s * Cfg::kStageBytes), b0 = a0 + Cfg::kABytes;
 #pragma unroll
-            for (int k = 0; k < kBK / 16; ++k)  // K = 16 per MMA: 32 bytes along the swizzled row
-                umma_bf16(tmem, sw128_desc(a0 + 32 * k), sw128_desc(b0 + 32 * k), idesc, (kt | k) ? 1u : 0u);
-            umma_commit(&empty[s]);
+            for (int k = 0; k < kBK / 16; ++k) {
+                // K = 16 per MMA: 32 bytes along the swizzled row (K-major), 16 rows of 128 bytes (MN)
+                const uint64_t da = MN ? sw128_desc_mn(a0 + 2048 * k) : sw128_desc(a0 + 32 * k);
+                const uint64_t db = MN ? sw128_desc_mn(b0 + 2048 * k) : sw128_desc(b0 + 32 * k);
+                umma_bf16(tmem, da, db, idesc, (kt | k) ? 1u : 0u);
+            }
+            umma_commit(&b.empty[s]);
             // refill the stage of the previous tile once its MMAs are done (this tile's MMAs are queued)
             const int t = kt - 1 + kStages;
             if (kt >= 1 && t < ktiles) {
-                if (!mbar_wait(&empty[(kt - 1) % kStages], (uint32_t)(((kt - 1) / kStages) & 1))) {
+                if (!mbar_wait(&b.empty[(kt - 1) % kStages], (uint32_t)(((kt - 1) / kStages) & 1))) {
                     ok = false;
                     break;
                 }
@@ -240,33 +293,43 @@ __global__ void __launch_bounds__(kThreads, 1)
                 ++issued;
             }
         }
-        umma_commit(done);
+        umma_commit(b.done);
         if (!ok) {
             s_fail = 1;
             // let the tile loads still in flight land (bounded) before the block may exit
-            for (int t = consumed; t < issued; ++t) mbar_wait(&full[t % kStages], (uint32_t)((t / kStages) & 1));
+            for (int t = consumed; t < issued; ++t) mbar_wait(&b.full[t % kStages], (uint32_t)((t / kStages) & 1));
         }
     }
     __syncthreads();
-    bool ok = mbar_wait(done, 0u) && !s_fail;
+    bool ok = mbar_wait(b.done, 0u) && !s_fail;
     ok = __all_sync(0xFFFFFFFFu, ok);
     if (!ok && lane == 0) atomicOr(status, PE_FLAG_TIMEOUT);
     tc_fence_after();
-    Epi e = epi;
     if (ok) {
-        const int row = m0 + warp * 32 + lane;
-        const uint32_t t_row = tmem + ((uint32_t)(warp * 32) << 16);
+        const int quarter = warp & 3, half = warp >> 2;
+        const int row = m0 + quarter * 32 + lane;
+        const uint32_t t_row = tmem + ((uint32_t)(quarter * 32) << 16);
 #pragma unroll 1
-        for (int c = 0; c < BN; c += 32) {
+        for (int c = half * (BN / 2); c < (half + 1) * (BN / 2); c += 32) {
             float v[32];
             tmem_ld32(t_row + (uint32_t)c, v);
-            e(row, n0 + c, v);
+            epi(row, n0 + c, v);
         }
     }
-    e.finish();
+    epi.finish();
     tc_fence_before();
     __syncthreads();
     if (warp == 0) tmem_dealloc(tmem, BN);
+}
+
+// One tile per block, C tile (blockIdx.y, blockIdx.x), K-major operands. N % BN == 0.
+template <int BN, class Epi>
+__global__ void __launch_bounds__(kThreads, 1)
+    k_tc_gemm(const __grid_constant__ CUtensorMap ta, const __grid_constant__ CUtensorMap tb, int K, Epi epi,
+              uint32_t* status)
+{
+    Epi e = epi;
+    gemm_tile<BN, false>(&ta, &tb, (int)blockIdx.y * kBM, (int)blockIdx.x * BN, K, e, status);
 }
 
 }  // namespace tc

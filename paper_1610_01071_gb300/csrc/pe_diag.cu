@@ -3,12 +3,21 @@
 // fine step, the particle-level counterpart of the macroscopic condition Eq. (CFL)) and the
 // coarse-variable error measure of Section 4.1.1.
 //
-// Two launches: a particle pass (grid-stride, fixed grid for a given n, so the
-// floating-point sums are reproduced bit for bit) writes one partial per block; a
-// single 1024-thread block adds the partials in a fixed tree and the grid energies.
+// Two launches: a particle pass (grid-stride, fixed grid for a given n and ncell, so the
+// floating-point sums are reproduced bit for bit) writes one partial per block, the nodal energies
+// among them; a single block adds the partials in a fixed order.
+//
+// The FP64 pipe bounds a direct form (seven FP64 instructions per particle at 1.7 lanes per
+// cycle and SM: 128 us for 2^23 particles, 16 % of the memory bandwidth). The sums run in FP32
+// instead, as unevaluated sums of three floats with error-free additions and products (Knuth's
+// and Dekker's two-sum and two-product): about 70 bits, so that a sum is rounded once, at its
+// conversion to FP64; FP64 takes only the conversion of the block sums: 42 us for 2^23 particles
+// (128 before), and the final pass 6 us (35 with the nodal exponentials in its one block).
 #include <cuda_runtime.h>
 #include <math.h>
 #include <stdint.h>
+
+#include <algorithm>
 
 #include "pe_common.cuh"
 #include "pe_internal.h"
@@ -18,16 +27,17 @@ namespace pe {
 namespace {
 
 constexpr int kDiagThreads = 256;
-constexpr int kDiagMaxBlocks = 1024;
+constexpr int kDiagMaxBlocks = 608;  // four per SM: enough loads in flight to stream the particles
 constexpr int kFinalThreads = 1024;
 
 struct DiagScratch {
-    long long charge[kDiagMaxBlocks];
     long long wq[kDiagMaxBlocks];
     long long invalid[kDiagMaxBlocks];
     double mom[kDiagMaxBlocks];
     double kin[kDiagMaxBlocks];
     double wsum[kDiagMaxBlocks];
+    double fe[kDiagMaxBlocks];
+    double ee[kDiagMaxBlocks];
     float vmax[kDiagMaxBlocks];
 };
 static_assert(sizeof(DiagScratch) <= PE_MOMENTS_SCRATCH_BYTES, "scratch size");
@@ -44,76 +54,198 @@ __device__ __forceinline__ float warp_maxf(float v)
     return v;
 }
 
-// Particle pass. Vbar = v + (kick - 1/2) qm dt E(X) is the integer-time velocity; a
-// particle with a cell outside [0, ncell), a non-finite offset or velocity, or an offset
-// outside [0, 1] is counted as invalid, sets PE_FLAG_RANGE and is left out of the sums.
-__global__ void __launch_bounds__(kDiagThreads) k_moments_particles(
-    const int32_t* __restrict__ cell, const float* __restrict__ theta, const float* __restrict__ v,
-    const float* __restrict__ w, int64_t n, const float* __restrict__ Ef, int ncell, float hk, float wscale,
-    DiagScratch* __restrict__ out, uint32_t* status)
+// a + b = s + e exactly (Knuth).
+__device__ __forceinline__ float two_sum(float a, float b, float& e)
 {
-    long long q = 0, bad = 0, qw = 0;
-    double mom = 0.0, kin = 0.0, ws = 0.0;
-    float vmax = 0.0f;
-    const int64_t stride = (int64_t)gridDim.x * blockDim.x;
-    for (int64_t i = (int64_t)blockIdx.x * blockDim.x + threadIdx.x; i < n; i += stride) {
-        const int c = cell[i];
-        const float th = theta[i], vv = v[i], ww = w[i];
-        if ((unsigned)c >= (unsigned)ncell || !isfinite(vv) || !isfinite(ww) || !(th >= 0.0f && th <= 1.0f)) {
-            ++bad;
-            continue;
-        }
-        const int c1 = (c + 1 == ncell) ? 0 : c + 1;
-        const float Ec = __ldg(Ef + c), Ec1 = __ldg(Ef + c1);
-        const float vb = fmaf(hk, fmaf(th, Ec1 - Ec, Ec), vv);
-        const long long wqi = (long long)__float2int_rn(ww * wscale);
-        q += wqi * (long long)kThetaOne;
-        qw += wqi;
-        const double wd = (double)ww, vd = (double)vb;
-        mom += wd * vd;
-        kin += 0.5 * wd * vd * vd;
-        ws += wd;
-        vmax = fmaxf(vmax, fabsf(vb));
+    const float s = __fadd_rn(a, b), bb = __fsub_rn(s, a);
+    e = __fadd_rn(__fsub_rn(a, __fsub_rn(s, bb)), __fsub_rn(b, bb));
+    return s;
+}
+
+// Sum kept as h + l + t; only the additions to t round (2^-72 of the terms).
+struct Sum3 {
+    float h, l, t;
+    __device__ __forceinline__ void reset() { h = l = t = 0.0f; }
+    __device__ __forceinline__ void add_low(float x)  // x of the size of an error of h
+    {
+        float f;
+        l = two_sum(l, x, f);
+        t = __fadd_rn(t, f);
     }
-    __shared__ long long sq[kDiagThreads / 32], sb[kDiagThreads / 32], sqw[kDiagThreads / 32];
-    __shared__ double sm[kDiagThreads / 32], sk[kDiagThreads / 32], sw[kDiagThreads / 32];
-    __shared__ float sv[kDiagThreads / 32];
+    __device__ __forceinline__ void add(float x)
+    {
+        float e;
+        h = two_sum(h, x, e);
+        add_low(e);
+    }
+    __device__ __forceinline__ void add(const Sum3& o)
+    {
+        add(o.h);
+        add_low(o.l);
+        t = __fadd_rn(t, o.t);
+    }
+    __device__ __forceinline__ void warp_fold()
+    {
+        for (int o = 16; o > 0; o >>= 1) {
+            Sum3 x;
+            x.h = __shfl_xor_sync(0xffffffffu, h, o);
+            x.l = __shfl_xor_sync(0xffffffffu, l, o);
+            x.t = __shfl_xor_sync(0xffffffffu, t, o);
+            add(x);
+        }
+    }
+    __device__ __forceinline__ double value() const { return (double)h + ((double)l + (double)t); }
+};
+
+struct MomentSums {
+    Sum3 ws, mom, kin;  // sum w, sum w V, sum w V^2
+    double ws64, mom64, kin64;  // the same of particles whose products leave FP32's range
+    long long wq;
+    int bad;
+    bool wide;  // the FP64 sums were used
+    float vmax;
+};
+
+// One particle. Vbar = v + (kick - 1/2) qm dt E(X) is the integer-time velocity; a particle with a
+// cell outside [0, ncell), a non-finite offset or velocity, or an offset outside [0, 1] is
+// counted as invalid and left out of the sums.
+__device__ __forceinline__ void moment_one(MomentSums& S, int c, float th, float vv, float ww,
+                                           const float* __restrict__ Ef, int ncell, float hk, float wscale)
+{
+    if ((unsigned)c >= (unsigned)ncell || !isfinite(vv) || !isfinite(ww) || !(th >= 0.0f && th <= 1.0f)) {
+        ++S.bad;
+        return;
+    }
+    const int c1 = (c + 1 == ncell) ? 0 : c + 1;
+    const float Ec = __ldg(Ef + c), Ec1 = __ldg(Ef + c1);
+    const float vb = fmaf(hk, fmaf(th, Ec1 - Ec, Ec), vv);
+    S.wq += (long long)__float2int_rn(ww * wscale);
+    S.vmax = fmaxf(S.vmax, fabsf(vb));
+    const float p = __fmul_rn(ww, vb), q = __fmul_rn(p, vb), m = fabsf(q);
+    // products whose error terms FP32 represents (or a zero factor); others in FP64
+    if (fabsf(ww) <= 1.2676506e30f && ((m >= 3.3087225e-24f && m <= 1.2676506e30f) || ww == 0.0f || vb == 0.0f)) {
+        S.ws.add(ww);  // 2^-78 <= m <= 2^100
+        const float e = fmaf(ww, vb, -p);  // w V = p + e
+        S.mom.add(p);
+        S.mom.add_low(e);
+        const float g = __fmul_rn(e, vb);
+        S.kin.add(q);                      // w V^2 = q + (p V - q) + e V
+        S.kin.add_low(fmaf(p, vb, -q));
+        S.kin.add_low(g);
+        S.kin.t = __fadd_rn(S.kin.t, fmaf(e, vb, -g));
+    } else {
+        const double wd = (double)ww, vd = (double)vb;
+        S.wide = true;
+        S.ws64 += wd;
+        S.mom64 += wd * vd;
+        S.kin64 += wd * vd * vd;
+    }
+}
+
+template <bool VEC>
+__global__ void __launch_bounds__(kDiagThreads, 4) k_moments_particles(
+    const int32_t* __restrict__ cell, const float* __restrict__ theta, const float* __restrict__ v,
+    const float* __restrict__ w, int64_t n, const float* __restrict__ Ef, const double* __restrict__ phi,
+    const double* __restrict__ E, int ncell, float hk, float wscale, int mode, DiagScratch* __restrict__ out,
+    uint32_t* status)
+{
+    MomentSums S;
+    S.ws.reset();
+    S.mom.reset();
+    S.kin.reset();
+    S.ws64 = S.mom64 = S.kin64 = 0.0;
+    S.wq = 0;
+    S.bad = 0;
+    S.wide = false;
+    S.vmax = 0.0f;
+    const int64_t stride = (int64_t)gridDim.x * blockDim.x, t0 = (int64_t)blockIdx.x * blockDim.x + threadIdx.x;
+    // nodal energies, the nodes spread over the blocks (the exponential is FP64 work)
+    double fe = 0.0, ee = 0.0;
+    for (int64_t j = t0; j < ncell; j += stride) {
+        const double e = E ? E[j] : 0.0;
+        fe += 0.5 * e * e;
+        if (phi) {
+            const double p = phi[j];
+            ee += (mode == PE_POISSON_BOLTZMANN) ? (p * exp(p) - exp(p) + 1.0) : 0.5 * p * p;
+        }
+    }
+    const bool nodes = (int64_t)blockIdx.x * blockDim.x < ncell;  // this block has some
+    const int64_t n4 = VEC ? n >> 2 : 0;
+    if (VEC) {
+        for (int64_t g = t0; g < n4; g += stride) {
+            const int4 c = __ldg(reinterpret_cast<const int4*>(cell) + g);
+            const float4 th = __ldg(reinterpret_cast<const float4*>(theta) + g);
+            const float4 vv = __ldg(reinterpret_cast<const float4*>(v) + g);
+            const float4 ww = __ldg(reinterpret_cast<const float4*>(w) + g);
+            moment_one(S, c.x, th.x, vv.x, ww.x, Ef, ncell, hk, wscale);
+            moment_one(S, c.y, th.y, vv.y, ww.y, Ef, ncell, hk, wscale);
+            moment_one(S, c.z, th.z, vv.z, ww.z, Ef, ncell, hk, wscale);
+            moment_one(S, c.w, th.w, vv.w, ww.w, Ef, ncell, hk, wscale);
+        }
+    }
+    for (int64_t i = 4 * n4 + t0; i < n; i += stride)
+        moment_one(S, cell[i], theta[i], v[i], w[i], Ef, ncell, hk, wscale);
+
+    constexpr int kW = kDiagThreads / 32;
+    __shared__ Sum3 ss[3][kW];
+    __shared__ double s64[5][kW];  // FP64 sums of w, w V and w V^2, field and electron energies
+    __shared__ long long sq[kW];
+    __shared__ int sb[kW];
+    __shared__ float sv[kW];
     const int lane = threadIdx.x & 31, wid = threadIdx.x >> 5;
-    q = warp_sum_i64(q);
-    bad = warp_sum_i64(bad);
-    qw = warp_sum_i64(qw);
-    mom = warp_sum(mom);
-    kin = warp_sum(kin);
-    ws = warp_sum(ws);
-    vmax = warp_maxf(vmax);
+    S.ws.warp_fold();
+    S.mom.warp_fold();
+    S.kin.warp_fold();
+    const long long wq = warp_sum_i64(S.wq);
+    const int bad = __reduce_add_sync(0xffffffffu, S.bad);
+    const float vm = warp_maxf(S.vmax);
+    const bool wide = __any_sync(0xffffffffu, S.wide);
+    const double w64 = wide ? warp_sum(S.ws64) : 0.0, m64 = wide ? warp_sum(S.mom64) : 0.0;
+    const double k64 = wide ? warp_sum(S.kin64) : 0.0;
+    if (nodes) {
+        fe = warp_sum(fe);
+        ee = warp_sum(ee);
+    }
     if (lane == 0) {
-        sq[wid] = q;
+        ss[0][wid] = S.ws;
+        ss[1][wid] = S.mom;
+        ss[2][wid] = S.kin;
+        s64[0][wid] = w64;
+        s64[1][wid] = m64;
+        s64[2][wid] = k64;
+        s64[3][wid] = fe;
+        s64[4][wid] = ee;
+        sq[wid] = wq;
         sb[wid] = bad;
-        sqw[wid] = qw;
-        sm[wid] = mom;
-        sk[wid] = kin;
-        sw[wid] = ws;
-        sv[wid] = vmax;
+        sv[wid] = vm;
     }
     __syncthreads();
-    if (threadIdx.x == 0) {
-        for (int k = 1; k < kDiagThreads / 32; ++k) {
-            q += sq[k];
-            bad += sb[k];
-            qw += sqw[k];
-            mom += sm[k];
-            kin += sk[k];
-            ws += sw[k];
-            vmax = fmaxf(vmax, sv[k]);
+    if (wid == 0) {
+        if (lane < 3) {
+            Sum3 a = ss[lane][0];
+            for (int k = 1; k < kW; ++k) a.add(ss[lane][k]);
+            double x = a.value();
+            for (int k = 0; k < kW; ++k)
+                if (s64[lane][k] != 0.0) x += s64[lane][k];
+            (lane == 0 ? out->wsum : (lane == 1 ? out->mom : out->kin))[blockIdx.x] = x;
+        } else if (lane < 5) {
+            double x = s64[lane][0];
+            if (nodes)
+                for (int k = 1; k < kW; ++k) x += s64[lane][k];
+            (lane == 3 ? out->fe : out->ee)[blockIdx.x] = x;
+        } else if (lane == 5) {
+            long long q = 0, b = 0;
+            float m = 0.0f;
+            for (int k = 0; k < kW; ++k) {
+                q += sq[k];
+                b += sb[k];
+                m = fmaxf(m, sv[k]);
+            }
+            out->wq[blockIdx.x] = q;
+            out->invalid[blockIdx.x] = b;
+            out->vmax[blockIdx.x] = m;
+            if (b) raise_flag(status, PE_FLAG_RANGE);
         }
-        out->charge[blockIdx.x] = q;
-        out->invalid[blockIdx.x] = bad;
-        out->wq[blockIdx.x] = qw;
-        out->mom[blockIdx.x] = mom;
-        out->kin[blockIdx.x] = kin;
-        out->wsum[blockIdx.x] = ws;
-        out->vmax[blockIdx.x] = vmax;
-        if (bad) raise_flag(status, PE_FLAG_RANGE);
     }
 }
 
@@ -132,60 +264,48 @@ __device__ T block_reduce(T x, T* red, Op op)
     return x;  // valid in warp 0
 }
 
-// Final pass: sums of the block partials (fixed order) and of the nodal energies.
-__global__ void __launch_bounds__(kFinalThreads) k_moments_final(
-    const DiagScratch* __restrict__ part, int nblocks, const double* __restrict__ phi, const double* __restrict__ E,
-    int ncell, double dx, double dt, double charge_scale, int mode, pe_moments* out)
+// Final pass, one quantity per warp (each FP64 addition of a warp holds its scheduler's pipe): the
+// block partials in a fixed order.
+__global__ void __launch_bounds__(256) k_moments_final(const DiagScratch* __restrict__ part, int nblocks, double dx,
+                                                       double dt, double charge_scale, pe_moments* out)
 {
-    __shared__ double rd[32];
-    __shared__ long long ri[32];
-    __shared__ float rf[32];
-    const int t = threadIdx.x;
-    const bool have = t < nblocks;
-    long long q = have ? part->charge[t] : 0, bad = have ? part->invalid[t] : 0, qw = have ? part->wq[t] : 0;
-    double mom = have ? part->mom[t] : 0.0, kin = have ? part->kin[t] : 0.0, ws = have ? part->wsum[t] : 0.0;
-    float vmax = have ? part->vmax[t] : 0.0f;
-    double fe = 0.0, ee = 0.0;
-    for (int j = t; j < ncell; j += kFinalThreads) {
-        const double e = E ? E[j] : 0.0;
-        fe += 0.5 * e * e;
-        if (phi) {
-            const double p = phi[j];
-            ee += (mode == PE_POISSON_BOLTZMANN) ? (p * exp(p) - exp(p) + 1.0) : 0.5 * p * p;
-        }
+    __shared__ double sd[5];
+    __shared__ long long si[2];
+    __shared__ float sf;
+    const int lane = threadIdx.x & 31, wid = threadIdx.x >> 5;
+    if (wid < 5) {
+        const double* src = wid == 0 ? part->mom : (wid == 1 ? part->kin : (wid == 2 ? part->wsum : (wid == 3 ? part->fe : part->ee)));
+        double x = 0.0;
+        for (int b = lane; b < nblocks; b += 32) x += src[b];
+        x = warp_sum(x);
+        if (lane == 0) sd[wid] = x;
+    } else if (wid < 7) {
+        const long long* src = wid == 5 ? part->wq : part->invalid;
+        long long x = 0;
+        for (int b = lane; b < nblocks; b += 32) x += src[b];
+        x = warp_sum_i64(x);
+        if (lane == 0) si[wid - 5] = x;
+    } else {
+        float x = 0.0f;
+        for (int b = lane; b < nblocks; b += 32) x = fmaxf(x, part->vmax[b]);
+        x = warp_maxf(x);
+        if (lane == 0) sf = x;
     }
-    auto add_i = [](long long a, long long b) { return a + b; };
-    auto add_d = [](double a, double b) { return a + b; };
-    auto max_f = [](float a, float b) { return fmaxf(a, b); };
-    q = block_reduce(q, ri, add_i);
-    const long long qs = q;
-    bad = block_reduce(bad, ri, add_i);
-    const long long bads = bad;
-    qw = block_reduce(qw, ri, add_i);
-    mom = block_reduce(mom, rd, add_d);
-    const double moms = mom;
-    kin = block_reduce(kin, rd, add_d);
-    const double kins = kin;
-    ws = block_reduce(ws, rd, add_d);
-    const double wss = ws;
-    fe = block_reduce(fe, rd, add_d);
-    const double fes = fe;
-    ee = block_reduce(ee, rd, add_d);
-    vmax = block_reduce(vmax, rf, max_f);
-    if (t == 0) {
+    __syncthreads();
+    if (threadIdx.x == 0) {
         pe_moments m;
-        m.charge_fx = qs;
-        m.invalid = bads;
-        m.charge_wq = qw;
-        m.charge_fixed_point = (double)qs * charge_scale * dx;
-        m.charge = wss * dx;
-        m.momentum = moms * dx;
-        m.kinetic = kins * dx;
-        m.field_energy = fes * dx;
-        m.electron_energy = ee * dx;
+        m.charge_fx = (long long)((unsigned long long)si[0] << 24);  // modulo 2^64
+        m.invalid = si[1];
+        m.charge_wq = si[0];
+        m.charge_fixed_point = (double)m.charge_fx * charge_scale * dx;
+        m.charge = sd[2] * dx;
+        m.momentum = sd[0] * dx;
+        m.kinetic = 0.5 * sd[1] * dx;
+        m.field_energy = sd[3] * dx;
+        m.electron_energy = sd[4] * dx;
         m.total_energy = m.kinetic + m.field_energy + m.electron_energy;
-        m.max_speed = (double)vmax;
-        m.cfl = (double)vmax * dt / dx;
+        m.max_speed = (double)sf;
+        m.cfl = (double)sf * dt / dx;
         *out = m;
     }
 }
@@ -209,10 +329,11 @@ __global__ void __launch_bounds__(kFinalThreads) k_rel_l2(const double* __restri
 
 }  // namespace
 
-int moments_blocks(int64_t n)
+// Blocks of the particle pass: 16 particles per thread, and a thread per node, up to kDiagMaxBlocks.
+static int moments_blocks(int64_t n, int ncell)
 {
     const int64_t per = (int64_t)kDiagThreads * 16;
-    int64_t b = (n + per - 1) / per;
+    int64_t b = std::max((n + per - 1) / per, ((int64_t)ncell + kDiagThreads - 1) / kDiagThreads);
     if (b < 1) b = 1;
     if (b > kDiagMaxBlocks) b = kDiagMaxBlocks;
     return (int)b;
@@ -297,12 +418,14 @@ extern "C" PE_API int pe_compute_moments(const int32_t* cell, const float* theta
     if (mode != PE_POISSON_BOLTZMANN && mode != PE_POISSON_LINEARIZED) return PE_EINVAL;
     if (s_w < -60 || s_w > 60) return PE_EINVAL;
     cudaStream_t s = (cudaStream_t)stream;
-    const int nb = moments_blocks(n);
+    const int nb = moments_blocks(n, ncell);
     DiagScratch* part = (DiagScratch*)scratch;
     const float wscale = ldexpf(1.0f, s_w);
     const float hk = (kick - 0.5f) * qm_dt;
-    k_moments_particles<<<nb, kDiagThreads, 0, s>>>(cell, theta, v, w, n, Ef, ncell, hk, wscale, part, status);
-    k_moments_final<<<1, kFinalThreads, 0, s>>>(part, nb, phi, E, ncell, dx, dt, ldexp(1.0, -(s_w + 24)), mode, out);
+    const bool vec = aligned16(cell) && aligned16(theta) && aligned16(v) && aligned16(w);
+    (vec ? k_moments_particles<true> : k_moments_particles<false>)<<<nb, kDiagThreads, 0, s>>>(
+        cell, theta, v, w, n, Ef, phi, E, ncell, hk, wscale, mode, part, status);
+    k_moments_final<<<1, 256, 0, s>>>(part, nb, dx, dt, ldexp(1.0, -(s_w + 24)), out);
     return launch_status(2);
 }
 

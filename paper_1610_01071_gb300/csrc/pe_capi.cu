@@ -442,20 +442,28 @@ extern "C" PE_API int pe_profile_read(pe_ctx* ctx, double* push_ms, int64_t* pus
 // diagnostics): the solution history is left alone. mode 1: the solve that starts a burst or a
 // plain-PIC step: records the history; its Newton start extrapolates the last two solutions
 // when they belong to the same trajectory one fine step apart (phi_hist).
-static int field_solve(pe_ctx* x, int step = 0)
+// chain: the solve directly follows a push of the same loop; clear: a push follows, whose charge
+// grid the solve leaves zeroed.
+static int field_solve(pe_ctx* x, int step = 0, bool chain = false, bool clear = false)
 {
     const pe_config& c = x->cfg;
-    if (x->kinetic)  // Section 4.1's two-species bursts: Poisson for the net charge
-        return timed(x, PE_PROF_FIELD, [&] {
-            return pe_field_kinetic(x->rho, x->rho_e, c.ncell, x->dx, x->s_w, x->phi, x->E, x->Ef, x->stream);
-        });
+    if (x->kinetic) {  // Section 4.1's two-species bursts: Poisson for the net charge
+        PE_TRY(timed(x, PE_PROF_FIELD, [&] {
+            return field_solve_kinetic(x->rho, x->rho_e, c.ncell, x->dx, x->s_w, x->phi, x->E, x->Ef, chain, clear,
+                                       x->stream);
+        }));
+        if (clear) x->rho_valid = 0;  // until the pushes
+        return PE_OK;
+    }
     const int extrap = step && x->phi_hist;
     double* prev = step ? x->phi + c.ncell : nullptr;
     PE_TRY(timed(x, PE_PROF_FIELD, [&] {
         return field_solve_history(x->rho, c.ncell, x->dx, x->s_w, c.poisson, c.boundary, c.newton_tol,
-                                   c.newton_maxit, x->phi, x->E, x->Ef, x->diag, x->status, prev, extrap, x->stream);
+                                   c.newton_maxit, x->phi, x->E, x->Ef, x->diag, x->status, prev, extrap, chain, clear,
+                                   x->stream);
     }));
     if (step) x->phi_hist = 1;
+    if (clear) x->rho_valid = 0;  // until the push
     return PE_OK;
 }
 
@@ -529,7 +537,7 @@ static int load_boltzmann_electrons(pe_ctx* x, uint64_t seed, ElectronDrift drif
     }
     PE_TRY(field_solve_history(x->rho, c.ncell, x->dx / sqrt(te), x->s_w, PE_POISSON_BOLTZMANN,
                                PE_BOUNDARY_PERIODIC, c.newton_tol, c.newton_maxit, x->phi, x->E, x->Ef, x->diag,
-                               x->status, nullptr, 0, x->stream));
+                               x->status, nullptr, 0, false, false, x->stream));
     PE_TRY(pe_boltzmann_profile(x->phi, mom, x->s_w, x->s_p, c.ncell, x->prof, mom ? u : nullptr, x->stream));
     const int e = x->ebank;
     PE_TRY(timed(x, PE_PROF_LOAD, [&] {
@@ -540,16 +548,17 @@ static int load_boltzmann_electrons(pe_ctx* x, uint64_t seed, ElectronDrift drif
     return PE_OK;
 }
 
-// Electron push of a fine step (kinetic electrons), in the field Ef of the ions' push.
+// Electron push of a fine step (kinetic electrons), in the field Ef of the ions' push, beside which
+// it runs; the charge grid is zeroed already.
 static int push_electrons(pe_ctx* x)
 {
     const pe_config& c = x->cfg;
     const int e = x->ebank;
     const float kick = x->e_v_at_integer ? 0.5f : 1.0f;
     PE_TRY(timed(x, PE_PROF_PUSH, [&] {
-        return pe_push_ex(x->ecell[e], x->etheta[e], x->ev[e], x->ew[e], c.nparticles, x->Ef, c.ncell,
-                          (float)(c.dt / x->dx), (float)(x->qm_e * c.dt), kick, x->s_w, c.boundary, x->rho_e, nullptr,
-                          x->status, x->stream);
+        return push_pass(x->ecell[e], x->etheta[e], x->ev[e], x->ew[e], c.nparticles, x->Ef, c.ncell,
+                         (float)(c.dt / x->dx), (float)(x->qm_e * c.dt), kick, x->s_w, c.boundary, x->rho_e, nullptr,
+                         x->status, x->stream, false, kChainBeside);
     }));
     x->e_v_at_integer = 0;
     return PE_OK;
@@ -729,6 +738,16 @@ extern "C" PE_API int pe_load_initial(pe_ctx* ctx, int32_t profile, double ampli
     return pe_measure(x, x->coarse, 1);
 }
 
+// Zeroes the charge grids for a push that does not follow a clearing field solve.
+static int clear_charge(pe_ctx* x)
+{
+    const size_t bytes = sizeof(int64_t) * (size_t)x->cfg.ncell;
+    if (cudaMemsetAsync(x->rho, 0, bytes, x->stream) != cudaSuccess ||
+        (x->kinetic && cudaMemsetAsync(x->rho_e, 0, bytes, x->stream) != cudaSuccess))
+        return PE_ECUDA;
+    return PE_OK;
+}
+
 // Fine steps p_begin .. p_end-1 of a burst, each a fused push + co-moving sample of row p
 // followed by a field solve; then, with final_sample, the sample-only row p_end. A burst
 // that starts (p_begin == 0) first solves the field of the current particles and keeps it
@@ -741,7 +760,7 @@ int pe_ctx_burst_range(pe_ctx* x, int p_begin, int p_end, int final_sample)
     if (p_begin == 0) {
         if (!x->rho_valid) PE_TRY(deposit_current(x));
         x->phi_hist = 0;  // a burst starts a new stretch of trajectory (after a lift or a load)
-        PE_TRY(field_solve(x, 1));
+        PE_TRY(field_solve(x, 1, false, p_end > 0));
         if (cudaMemcpyAsync(x->E0f, x->Ef, sizeof(float) * c.ncell, cudaMemcpyDeviceToDevice, x->stream) != cudaSuccess)
             return PE_ECUDA;
     }
@@ -753,17 +772,20 @@ int pe_ctx_burst_range(pe_ctx* x, int p_begin, int p_end, int final_sample)
         cudaMemsetAsync(sample_row(x, p_begin), 0, sizeof(int64_t) * (size_t)x->row_fx * (size_t)(last_row - p_begin + 1),
                         x->stream) != cudaSuccess)
         return PE_ECUDA;
+    // Each step is a chain of dependent launches: a push (or two), then the field solve, which also
+    // zeroes the charge for the next push.
+    if (p_begin > 0 && p_end > p_begin) PE_TRY(clear_charge(x));
     for (int p = p_begin; p < p_end; ++p) {
         if (x->te_active) PE_TRY(electron_energy_sample(x, p));
         const double tau = c.comoving ? x->dT_cur - p * c.dt : 0.0;
         pe_sample_args a = sample_args(x, tau, sample_row(x, p));
-        if (cudaMemsetAsync(x->rho, 0, sizeof(int64_t) * (size_t)c.ncell, x->stream) != cudaSuccess) return PE_ECUDA;
         PE_TRY(timed(x, x->ps ? PE_PROF_PUSH_SAMPLE_PS : PE_PROF_PUSH_SAMPLE, [&] {
             return push_pass(x->cell[b], x->theta[b], x->v[b], x->w[b], c.nparticles, x->Ef, c.ncell, dt_dx, qm_dt,
-                             kick, x->s_w, c.boundary, x->rho, &a, x->status, x->stream, false);
+                             kick, x->s_w, c.boundary, x->rho, &a, x->status, x->stream, false,
+                             p > p_begin ? kChainFirst : kChainNone);
         }));
         if (x->kinetic) PE_TRY(push_electrons(x));
-        PE_TRY(field_solve(x, 1));
+        PE_TRY(field_solve(x, 1, true, p + 1 < p_end));
         kick = 1.0f;
         x->v_at_integer = 0;
         x->rho_valid = 1;
@@ -775,7 +797,7 @@ int pe_ctx_burst_range(pe_ctx* x, int p_begin, int p_end, int final_sample)
         pe_sample_args a = sample_args(x, tau, sample_row(x, p_end));
         PE_TRY(timed(x, PE_PROF_SAMPLE, [&] {
             return sample_pass(x->cell[b], x->theta[b], x->v[b], x->w[b], c.nparticles, x->Ef, c.ncell, qm_dt, kick, &a,
-                               x->status, x->stream, false);
+                               x->status, x->stream, false, p_end > p_begin ? kChainFirst : kChainNone);
         }));
     }
     x->fresh = 0;
@@ -1023,12 +1045,14 @@ extern "C" PE_API int pe_pic_steps(pe_ctx* ctx, int32_t nsteps)
     const pe_config& c = x->cfg;
     const float dt_dx = (float)(c.dt / x->dx), qm_dt = (float)(c.qm * c.dt);
     if (nsteps > 0) x->coarse_state = 0;  // the particles move on alone
+    bool pushed = false;  // the last launch was this loop's push
     for (int s = 0; s < nsteps; ++s) {
         if (c.sort_every > 0 && (x->fine_steps % c.sort_every) == 0 && !x->fresh) {
             const int b = x->bank, o = 1 - b;
             PE_TRY(pe_sort(x->cell[b], x->theta[b], x->v[b], x->w[b], c.nparticles, c.ncell, x->cell[o], x->theta[o],
                            x->v[o], x->w[o], x->sort, x->status, x->stream));
             x->bank = o;
+            pushed = false;
             if (x->kinetic) {
                 const int e = x->ebank, eo = 1 - e;
                 PE_TRY(pe_sort(x->ecell[e], x->etheta[e], x->ev[e], x->ew[e], c.nparticles, c.ncell, x->ecell[eo],
@@ -1037,17 +1061,20 @@ extern "C" PE_API int pe_pic_steps(pe_ctx* ctx, int32_t nsteps)
             }
         }
         if (!x->rho_valid) PE_TRY(deposit_current(x));
-        if (x->kinetic && c.reset_every > 0 && (x->fine_steps % c.reset_every) == 0 && !x->fresh)
+        if (x->kinetic && c.reset_every > 0 && (x->fine_steps % c.reset_every) == 0 && !x->fresh) {
+            pushed = false;
             PE_TRY(load_boltzmann_electrons(x, electron_seed(c.seed + 0x9E3779B97F4A7C15ULL * (uint64_t)x->fine_steps),
                                             kDriftParticles));
-        PE_TRY(field_solve(x, 1));
+        }
+        PE_TRY(field_solve(x, 1, pushed, true));
         const int b = x->bank;
         const float kick = x->v_at_integer ? 0.5f : 1.0f;
         PE_TRY(timed(x, PE_PROF_PUSH, [&] {
-            return pe_push_ex(x->cell[b], x->theta[b], x->v[b], x->w[b], c.nparticles, x->Ef, c.ncell, dt_dx, qm_dt,
-                              kick, x->s_w, c.boundary, x->rho, nullptr, x->status, x->stream);
+            return push_pass(x->cell[b], x->theta[b], x->v[b], x->w[b], c.nparticles, x->Ef, c.ncell, dt_dx, qm_dt,
+                             kick, x->s_w, c.boundary, x->rho, nullptr, x->status, x->stream, false, kChainFirst);
         }));
         if (x->kinetic) PE_TRY(push_electrons(x));
+        pushed = true;
         x->v_at_integer = 0;
         x->rho_valid = 1;
         x->fresh = 0;

@@ -13,6 +13,14 @@ namespace pe {
 constexpr float kThetaOneF = 16777216.0f;  // 2^24: offset resolution of the deposit rule
 constexpr uint32_t kThetaOne = 1u << 24;
 
+// Programmatic dependent launch: grid_wait returns once the kernels this one depends on have
+// completed and their writes are visible (at once in a launch without the attribute); grid_release
+// lets the dependent launch start. A kernel that calls grid_wait before it reads or writes
+// anything may release at once; one that starts work before grid_wait relies on its predecessor
+// releasing only after its own wait (then everything before the predecessor is complete).
+__device__ __forceinline__ void grid_wait() { asm volatile("griddepcontrol.wait;" ::: "memory"); }
+__device__ __forceinline__ void grid_release() { asm volatile("griddepcontrol.launch_dependents;" ::: "memory"); }
+
 __device__ __forceinline__ void raise_flag(uint32_t* status, uint32_t bits)
 {
     if (status) atomicOr(status, bits);

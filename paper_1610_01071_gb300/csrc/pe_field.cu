@@ -12,6 +12,7 @@
 #include <string.h>
 
 #include "pe_common.cuh"
+#include "pe_ctx.h"
 #include "pe_internal.h"
 
 namespace cg = cooperative_groups;
@@ -222,7 +223,7 @@ __device__ __forceinline__ void warp_pcr(float a, float b, float c, float& d, fl
 
 // Parameters of one field solve (one realisation).
 struct FieldDesc {
-    const long long* rho;
+    long long* rho;
     double* phi;
     double* E;
     float* Ef;
@@ -235,7 +236,8 @@ struct FieldDesc {
     // Newton start: phi_prev (may be null) keeps the solution before the current one; with
     // extrap the start is the linear extrapolation 2 phi - phi_prev (solves one fine step apart)
     double* phi_prev;
-    int extrap, pad;
+    int extrap;
+    int clear;  // zero rho once read (the push that follows accumulates into it)
 };
 
 // A unit's (a warp's, a block's) rows as its neighbours see them: its first row and its last
@@ -292,12 +294,16 @@ __device__ __forceinline__ void newton_body(const FieldDesc& d, cg::cluster_grou
     // stay bit-identical to the owners' values.
     const bool hist = d.phi_prev != nullptr, ex = hist && d.extrap;
     auto start = [&](int node) { return ex ? 2.0 * d.phi[node] - d.phi_prev[node] : d.phi[node]; };
-    const long long q = __ldg(d.rho + j);
     double p = start(j);
     double halo = start(lane == 0 ? ((j - 1) & mask) : ((j + 1) & mask));
+    double gj = boltz ? exp(p) : 1.0 + p;
+    // the charge is the last push's: everything above overlaps with it in a chain of dependent launches
+    grid_wait();
+    grid_release();
+    const long long q = d.rho[j];
+    if (d.clear && act) d.rho[j] = 0;
     // density; a wall node's is twice its deposit
     const double nj = fixed_to_double(q, d.shift - ((wl || wr) ? 1 : 0));
-    double gj = boltz ? exp(p) : 1.0 + p;
     if (G > 1) asm volatile("barrier.cluster.wait.acquire.aligned;" ::: "memory");  // every block has started
 
     int it = 0;
@@ -560,7 +566,9 @@ int newton_batch_cluster_size(int ncell)
     return G <= gmax ? G : 0;
 }
 
-static cudaLaunchConfig_t cluster_config(cudaLaunchAttribute* attr, int G, int nclusters, int B, cudaStream_t s)
+// attr[2]: the cluster size, and (chain) the programmatic dependence.
+static cudaLaunchConfig_t cluster_config(cudaLaunchAttribute* attr, int G, int nclusters, int B, bool chain,
+                                         cudaStream_t s)
 {
     cudaLaunchConfig_t cfg = {};
     attr[0].id = cudaLaunchAttributeClusterDimension;
@@ -568,19 +576,21 @@ static cudaLaunchConfig_t cluster_config(cudaLaunchAttribute* attr, int G, int n
     attr[0].val.clusterDim.y = 1;
     attr[0].val.clusterDim.z = 1;
     cfg.gridDim = dim3(G * nclusters);
+    attr[1].id = cudaLaunchAttributeProgrammaticStreamSerialization;
+    attr[1].val.programmaticStreamSerializationAllowed = 1;
     cfg.blockDim = dim3(B < 32 ? 32 : B);
     cfg.stream = s;
     cfg.attrs = attr;
-    cfg.numAttrs = 1;
+    cfg.numAttrs = chain ? 2 : 1;
     return cfg;
 }
 
-static int launch_newton_cluster(int G, const FieldDesc& d, cudaStream_t s)
+static int launch_newton_cluster(int G, const FieldDesc& d, bool chain, cudaStream_t s)
 {
     const int B = d.ncell / G;  // one node per thread
     if (B > kNewtonMaxThreads || B < 2) return PE_EINVAL;
-    cudaLaunchAttribute attr[1];
-    cudaLaunchConfig_t cfg = cluster_config(attr, G, 1, B, s);
+    cudaLaunchAttribute attr[2];
+    cudaLaunchConfig_t cfg = cluster_config(attr, G, 1, B, chain, s);
     if (cudaLaunchKernelEx(&cfg, k_newton_cluster, d) != cudaSuccess) return PE_ECUDA;
     return launch_status();
 }
@@ -590,8 +600,8 @@ int launch_newton_batch(const void* descs, int R, int ncell, bool extrap, cudaSt
 {
     const int G = newton_batch_cluster_size(ncell);
     if (G < 1 || R < 1) return PE_EINVAL;
-    cudaLaunchAttribute attr[1];
-    cudaLaunchConfig_t cfg = cluster_config(attr, G, R, ncell / G, s);
+    cudaLaunchAttribute attr[2];
+    cudaLaunchConfig_t cfg = cluster_config(attr, G, R, ncell / G, false, s);
     if (cudaLaunchKernelEx(&cfg, k_newton_batch, static_cast<const FieldDesc*>(descs), extrap ? 1 : 0) != cudaSuccess)
         return PE_ECUDA;
     return launch_status();
@@ -599,10 +609,10 @@ int launch_newton_batch(const void* descs, int R, int ncell, bool extrap, cudaSt
 
 static FieldDesc field_desc(const int64_t* rho, int ncell, double dx, int s_w, int mode, int walls, double tol, int maxit,
                             double* phi, double* E, float* Ef, int32_t* diag, uint32_t* status, double* phi_prev,
-                            int extrap)
+                            int extrap, int clear)
 {
-    return FieldDesc{reinterpret_cast<const long long*>(rho), phi, E, Ef, diag, status, 1.0 / (dx * dx), 0.5 / dx,
-                     (float)tol, s_w + 24, ncell, mode, maxit, walls ? 1 : 0, phi_prev, extrap ? 1 : 0, 0};
+    return FieldDesc{reinterpret_cast<long long*>(const_cast<int64_t*>(rho)), phi, E, Ef, diag, status, 1.0 / (dx * dx), 0.5 / dx,
+                     (float)tol, s_w + 24, ncell, mode, maxit, walls ? 1 : 0, phi_prev, extrap ? 1 : 0, clear};
 }
 
 size_t field_desc_size() { return sizeof(FieldDesc); }
@@ -610,7 +620,7 @@ size_t field_desc_size() { return sizeof(FieldDesc); }
 void make_field_desc(void* out, const int64_t* rho, int ncell, double dx, int s_w, int mode, int walls, double tol,
                      int maxit, double* phi, double* E, float* Ef, int32_t* diag, uint32_t* status, double* phi_prev)
 {
-    const FieldDesc d = field_desc(rho, ncell, dx, s_w, mode, walls, tol, maxit, phi, E, Ef, diag, status, phi_prev, 0);
+    const FieldDesc d = field_desc(rho, ncell, dx, s_w, mode, walls, tol, maxit, phi, E, Ef, diag, status, phi_prev, 0, 0);
     memcpy(out, &d, sizeof(d));
 }
 
@@ -623,7 +633,7 @@ namespace pe {
 // solution before the current one, extrap selects the extrapolated start.
 int field_solve_history(const int64_t* rho_fx, int ncell, double dx, int s_w, int mode, int boundary, double tol,
                         int maxit, double* phi, double* E, float* Ef, int32_t* diag, uint32_t* status,
-                        double* phi_prev, int extrap, cudaStream_t s)
+                        double* phi_prev, int extrap, bool chain, bool clear, cudaStream_t s)
 {
     if (!is_pow2(ncell) || ncell < 8 || !rho_fx || !phi || !E || !Ef || !(dx > 0.0) || maxit < 0) return PE_EINVAL;
     if (mode != PE_POISSON_BOLTZMANN && mode != PE_POISSON_LINEARIZED) return PE_EINVAL;
@@ -632,8 +642,8 @@ int field_solve_history(const int64_t* rho_fx, int ncell, double dx, int s_w, in
     const int G = cluster_size_for(ncell);
     if (G < 1) return PE_EINVAL;
     const FieldDesc d = field_desc(rho_fx, ncell, dx, s_w, mode, boundary == PE_BOUNDARY_ABSORBING, tol, maxit, phi, E, Ef,
-                                   diag, status, phi_prev, extrap);
-    return launch_newton_cluster(G, d, s);
+                                   diag, status, phi_prev, extrap, clear ? 1 : 0);
+    return launch_newton_cluster(G, d, chain, s);
 }
 }  // namespace pe
 
@@ -677,7 +687,7 @@ __device__ __forceinline__ V block_exclusive_scan(V x, V* total, V* wsum)
     return base + incl - x;
 }
 
-__global__ void __launch_bounds__(kPoissonThreads) k_poisson_periodic(const long long* rho_i, const long long* rho_e,
+__global__ void __launch_bounds__(kPoissonThreads) k_poisson_periodic(long long* rho_i, long long* rho_e, int clear,
                                                                       int n, double dx, double nscale, double* phi,
                                                                       double* E, float* Ef)
 {
@@ -685,6 +695,8 @@ __global__ void __launch_bounds__(kPoissonThreads) k_poisson_periodic(const long
     double* F = psh;      // [n]: net charge, then the face fields F_{j+1/2}
     double* P = psh + n;  // [n]: potential before its mean is removed
     __shared__ double wd[32];
+    grid_wait();
+    grid_release();
     const int t = threadIdx.x;
     const int m = n >= (int)blockDim.x ? n / (int)blockDim.x : 1;
     const int nt = n / m;  // threads that own nodes
@@ -694,7 +706,8 @@ __global__ void __launch_bounds__(kPoissonThreads) k_poisson_periodic(const long
     double s = 0.0;
     if (act)
         for (int k = 0; k < m; ++k) {
-            const double q = (double)(__ldg(rho_i + j0 + k) - __ldg(rho_e + j0 + k));
+            const double q = (double)(rho_i[j0 + k] - rho_e[j0 + k]);
+            if (clear) rho_i[j0 + k] = rho_e[j0 + k] = 0;  // the pushes that follow accumulate
             F[j0 + k] = q;
             s += q;
         }
@@ -764,18 +777,32 @@ __global__ void k_boltzmann_profile(const double* phi, const long long* mom, int
     }
 }
 
-extern "C" PE_API int pe_field_kinetic(const int64_t* rho_i, const int64_t* rho_e, int32_t ncell, double dx,
-                                       int32_t s_w, double* phi, double* E, float* Ef, void* stream)
+namespace pe {
+int field_solve_kinetic(int64_t* rho_i, int64_t* rho_e, int ncell, double dx, int s_w, double* phi, double* E,
+                        float* Ef, bool chain, bool clear, cudaStream_t s)
 {
     if (!is_pow2(ncell) || ncell < 8 || ncell > kFullGridMax || !rho_i || !rho_e || !phi || !E || !Ef ||
         !(dx > 0.0))
         return PE_EINVAL;
     const size_t smem = 2 * sizeof(double) * (size_t)ncell;
     if (ensure_smem((const void*)k_poisson_periodic, smem) != PE_OK) return PE_ECUDA;
-    k_poisson_periodic<<<1, kPoissonThreads, smem, (cudaStream_t)stream>>>(
-        reinterpret_cast<const long long*>(rho_i), reinterpret_cast<const long long*>(rho_e), ncell, dx,
-        ldexp(1.0, -(s_w + 24)), phi, E, Ef);
+    long long* ri = reinterpret_cast<long long*>(rho_i);
+    long long* re = reinterpret_cast<long long*>(rho_e);
+    const double scale = ldexp(1.0, -(s_w + 24));
+    if (chain)
+        PE_TRY(launch_dependent(k_poisson_periodic, dim3(1), kPoissonThreads, smem, s, ri, re, clear ? 1 : 0, ncell, dx,
+                                scale, phi, E, Ef));
+    else
+        k_poisson_periodic<<<1, kPoissonThreads, smem, s>>>(ri, re, clear ? 1 : 0, ncell, dx, scale, phi, E, Ef);
     return launch_status();
+}
+}  // namespace pe
+
+extern "C" PE_API int pe_field_kinetic(const int64_t* rho_i, const int64_t* rho_e, int32_t ncell, double dx,
+                                       int32_t s_w, double* phi, double* E, float* Ef, void* stream)
+{
+    return field_solve_kinetic(const_cast<int64_t*>(rho_i), const_cast<int64_t*>(rho_e), ncell, dx, s_w, phi, E, Ef,
+                               false, false, (cudaStream_t)stream);
 }
 
 extern "C" PE_API int pe_boltzmann_profile(const double* phi, const int64_t* ion_moments, int32_t s_w, int32_t s_p,
@@ -793,7 +820,7 @@ extern "C" PE_API int pe_field_ex(const int64_t* rho_fx, int32_t ncell, double d
                                   int32_t* diag, uint32_t* status, void* stream)
 {
     return field_solve_history(rho_fx, ncell, dx, s_w, mode, boundary, tol, maxit, phi, E, Ef, diag, status, nullptr,
-                               0, (cudaStream_t)stream);
+                               0, false, false, (cudaStream_t)stream);
 }
 
 extern "C" PE_API int pe_field(const int64_t* rho_fx, int32_t ncell, double dx, int32_t s_w, int32_t mode, double tol,

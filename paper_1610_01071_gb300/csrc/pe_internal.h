@@ -39,6 +39,25 @@ int ensure_smem(const void* kernel, size_t smem);
 // Resident blocks per SM for (kernel, block, smem) on the current device (cached).
 int blocks_per_sm(const void* kernel, int block, size_t smem);
 
+// Launch with the programmatic-dependence attribute: the kernel may start while its predecessor on
+// the stream drains (grid_wait in pe_common.cuh).
+template <class... P, class... A>
+int launch_dependent(void (*kernel)(P...), dim3 grid, int block, size_t smem, cudaStream_t s, A... args)
+{
+    if (ensure_smem((const void*)kernel, smem) != PE_OK) return PE_ECUDA;
+    cudaLaunchAttribute attr[1];
+    attr[0].id = cudaLaunchAttributeProgrammaticStreamSerialization;
+    attr[0].val.programmaticStreamSerializationAllowed = 1;
+    cudaLaunchConfig_t cfg = {};
+    cfg.gridDim = grid;
+    cfg.blockDim = dim3(block);
+    cfg.dynamicSmemBytes = smem;
+    cfg.stream = s;
+    cfg.attrs = attr;
+    cfg.numAttrs = 1;
+    return cudaLaunchKernelEx(&cfg, kernel, P(args)...) == cudaSuccess ? PE_OK : PE_ECUDA;
+}
+
 // Batched field solves (pe_field.cu): descriptor size, descriptor builder, the cluster size of a
 // realisation's solve (0: the grid does not fit), the launch over R realisations of one grid size.
 size_t field_desc_size();
@@ -48,22 +67,33 @@ void make_field_desc(void* out, const int64_t* rho, int ncell, double dx, int s_
 int newton_batch_cluster_size(int ncell);
 int launch_newton_batch(const void* descs, int R, int ncell, bool extrap, cudaStream_t s);
 // Single field solve whose Newton start may extrapolate the solution history (context path).
+// chain: the solve is a link of a time step's chain of dependent launches (its predecessor on the
+// stream is a kernel of the same chain, or no kernel); clear zeroes rho_fx behind the solve's read,
+// for the push that follows.
 int field_solve_history(const int64_t* rho_fx, int ncell, double dx, int s_w, int mode, int boundary, double tol,
                         int maxit, double* phi, double* E, float* Ef, int32_t* diag, uint32_t* status,
-                        double* phi_prev, int extrap, cudaStream_t s);
+                        double* phi_prev, int extrap, bool chain, bool clear, cudaStream_t s);
+// pe_field_kinetic with the same options.
+int field_solve_kinetic(int64_t* rho_i, int64_t* rho_e, int ncell, double dx, int s_w, double* phi, double* E,
+                        float* Ef, bool chain, bool clear, cudaStream_t s);
 
 // Grid of a particle pass (pe_particles.cu): one chunk of particles (a multiple of 4, at most
 // max_chunk or 65536) per block, filling whole waves of resident blocks; returns the block count.
 int particle_grid(const void* kernel, int block, size_t smem, int64_t n, int64_t* chunk, int64_t max_chunk = 0);
 
 // pe_push_ex and pe_sample with their zeroing of the charge grid and of the sample row made
-// optional (zero = false: the caller has zeroed both, e.g. all sample rows of a burst at once).
+// optional (zero = false: the caller has zeroed both, e.g. all sample rows of a burst at once), as
+// links of a time step's chain of dependent launches. kChainNone: a launch of its own. kChainFirst:
+// after a field solve of the chain; the particles are read and the shared memory prepared before
+// the solve has ended. kChainBeside: after another species' push of the same step, which it need
+// not wait for until its own end.
+enum Chain { kChainNone = 0, kChainFirst = 1, kChainBeside = 2 };
 int push_pass(int32_t* cell, float* theta, float* v, float* w, int64_t n, const float* Ef, int32_t ncell,
               float dt_over_dx, float qm_dt, float kick, int32_t s_w, int32_t boundary, int64_t* rho_fx,
-              const pe_sample_args* sample, uint32_t* status, void* stream, bool zero);
+              const pe_sample_args* sample, uint32_t* status, void* stream, bool zero, Chain chain);
 int sample_pass(const int32_t* cell, const float* theta, const float* v, const float* w, int64_t n, const float* Ef,
                 int32_t ncell, float qm_dt, float kick, const pe_sample_args* sample, uint32_t* status, void* stream,
-                bool zero);
+                bool zero, Chain chain);
 
 // Batched particle passes (pe_particles.cu).
 size_t push_desc_size();

@@ -418,8 +418,8 @@ __global__ void __launch_bounds__(128) k_prep(const T* __restrict__ X, const flo
                                               const float* __restrict__ mu_o, const float* __restrict__ sd_o,
                                               __nv_bfloat16* __restrict__ xz, float* __restrict__ tz)
 {
-    tc::grid_release();
-    tc::grid_wait();
+    grid_release();
+    grid_wait();
     const int i = blockIdx.x;
     int64_t r = rows ? rows[i] : i;
     int s = 0;
@@ -532,8 +532,8 @@ __global__ void __launch_bounds__(tc::kThreads, 1) k_mlp_wgrad(const __grid_cons
         tc::gemm_tile<64, true>(&w.a[l], &w.b[l], (t / nx) * tc::kBM, (t % nx) * 64, w.B, e, status);
         return;
     }
-    tc::grid_release();
-    tc::grid_wait();
+    grid_release();
+    grid_wait();
     if (blk < w.bias0[L]) {
         int l = 0;
         while (blk >= w.bias0[l + 1]) ++l;
@@ -569,8 +569,8 @@ __global__ void __launch_bounds__(256) k_adam(float* __restrict__ p, __nv_bfloat
                                               double b2, float eps)
 {
     __shared__ __nv_bfloat16 tile[64][66];
-    tc::grid_release();
-    tc::grid_wait();
+    grid_release();
+    grid_wait();
     const float c1 = corr[0], c2 = corr[1];
     const float fb1 = (float)b1, fb2 = (float)b2, ob1 = (float)(1.0 - b1), ob2 = (float)(1.0 - b2);
     auto update = [&](float& w, float& mi, float& vi, float gi) {
@@ -710,25 +710,6 @@ WorkPlan plan_work(int L, const int32_t* dims, int Bm)
     for (int l = 0; l < L; ++l) w.g[l] = take(2 * (size_t)Bm * dims[l + 1]);
     w.total = o;
     return w;
-}
-
-// Launch with the programmatic-dependence attribute: the kernel may start while its predecessor on
-// the stream drains (it waits with grid_wait before touching anything a predecessor wrote).
-template <class... P, class... A>
-int launch_dependent(void (*kernel)(P...), dim3 grid, int block, size_t smem, cudaStream_t s, A... args)
-{
-    if (ensure_smem((const void*)kernel, smem) != PE_OK) return PE_ECUDA;
-    cudaLaunchAttribute attr[1];
-    attr[0].id = cudaLaunchAttributeProgrammaticStreamSerialization;
-    attr[0].val.programmaticStreamSerializationAllowed = 1;
-    cudaLaunchConfig_t cfg = {};
-    cfg.gridDim = grid;
-    cfg.blockDim = dim3(block);
-    cfg.dynamicSmemBytes = smem;
-    cfg.stream = s;
-    cfg.attrs = attr;
-    cfg.numAttrs = 1;
-    return cudaLaunchKernelEx(&cfg, kernel, P(args)...) == cudaSuccess ? PE_OK : PE_ECUDA;
 }
 
 // C[M][N] = A[M][K] B[N][K]^T on the tensor cores with the epilogue EPI; A and B stored

@@ -15,6 +15,7 @@
 #include <type_traits>
 
 #include "pe_common.cuh"
+#include "pe_ctx.h"
 #include "pe_eq.cuh"
 #include "pe_internal.h"
 
@@ -58,6 +59,7 @@ struct PushParams {
     // with v = 0); particles of weight 0 are not moved; co-moving targets outside are dropped
     int walls;
     float* w_out;
+    int chain;  // Chain: a link of a time step's chain of dependent launches
 };
 
 enum Mode {
@@ -146,6 +148,16 @@ __device__ __forceinline__ int4 lds_i4(uint32_t a)
     return v;
 }
 
+// Field values: plain loads (the field may be written while the kernel's prologue runs).
+__device__ __forceinline__ float ld_field(const float* p)
+{
+    float v;
+    asm volatile("ld.global.f32 %0, [%1];" : "=f"(v) : "l"(p));
+    return v;
+}
+
+__device__ __forceinline__ void prefetch_l2(const void* p) { asm volatile("prefetch.global.L2 [%0];" ::"l"(p)); }
+
 // 16-byte asynchronous copy global -> shared (cached in L2 only) and its group controls: each
 // lane copies its own next group of particles and waits only for its own copies.
 __device__ __forceinline__ void cp_async16(uint32_t dst, const void* src)
@@ -230,11 +242,11 @@ __device__ __forceinline__ bool process(const PushParams& P, const FieldTab& ft,
         }
     } else {
         const int c1 = (c + 1) & P.mask;
-        Ec = __ldg(P.Ef + c);
-        dE = __ldg(P.Ef + c1) - Ec;
+        Ec = ld_field(P.Ef + c);
+        dE = ld_field(P.Ef + c1) - Ec;
         if (Tr::sample) {
-            E0c = __ldg(P.E0f + c);
-            dE0 = __ldg(P.E0f + c1) - E0c;
+            E0c = ld_field(P.E0f + c);
+            dE0 = ld_field(P.E0f + c1) - E0c;
         }
     }
     const float Ep = fmaf(th, dE, Ec);
@@ -396,22 +408,7 @@ __device__ __forceinline__ void particle_chunk(const PushParams& P, int64_t begi
     constexpr bool kPS = Tr::ps;
     uint32_t* s = smem;
     FieldTab ft{0u, 0, 0};
-    if (kNeedV) {  // field table first (16-byte aligned); filled before the block barrier below
-        ft.width = P.ncell < kFieldTabNodes ? P.ncell : kFieldTabNodes;
-        ft.base = P.ncell <= kFieldTabNodes ? 0 : ((c_first - kFieldTabNodes / 4) & P.mask);
-        ft.s = smem_u32(s);
-        for (int i = threadIdx.x; i < ft.width; i += blockDim.x) {
-            const int n0 = (ft.base + i) & P.mask, n1 = (n0 + 1) & P.mask;
-            const float e0 = __ldg(P.Ef + n0), e1 = __ldg(P.Ef + n1);
-            if (Tr::sample) {
-                const float f0 = __ldg(P.E0f + n0), f1 = __ldg(P.E0f + n1);
-                reinterpret_cast<float4*>(s)[i] = make_float4(e0, e1 - e0, f0, f1 - f0);
-            } else {
-                reinterpret_cast<float2*>(s)[i] = make_float2(e0, e1 - e0);
-            }
-        }
-        s += (Tr::sample ? 4 : 2) * kFieldTabNodes;
-    }
+    if (kNeedV) s += (Tr::sample ? 4 : 2) * kFieldTabNodes;  // field table first (16-byte aligned)
     if (kRho) s = grho.bind(s, P.rho, P.rho_width < P.ncell ? ((c_first - 64) & P.mask) : 0, P.rho_width, P.mask);
     if (kSamp) {
         const int sb = P.samp_width < P.ncell ? ((c_first - P.samp_width / 2) & P.mask) : 0;
@@ -444,30 +441,10 @@ __device__ __forceinline__ void particle_chunk(const PushParams& P, int64_t begi
         bsn.zero();
         bsm.zero();
     }
-    __syncthreads();
-
     const int64_t gb0 = begin >> 2, gb1 = end >> 2;  // begin is a multiple of 4
     int64_t g0, g1;
     warp_groups(gb0, gb1, &g0, &g1);
     const int lane = threadIdx.x & 31;
-    WarpWindow win;
-    win.reset(((g0 < g1 ? P.cell[g0 << 2] : c_first) - 1) & P.mask);  // the same address in every lane
-    typename std::conditional<Tr::energy, BinWindow3, BinWindow>::type bw;
-    bw.begin(0);
-    BinSample bs;
-    // adds this lane's binned sample of one particle (weight q) through the warp's bin window
-    auto bin_add = [&](int32_t q) {
-        if constexpr (Tr::energy)
-            bw.add(bs.b, q, bs.mq, bs.eq, bs.tq, bsn, bsm, bse);
-        else
-            bw.add(bs.b, q, bs.mq, bs.tq, bsn, bsm);
-    };
-    PSAccW acc;
-    PSAcc2 acc2;  // hat rows
-    acc.reset();
-    acc2.reset();
-    bool ovf = false;
-
     int4* cell4 = reinterpret_cast<int4*>(P.cell);
     float4* th4 = reinterpret_cast<float4*>(P.theta);
     float4* v4 = reinterpret_cast<float4*>(P.v);
@@ -487,7 +464,51 @@ __device__ __forceinline__ void particle_chunk(const PushParams& P, int64_t begi
     if (Tr::stage) {
         if (g0 + lane < g1) fetch(g0 + lane, stage);
         cp_async_commit();
+    } else if (P.chain == kChainFirst && g0 + lane < g1) {
+        prefetch_l2(cell4 + g0 + lane);
+        prefetch_l2(th4 + g0 + lane);
+        if (kNeedV) prefetch_l2(v4 + g0 + lane);
+        prefetch_l2(w4 + g0 + lane);
     }
+    // In a chain of dependent launches everything above runs while the field solve ends: the
+    // particles are the last push's, which ended before that solve began.
+    if (P.chain != kChainBeside) grid_wait();
+    grid_release();
+    if (kNeedV) {
+        ft.width = P.ncell < kFieldTabNodes ? P.ncell : kFieldTabNodes;
+        ft.base = P.ncell <= kFieldTabNodes ? 0 : ((c_first - kFieldTabNodes / 4) & P.mask);
+        ft.s = smem_u32(smem);
+        for (int i = threadIdx.x; i < ft.width; i += blockDim.x) {
+            const int n0 = (ft.base + i) & P.mask, n1 = (n0 + 1) & P.mask;
+            const float e0 = ld_field(P.Ef + n0), e1 = ld_field(P.Ef + n1);
+            if (Tr::sample) {
+                const float f0 = ld_field(P.E0f + n0), f1 = ld_field(P.E0f + n1);
+                reinterpret_cast<float4*>(smem)[i] = make_float4(e0, e1 - e0, f0, f1 - f0);
+            } else {
+                reinterpret_cast<float2*>(smem)[i] = make_float2(e0, e1 - e0);
+            }
+        }
+    }
+    __syncthreads();
+
+    WarpWindow win;
+    win.reset(((g0 < g1 ? P.cell[g0 << 2] : c_first) - 1) & P.mask);  // the same address in every lane
+    typename std::conditional<Tr::energy, BinWindow3, BinWindow>::type bw;
+    bw.begin(0);
+    BinSample bs;
+    // adds this lane's binned sample of one particle (weight q) through the warp's bin window
+    auto bin_add = [&](int32_t q) {
+        if constexpr (Tr::energy)
+            bw.add(bs.b, q, bs.mq, bs.eq, bs.tq, bsn, bsm, bse);
+        else
+            bw.add(bs.b, q, bs.mq, bs.tq, bsn, bsm);
+    };
+    PSAccW acc;
+    PSAcc2 acc2;  // hat rows
+    acc.reset();
+    acc2.reset();
+    bool ovf = false;
+
     uint32_t it = 0;
     for (int64_t gs = g0; gs < g1; gs += 32, ++it) {
         const int64_t g = gs + lane;
@@ -601,6 +622,7 @@ __device__ __forceinline__ void particle_chunk(const PushParams& P, int64_t begi
         bsm.flush();
     }
     if (kPS) gps.flush();
+    if (P.chain == kChainBeside) grid_wait();  // this launch's end tells the next one that the push beside has ended too
 }
 
 // WALLS: bounded grid (a separate instantiation, so that periodic launches carry no wall code)
@@ -1076,7 +1098,9 @@ static int launch_particles(PushParams& P, cudaStream_t s, bool zero = true)
     if (zero && samp && cudaMemsetAsync(P.samp_n, 0, sizeof(int64_t) * samp_words, s) != cudaSuccess)
         return PE_ECUDA;
     if (P.n == 0) return PE_OK;
-    if (P.walls)
+    if (P.chain)
+        PE_TRY(launch_dependent(P.walls ? k_particles<MODE, true> : k_particles<MODE, false>, dim3(grid), block, smem, s, P));
+    else if (P.walls)
         k_particles<MODE, true><<<grid, block, smem, s>>>(P);
     else
         k_particles<MODE, false><<<grid, block, smem, s>>>(P);
@@ -1220,7 +1244,7 @@ namespace pe {
 
 int push_pass(int32_t* cell, float* theta, float* v, float* w, int64_t n, const float* Ef, int32_t ncell,
               float dt_over_dx, float qm_dt, float kick, int32_t s_w, int32_t boundary, int64_t* rho_fx,
-              const pe_sample_args* sample, uint32_t* status, void* stream, bool zero)
+              const pe_sample_args* sample, uint32_t* status, void* stream, bool zero, Chain chain)
 {
     if (!is_pow2(ncell) || ncell < 8 || !rho_fx || !Ef || !particles_ok(cell, theta, v, w, n)) return PE_EINVAL;
     if (boundary != PE_BOUNDARY_PERIODIC && boundary != PE_BOUNDARY_ABSORBING) return PE_EINVAL;
@@ -1242,6 +1266,7 @@ int push_pass(int32_t* cell, float* theta, float* v, float* w, int64_t n, const 
     P.status = status;
     P.walls = boundary == PE_BOUNDARY_ABSORBING;
     P.w_out = w;
+    P.chain = chain;
     if (sample) {
         P.E0f = sample->E0f;
         P.tau_dx = sample->tau * sample->inv_dx;
@@ -1272,11 +1297,12 @@ int push_pass(int32_t* cell, float* theta, float* v, float* w, int64_t n, const 
 
 int sample_pass(const int32_t* cell, const float* theta, const float* v, const float* w, int64_t n, const float* Ef,
                 int32_t ncell, float qm_dt, float kick, const pe_sample_args* sample, uint32_t* status, void* stream,
-                bool zero)
+                bool zero, Chain chain)
 {
     if (!is_pow2(ncell) || ncell < 8 || !Ef || !particles_ok(cell, theta, v, w, n) || !sample_ok(sample, ncell))
         return PE_EINVAL;
     PushParams P{};
+    P.chain = chain;
     P.walls = sample->boundary == PE_BOUNDARY_ABSORBING;
     P.cell = const_cast<int32_t*>(cell);
     P.theta = const_cast<float*>(theta);
@@ -1323,7 +1349,7 @@ extern "C" PE_API int pe_push_ex(int32_t* cell, float* theta, float* v, float* w
                                  void* stream)
 {
     return push_pass(cell, theta, v, w, n, Ef, ncell, dt_over_dx, qm_dt, kick, s_w, boundary, rho_fx, sample, status,
-                     stream, true);
+                     stream, true, kChainNone);
 }
 
 extern "C" PE_API int pe_push(int32_t* cell, float* theta, float* v, const float* w, int64_t n, const float* Ef,
@@ -1340,7 +1366,7 @@ extern "C" PE_API int pe_sample(const int32_t* cell, const float* theta, const f
                                 const float* Ef, int32_t ncell, float qm_dt, float kick, const pe_sample_args* sample,
                                 uint32_t* status, void* stream)
 {
-    return sample_pass(cell, theta, v, w, n, Ef, ncell, qm_dt, kick, sample, status, stream, true);
+    return sample_pass(cell, theta, v, w, n, Ef, ncell, qm_dt, kick, sample, status, stream, true, kChainNone);
 }
 
 // Appendix C's loading of the slots [first, first + n); prof_t != NULL loads at the local

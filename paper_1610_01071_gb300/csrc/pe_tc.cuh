@@ -21,6 +21,7 @@
 #include <cuda_runtime.h>
 #include <stdint.h>
 
+#include "pe_common.cuh"
 #include "pepic.h"
 
 namespace pe {
@@ -130,12 +131,6 @@ __host__ __device__ constexpr uint32_t idesc_bf16(int M, int N, bool mn = false)
     return (1u << 4) | (1u << 7) | (1u << 10) | (mn ? (1u << 15) | (1u << 16) : 0u) | ((uint32_t)(N >> 3) << 17) |
            ((uint32_t)(M >> 4) << 24);
 }
-
-// Programmatic dependent launch: waits until the kernels this one depends on have completed and
-// their writes are visible (returns at once in a launch without the attribute), and lets the
-// dependent launch start its prologue.
-__device__ __forceinline__ void grid_wait() { asm volatile("griddepcontrol.wait;" ::: "memory"); }
-__device__ __forceinline__ void grid_release() { asm volatile("griddepcontrol.launch_dependents;" ::: "memory"); }
 
 // 32-byte global accesses (one full sector per lane): rows are written one lane each, so narrower
 // ones would touch every sector several times. 32-byte aligned addresses.

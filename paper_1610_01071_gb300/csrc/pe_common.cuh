@@ -112,6 +112,24 @@ struct SmemGrid {
         add_digits(node, (uint32_t)val & 0xFFFFu, (uint32_t)(val >> 16) & 0xFFFFu, (int32_t)((long long)val >> 32));
     }
 
+    // Adds left at node and right at the next one: one address for both where both are inside.
+    __device__ __forceinline__ void add_pair(int node, unsigned long long left, unsigned long long right, int m) const
+    {
+        const int idx = (node - base) & m;
+        if (idx < width - 1) {
+            const uint32_t at = s + 16u * (uint32_t)idx;
+            red_u32<0>(at, (uint32_t)left & 0xFFFFu);
+            red_u32<4>(at, (uint32_t)(left >> 16) & 0xFFFFu);
+            red_s32<8>(at, (int32_t)((long long)left >> 32));
+            red_u32<16>(at, (uint32_t)right & 0xFFFFu);
+            red_u32<20>(at, (uint32_t)(right >> 16) & 0xFFFFu);
+            red_s32<24>(at, (int32_t)((long long)right >> 32));
+        } else {
+            add(node, left);
+            add((node + 1) & m, right);
+        }
+    }
+
     __device__ __forceinline__ void zero() const
     {
         for (int i = threadIdx.x; i < width; i += blockDim.x)
@@ -327,6 +345,10 @@ __device__ __forceinline__ void ps_add_warp_w(const PSGrid& gr, int key, int32_t
     const int prev = __shfl_up_sync(act, key, 1);
     const bool head = (lane == 0) || (prev != key);
     const unsigned heads = __ballot_sync(act, head);
+    if (heads == act) {  // no two neighbours share a key (unordered velocities): nothing to sum
+        if (key >= 0) gr.add(key, (long long)w * (long long)kThetaOne);
+        return;
+    }
     const unsigned after = heads & (0xFFFFFFFEu << lane);
     const int run_end = after ? (__ffs(after) - 2) : (nact - 1);
     int32_t sw = w;
@@ -379,6 +401,10 @@ __device__ __forceinline__ void ps_add_warp2(const PSGrid& gr, int key, int32_t 
     const int prev = __shfl_up_sync(act, key, 1);
     const bool head = (lane == 0) || (prev != key);
     const unsigned heads = __ballot_sync(act, head);
+    if (heads == act) {  // no two neighbours share a key
+        if (key >= 0) gr.add_pair(key, w, r);
+        return;
+    }
     const unsigned after = heads & (0xFFFFFFFEu << lane);
     const int run_end = after ? (__ffs(after) - 2) : (nact - 1);
     int32_t sw = w;
@@ -549,15 +575,22 @@ struct BinWindow {
                                         const BinGrid& gm)
     {
         const int d = (b - K) & (gn.nb - 1);
-        if (d == 0) {
-            n0 += wq;
-            m0 += mq;
-            tn += (long long)wq * (long long)tq;
-            tm += (long long)mq * (long long)tq;
-        } else if (d == 1 && tq == 0u) {
-            n1 += wq;
-            m1 += mq;
-        } else {
+        const int in1 = (d == 1) & (tq == 0u);
+        // predicated: as branches the paths ran one after the other in nearly every warp
+        asm("{\n"
+            ".reg .pred p0, p1;\n"
+            "setp.eq.s32 p0, %10, 0;\n"
+            "setp.ne.s32 p1, %11, 0;\n"
+            "@p0 add.s32 %0, %0, %6;\n"
+            "@p0 add.s32 %1, %1, %7;\n"
+            "@p0 mad.wide.s32 %4, %6, %8, %4;\n"
+            "@p0 mad.wide.s32 %5, %7, %8, %5;\n"
+            "@p1 add.s32 %2, %2, %6;\n"
+            "@p1 add.s32 %3, %3, %7;\n"
+            "}\n"
+            : "+r"(n0), "+r"(m0), "+r"(n1), "+r"(m1), "+l"(tn), "+l"(tm)
+            : "r"(wq), "r"(mq), "r"((int32_t)tq), "r"(0), "r"(d), "r"(in1));
+        if (d != 0 && !in1) {
             gn.add_whole(b, wq);
             gm.add_whole(b, mq);
             if (tq) {

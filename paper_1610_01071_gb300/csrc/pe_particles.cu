@@ -102,6 +102,11 @@ struct ModeTraits {
     // passes (three blocks an SM) and the deposit gain from it; the other passes, at four blocks
     // an SM with their loads already in flight, run faster on direct loads and a larger L1
     static constexpr bool stage = ps || MODE == kDeposit;
+    // cell range checked once per group of four (lanes past a slice's end carry weightless
+    // particles) instead of particle by particle: push 2^23 particles 38.6 -> 35.0 us (the memory
+    // bandwidth), sample 2^24 73.3 -> 70.2; the fused passes have no register left for it (263 -> 270
+    // us on the slab)
+    static constexpr bool group_check = !(push && sample);
 };
 
 // Fixed-point value rn(x 2^s); records in *ovf whether it left the range |q| <= 2^23.
@@ -210,10 +215,12 @@ __device__ __forceinline__ bool process(const PushParams& P, const FieldTab& ft,
     if (Tr::energy) bs.eq = 0;
     bs.tq = 0u;
     bs.ok = false;
-    if (!act) return false;  // a lane past the end of its warp's slice
-    if ((unsigned)c >= (unsigned)P.ncell) {
-        raise_flag(P.status, PE_FLAG_RANGE);
-        return false;
+    if (!Tr::group_check) {
+        if (!act) return false;  // a lane past the end of its warp's slice
+        if ((unsigned)c >= (unsigned)P.ncell) {
+            raise_flag(P.status, PE_FLAG_RANGE);
+            return false;
+        }
     }
     if (WALLS) {
         if (ww == 0.0f) return false;  // absorbed: frozen, carries nothing
@@ -340,14 +347,20 @@ __device__ __forceinline__ bool process(const PushParams& P, const FieldTab& ft,
 __device__ __forceinline__ void deposit_direct(const SmemGrid& g, int c, float th, int32_t wq, int mask)
 {
     const FxSplit q = fx_split(wq, th);
-    g.add(c, q.left);
-    g.add((c + 1) & mask, q.right);
+    g.add_pair(c, q.left, q.right, mask);
 }
 
 // Deposits a group (four particles per lane, dep_k set where particle k deposits at cell c_k,
 // offset th_k, weight q_k) through the warp window: when the warp's cells leave the window's
-// three cells, the window moves (warp-uniformly) to the lowest cell; cells still beyond it
-// (a spread of more than three cells) go straight to the grid. Called by all 32 lanes.
+// three cells, the window moves (warp-uniformly): to the lowest cell, or (CENTRE) where the cells
+// spread over more than three (velocities without order in the cell, few particles per cell) to
+// the middle of the spread, so that it takes the densest cells and fewer particles go straight to
+// the grid, one lane at a time. The fused passes are bound by issued instructions and gain
+// (wavelet form, 1500 ions per cell in no order: 31 -> 25 us per pass of 1.5e6; batch of mixed sizes
+// 386 -> 360 us); the plain push is bound by the shared reductions there and keeps the lowest cell
+// (electrons crossing a cell per step: 62 us per pass of 2^23, 70 with the middle). Called by all
+// 32 lanes.
+template <bool CENTRE>
 __device__ __forceinline__ void deposit_group(WarpWindow& win, const SmemGrid& g, int ncell, int mask, const int4& c,
                                               const float4& th, int32_t q0, int32_t q1, int32_t q2, int32_t q3,
                                               bool e0, bool e1, bool e2, bool e3)
@@ -364,11 +377,14 @@ __device__ __forceinline__ void deposit_group(WarpWindow& win, const SmemGrid& g
     hi = __reduce_max_sync(0xFFFFFFFFu, hi);
     if (lo == INT_MAX) return;  // nothing to deposit in this group
     if (lo < 0 || hi > 2) {
-        win.move(g, lo);
-        r0 -= lo;
-        r1 -= lo;
-        r2 -= lo;
-        r3 -= lo;
+        const int sh = (CENTRE && hi - lo > 2) ? ((lo + hi) >> 1) - 1 : lo;
+        if (sh != 0) {
+            win.move(g, sh);
+            r0 -= sh;
+            r1 -= sh;
+            r2 -= sh;
+            r3 -= sh;
+        }
     }
     if (e0) {
         if ((unsigned)r0 <= 2u) win.add(r0, fx_split(q0, th.x));
@@ -513,7 +529,9 @@ __device__ __forceinline__ void particle_chunk(const PushParams& P, int64_t begi
     for (int64_t gs = g0; gs < g1; gs += 32, ++it) {
         const int64_t g = gs + lane;
         const bool act = g < g1;
-        int4 ca = make_int4(0, 0, 0, 0);
+        // a lane past the end of its warp's slice: weightless particles in a cell of the window
+        const int c_idle = Tr::group_check ? (win.base + 1) & P.mask : 0;
+        int4 ca = make_int4(c_idle, c_idle, c_idle, c_idle);
         float4 ta = make_float4(0.f, 0.f, 0.f, 0.f), va = ta, wa = ta;
         if (Tr::stage) {
             const uint32_t cur = stage + (it & 1u) * (uint32_t)kStageSlotBytes;
@@ -531,6 +549,18 @@ __device__ __forceinline__ void particle_chunk(const PushParams& P, int64_t begi
             ta = th4[g];
             if (kNeedV) va = v4[g];
             wa = __ldg(w4 + g);
+        }
+        // cells outside [0, ncell) (any bit beyond the mask): flagged, carried as weightless and left
+        // as they are in memory
+        uint32_t bad = 0u;
+        if (Tr::group_check && __any_sync(0xFFFFFFFFu, ((ca.x | ca.y | ca.z | ca.w) & ~P.mask) != 0)) {
+            bad = ((ca.x & ~P.mask) ? 1u : 0u) | ((ca.y & ~P.mask) ? 2u : 0u) | ((ca.z & ~P.mask) ? 4u : 0u) |
+                  ((ca.w & ~P.mask) ? 8u : 0u);
+            if (bad) raise_flag(P.status, PE_FLAG_RANGE);
+            if (bad & 1u) ca.x = c_idle, ta.x = va.x = wa.x = 0.f;
+            if (bad & 2u) ca.y = c_idle, ta.y = va.y = wa.y = 0.f;
+            if (bad & 4u) ca.z = c_idle, ta.z = va.z = wa.z = 0.f;
+            if (bad & 8u) ca.w = c_idle, ta.w = va.w = wa.w = 0.f;
         }
         int4 co;
         float4 to, vo, wo;
@@ -550,6 +580,14 @@ __device__ __forceinline__ void particle_chunk(const PushParams& P, int64_t begi
         const bool e3 = process<MODE, WALLS>(P, ft, act, ca.w, ta.w, va.w, wa.w, bs, gsn, gsm, gse, gps, acc, acc2, &ovf, co.w,
                                              to.w, vo.w, wo.w, q3);
         if (kBin && bs.ok) bin_add(q3);
+        if (kWrite && bad) {
+            const int4 c = cell4[g];
+            const float4 t = th4[g], v = v4[g];
+            if (bad & 1u) co.x = c.x, to.x = t.x, vo.x = v.x, wo.x = wa.x;
+            if (bad & 2u) co.y = c.y, to.y = t.y, vo.y = v.y, wo.y = wa.y;
+            if (bad & 4u) co.z = c.z, to.z = t.z, vo.z = v.z, wo.z = wa.z;
+            if (bad & 8u) co.w = c.w, to.w = t.w, vo.w = v.w, wo.w = wa.w;
+        }
         if (kWrite && act) {
             cell4[g] = co;
             th4[g] = to;
@@ -570,7 +608,7 @@ __device__ __forceinline__ void particle_chunk(const PushParams& P, int64_t begi
             bw.end(bsn, bsm, bse);
         else if constexpr (kBin)
             bw.end(bsn, bsm);
-        if (kRho) deposit_group(win, grho, P.ncell, P.mask, co, to, q0, q1, q2, q3, e0, e1, e2, e3);
+        if (kRho) deposit_group<Tr::sample>(win, grho, P.ncell, P.mask, co, to, q0, q1, q2, q3, e0, e1, e2, e3);
     }
     if (kRho) win.flush_first(grho, 4);
     for (int64_t i = (gb1 << 2) + threadIdx.x; i < end; i += blockDim.x) {  // ragged tail (< 4 particles)
@@ -579,6 +617,10 @@ __device__ __forceinline__ void particle_chunk(const PushParams& P, int64_t begi
         int32_t q;
         const float vi = kNeedV ? P.v[i] : 0.f;
         const float wi = P.w[i];
+        if (Tr::group_check && (P.cell[i] & ~P.mask)) {
+            raise_flag(P.status, PE_FLAG_RANGE);
+            continue;
+        }
         const bool e = process<MODE, WALLS>(P, ft, true, P.cell[i], P.theta[i], vi, wi, bs, gsn, gsm, gse, gps, acc, acc2, &ovf, co,
                                             to, vo, wo, q);
         if (kWrite) {

@@ -866,6 +866,7 @@ struct EqParams {
     const float* prof_n;
     const float* prof_u;
     EqTable tab;
+    int stage_cells;
     float v_th, wscale;
     uint32_t half, shift;
     unsigned long long* rho;
@@ -873,14 +874,13 @@ struct EqParams {
     uint32_t* status;
 };
 
-__device__ __forceinline__ void eq_one(const EqParams& P, uint32_t i, int& c, float& th, float& vv, float& ww,
-                                         EqCellCache& cache)
+__device__ __forceinline__ void eq_one(const EqParams& P, const EqStage& st, uint32_t i, int& c, float& th, float& vv,
+                                       EqCursor& cur)
 {
-    const float t = eq_position(P.tab, P.prof_n, P.wall_factor, P.ncell, i, c, cache);
+    const float t = eq_position(P.tab, st, P.prof_n, P.wall_factor, P.ncell, i, c, cur);
     th = t;
     const float u0 = __ldg(P.prof_u + c), u1 = __ldg(P.prof_u + c + 1);
     const float uX = fmaf(t, u1 - u0, u0);
-    ww = (float)__ldg(P.tab.MoN);
     const uint32_t Bi = __brev(i) + P.half + P.shift;
     const bool upper = (Bi & 0x80000000u) != 0u;
     const uint32_t bs = upper ? ~Bi : Bi;
@@ -897,10 +897,12 @@ __global__ void __launch_bounds__(256) k_quiet_start_equal(EqParams P)
     const bool dep = P.rho != nullptr;
     const int c_first = (begin < end) ? eq_cell_of(P.tab, P.ncell, eq_point_of_slot((uint32_t)begin, P.n)) : 0;
     SmemGrid grho{};
+    uint32_t* free_smem = smem;
     if (dep) {
-        grho.bind(smem, P.rho, P.rho_width < P.ncell ? ((c_first - 64) & P.mask) : 0, P.rho_width, P.mask);
+        free_smem = grho.bind(smem, P.rho, P.rho_width < P.ncell ? ((c_first - 64) & P.mask) : 0, P.rho_width, P.mask);
         grho.zero();
     }
+    const EqStage st = eq_stage(free_smem, P.stage_cells, P.tab, P.prof_n, P.wall_factor, P.ncell, P.n, begin, end);
     __syncthreads();
 
     const int64_t gb0 = begin >> 2, gb1 = end >> 2;
@@ -908,8 +910,10 @@ __global__ void __launch_bounds__(256) k_quiet_start_equal(EqParams P)
     warp_groups(gb0, gb1, &g0, &g1);
     LaneWindow lw;
     lw.reset((c_first - 1) & P.mask);
-    EqCellCache cache;
-    cache.reset();
+    EqCursor cur;
+    cur.reset();
+    const float ww = (float)__ldg(P.tab.MoN);
+    const float4 ww4 = make_float4(ww, ww, ww, ww);
     bool ovf = false;
     int4* cell4 = reinterpret_cast<int4*>(P.cell);
     float4* th4 = reinterpret_cast<float4*>(P.theta);
@@ -917,34 +921,33 @@ __global__ void __launch_bounds__(256) k_quiet_start_equal(EqParams P)
     float4* w4 = reinterpret_cast<float4*>(P.w);
     for (int64_t g = g0 + (threadIdx.x & 31); g < g1; g += 32) {
         int4 c;
-        float4 t, vv, ww;
+        float4 t, vv;
         const uint32_t s0 = (uint32_t)(g << 2);
         const uint32_t p0 = eq_point_of_slot(s0, P.n), p1 = eq_point_of_slot(s0 + 1, P.n),
                        p2 = eq_point_of_slot(s0 + 2, P.n), p3 = eq_point_of_slot(s0 + 3, P.n);
-        // the four points lie within one block; search from the smallest
-        const uint32_t pmin = min(min(p0, p1), min(p2, p3));
-        const int cb = eq_cell_of(P.tab, P.ncell, pmin);
-        c.x = c.y = c.z = c.w = cb;
-        eq_one(P, p0, c.x, t.x, vv.x, ww.x, cache);
-        eq_one(P, p1, c.y, t.y, vv.y, ww.y, cache);
-        eq_one(P, p2, c.z, t.z, vv.z, ww.z, cache);
-        eq_one(P, p3, c.w, t.w, vv.w, ww.w, cache);
+        // the four points lie within one block; a search of the global table starts from the smallest
+        c.x = c.y = c.z = c.w = st.n ? 0 : eq_cell_of(P.tab, P.ncell, min(min(p0, p1), min(p2, p3)));
+        eq_one(P, st, p0, c.x, t.x, vv.x, cur);
+        eq_one(P, st, p1, c.y, t.y, vv.y, cur);
+        eq_one(P, st, p2, c.z, t.z, vv.z, cur);
+        eq_one(P, st, p3, c.w, t.w, vv.w, cur);
         cell4[g] = c;
         th4[g] = t;
         v4[g] = vv;
-        w4[g] = ww;
+        w4[g] = ww4;
         if (dep) {
-            lw.add(c.x, fx_split(fx_weight(ww.x, P.wscale, &ovf), t.x), grho);
-            lw.add(c.y, fx_split(fx_weight(ww.y, P.wscale, &ovf), t.y), grho);
-            lw.add(c.z, fx_split(fx_weight(ww.z, P.wscale, &ovf), t.z), grho);
-            lw.add(c.w, fx_split(fx_weight(ww.w, P.wscale, &ovf), t.w), grho);
+            const auto qw = fx_weight(ww, P.wscale, &ovf);
+            lw.add(c.x, fx_split(qw, t.x), grho);
+            lw.add(c.y, fx_split(qw, t.y), grho);
+            lw.add(c.z, fx_split(qw, t.z), grho);
+            lw.add(c.w, fx_split(qw, t.w), grho);
         }
     }
     for (int64_t i = (gb1 << 2) + threadIdx.x; i < end; i += blockDim.x) {
         const uint32_t pi = eq_point_of_slot((uint32_t)i, P.n);
-        int c = eq_cell_of(P.tab, P.ncell, pi);
-        float t, vv, ww;
-        eq_one(P, pi, c, t, vv, ww, cache);
+        int c = st.n ? 0 : eq_cell_of(P.tab, P.ncell, pi);
+        float t, vv;
+        eq_one(P, st, pi, c, t, vv, cur);
         P.cell[i] = c;
         P.theta[i] = t;
         P.v[i] = vv;
@@ -1505,7 +1508,8 @@ extern "C" PE_API int pe_quiet_start_equal(int32_t* cell, float* theta, float* v
     double* C = static_cast<double*>(scratch);
     long long* first = reinterpret_cast<long long*>(C + ncl + 1);
     double* MoN = reinterpret_cast<double*>(first + ncl + 1);
-    k_eq_table<float><<<1, kEqThreads, 0, s>>>(prof_n, ncell, wall_factor, n, C, first, MoN, status);
+    int* mono = reinterpret_cast<int*>(MoN + 1);
+    k_eq_table<float><<<kEqCluster, kEqBlock, 0, s>>>(prof_n, ncell, wall_factor, n, C, first, MoN, mono, status);
     EqParams P{};
     P.cell = cell;
     P.theta = theta;
@@ -1517,7 +1521,8 @@ extern "C" PE_API int pe_quiet_start_equal(int32_t* cell, float* theta, float* v
     P.wall_factor = wall_factor;
     P.prof_n = prof_n;
     P.prof_u = prof_u;
-    P.tab = EqTable{C, first, MoN};
+    P.tab = EqTable{C, first, MoN, mono};
+    P.stage_cells = eq_stage_cells(ncell);
     P.v_th = v_th;
     P.wscale = ldexpf(1.0f, s_w);
     P.half = (uint32_t)(2147483648.0 / (double)n);
@@ -1530,7 +1535,7 @@ extern "C" PE_API int pe_quiet_start_equal(int32_t* cell, float* theta, float* v
     P.rho_width = rho_fx ? (ncell <= kRhoWindowNodes ? ncell : kRhoWindowNodes) : 0;
     P.status = status;
     const int block = 256;
-    const size_t smem = kSmemGridWords * sizeof(uint32_t) * (size_t)P.rho_width;
+    const size_t smem = kSmemGridWords * sizeof(uint32_t) * (size_t)P.rho_width + eq_stage_bytes(P.stage_cells);
     const void* k = (const void*)k_quiet_start_equal;
     if (ensure_smem(k, smem) != PE_OK) return PE_ECUDA;
     const int grid = particle_grid(k, block, smem, n, &P.chunk);

@@ -363,30 +363,37 @@ __global__ void __launch_bounds__(256) k_ps_cdf(const double* __restrict__ H, in
     }
 }
 
-// Negative masses clamped to 0, the others rescaled to keep the total (summed by one thread
-// in bin order, as the host evaluation does). The masses are staged in shared memory a block
-// at a time, so the serial sums wait on FP64 adds only, not on global loads.
+// Negative masses clamped to 0, the others rescaled to keep the total (both sums in bin order,
+// as the host evaluation does). Bound by the two chains of dependent FP64 adds, 64 to 76 cycles an
+// add and scheduler: each chain has its own warp, and the values are staged (and clamped) in shared
+// memory by the whole block (512 bins: 70 us with both chains and the clamp in one thread, 21.5 us).
 __global__ void __launch_bounds__(1024) k_ps_mass(int nxc, double* __restrict__ mass)
 {
-    __shared__ double stage[1024];
-    __shared__ double sscale;
-    double tot = 0.0, pos = 0.0;
+    __shared__ double stage[2][1024];
+    __shared__ double sums[2];
+    const int wid = threadIdx.x >> 5;
+    double acc = 0.0;  // lane 0 of warp 0: the total; of warp 1: the total of the positive masses
     for (int i0 = 0; i0 < nxc; i0 += blockDim.x) {
         const int n = min((int)blockDim.x, nxc - i0);
-        if ((int)threadIdx.x < n) stage[threadIdx.x] = mass[i0 + threadIdx.x];
+        if ((int)threadIdx.x < n) {
+            const double m = mass[i0 + threadIdx.x];
+            stage[0][threadIdx.x] = m;
+            stage[1][threadIdx.x] = m > 0.0 ? m : 0.0;
+        }
         __syncthreads();
-        if (threadIdx.x == 0) {
-            for (int i = 0; i < n; ++i) {
-                const double m = stage[i];
-                tot = add_(tot, m);
-                pos = add_(pos, m > 0.0 ? m : 0.0);
-            }
+        if (wid < 2 && (threadIdx.x & 31) == 0) {
+            const double* v = stage[wid];
+#pragma unroll 8
+            for (int i = 0; i < n; ++i) acc = add_(acc, v[i]);
         }
         __syncthreads();
     }
-    if (threadIdx.x == 0) sscale = pos > 0.0 ? div_(tot, pos) : 0.0;
+    if (wid < 2 && (threadIdx.x & 31) == 0) sums[wid] = acc;
     __syncthreads();
-    for (int i = threadIdx.x; i < nxc; i += blockDim.x) mass[i] = mass[i] > 0.0 ? mul_(mass[i], sscale) : 0.0;
+    if (threadIdx.x == 0) sums[0] = sums[1] > 0.0 ? div_(sums[0], sums[1]) : 0.0;
+    __syncthreads();
+    const double scale = sums[0];
+    for (int i = threadIdx.x; i < nxc; i += blockDim.x) mass[i] = mass[i] > 0.0 ? mul_(mass[i], scale) : 0.0;
 }
 
 struct PSLoad {
@@ -879,22 +886,28 @@ __device__ __forceinline__ void ps_bracket_f(float x, int nxc, float width, floa
     phi = fminf(fmaxf((x - m0) / (m1 - m0), 0.0f), 1.0f);
 }
 
-// One block: the nodal profile prof[ncell] (FP64) of the bin densities, total = sum of the bin
-// masses (fixed-order tree), and for the per-ion blend the FP32 bin densities densf[nxc] and the
-// ion weight total / n.
+// The nodal profile prof[ncell] (FP64) of the bin densities (every block but the first,
+// kProfileNodes nodes each: ~80 FP64 instructions a node, 185 us at 8192 nodes on one SM,
+// 8.3 us spread over the GPU); in the first block, for the per-ion blend, the FP32 bin densities
+// densf[nxc] and the ion weight wn, the sum of the bin masses (fixed-order tree) over n.
+constexpr int kProfileNodes = 64;
+
 __global__ void __launch_bounds__(1024) k_ps_profile(const double* __restrict__ mass, int nxc, int bin_shift,
-                                                     int ncell, int64_t n, double* __restrict__ prof, double* total,
+                                                     int ncell, int64_t n, double* __restrict__ prof,
                                                      float* __restrict__ densf, float* wn)
 {
     __shared__ double red[32];
     const double width = ldexp(1.0, bin_shift);
-    for (int j = threadIdx.x; j < ncell; j += blockDim.x) {
+    if (blockIdx.x > 0) {
+        const int j = (blockIdx.x - 1) * kProfileNodes + threadIdx.x;
+        if (threadIdx.x >= kProfileNodes || j >= ncell) return;
         int b0, b1;
         double phi;
         ps_bracket((double)j, nxc, width, ncell, b0, b1, phi);
         const double w0 = (b0 == 0 || b0 == nxc - 1) ? width - 0.5 : width;
         const double w1 = (b1 == 0 || b1 == nxc - 1) ? width - 0.5 : width;
         prof[j] = (1.0 - phi) * (mass[b0] / w0) + phi * (mass[b1] / w1);
+        return;
     }
     for (int i = threadIdx.x; i < nxc; i += blockDim.x)
         densf[i] = (float)(mass[i] / ((i == 0 || i == nxc - 1) ? width - 0.5 : width));
@@ -906,12 +919,22 @@ __global__ void __launch_bounds__(1024) k_ps_profile(const double* __restrict__ 
     if (threadIdx.x < 32) {
         double v = (threadIdx.x < (blockDim.x >> 5)) ? red[threadIdx.x] : 0.0;
         v = warp_sum(v);
-        if (threadIdx.x == 0) {
-            *total = v;
-            *wn = (float)(v / (double)n);
-        }
+        if (threadIdx.x == 0) *wn = (float)(v / (double)n);
     }
 }
+
+// SearchHint by bin index: the storage order keeps a lane's quantiles ascending within 4096 slots, so
+// most searches start at the answer or next to it.
+struct BinHint {
+    int b0, b1, k0, k1;
+    float b;
+
+    __device__ __forceinline__ int start(int bin, float bq) const
+    {
+        if (bq < b) return 0;
+        return bin == b0 ? k0 : (bin == b1 ? k1 : 0);
+    }
+};
 
 struct PSEqLoad {
     int32_t* cell;
@@ -926,6 +949,7 @@ struct PSEqLoad {
     const float* wn;
     float width, inv_width, mid_first, mid_last;
     EqTable tab;
+    int stage_cells;
     const float* table;
     uint32_t half, shift;
     float wscale;
@@ -934,10 +958,10 @@ struct PSEqLoad {
     uint32_t* status;
 };
 
-__device__ __forceinline__ void ps_eq_one(const PSEqLoad& P, uint32_t i, int& c, float& th, float& vv, float& ww,
-                                          EqCellCache& cache)
+__device__ __forceinline__ void ps_eq_one(const PSEqLoad& P, const EqStage& st, uint32_t i, int& c, float& th, float& vv,
+                                          EqCursor& cur, BinHint& hint)
 {
-    const float t = eq_position(P.tab, P.prof, 1.0f, P.ncell, i, c, cache);
+    const float t = eq_position(P.tab, st, P.prof, 1.0f, P.ncell, i, c, cur);
     th = t;
     int b0, b1;
     float phi;
@@ -954,16 +978,21 @@ __device__ __forceinline__ void ps_eq_one(const PSEqLoad& P, uint32_t i, int& c,
     const uint32_t B = __brev(i) + P.half + P.shift;
     const float b = fmaf(__uint2float_rn(B), 2.3283064365386963e-10f, 1.1641532182693481e-10f);
     const int row = 3 * P.nv + 1;
-    const float v0 = cdf_inverse_f(P.table + (size_t)b0 * row, P.nv, b, P.vmin, P.dv);
-    const float v1 = (b1 == b0) ? v0 : cdf_inverse_f(P.table + (size_t)b1 * row, P.nv, b, P.vmin, P.dv);
+    const float* T0 = P.table + (size_t)b0 * row;
+    const float* T1 = P.table + (size_t)b1 * row;
+    int k0, k1;
+    const float v0 = cdf_inverse_f(T0, P.nv, b, P.vmin, P.dv, hint.start(b0, b), &k0);
+    float v1 = v0;
+    k1 = k0;
+    if (b1 != b0) v1 = cdf_inverse_f(T1, P.nv, b, P.vmin, P.dv, hint.start(b1, b), &k1);
+    hint = BinHint{b0, b1, k0, k1, b};
     // quantiles blended by each bin's share of the density at x: a bin without ions (whose
     // table is a placeholder) contributes nothing
     const float f = (r0 + r1 > 0.0f) ? r1 / (r0 + r1) : phi;
     vv = fmaf(f, v1 - v0, v0);
-    ww = __ldg(P.wn);
 }
 
-__global__ void __launch_bounds__(256) k_ps_quiet_start_equal(PSEqLoad P)
+__global__ void __launch_bounds__(256, 4) k_ps_quiet_start_equal(PSEqLoad P)
 {
     extern __shared__ uint32_t smem[];
     int64_t begin, end;
@@ -971,18 +1000,23 @@ __global__ void __launch_bounds__(256) k_ps_quiet_start_equal(PSEqLoad P)
     const bool dep = P.rho != nullptr;
     const int c_first = (begin < end) ? eq_cell_of(P.tab, P.ncell, eq_point_of_slot((uint32_t)begin, P.n)) : 0;
     SmemGrid grho{};
+    uint32_t* free_smem = smem;
     if (dep) {
-        grho.bind(smem, P.rho, P.rho_width < P.ncell ? ((c_first - 64) & P.mask) : 0, P.rho_width, P.mask);
+        free_smem = grho.bind(smem, P.rho, P.rho_width < P.ncell ? ((c_first - 64) & P.mask) : 0, P.rho_width, P.mask);
         grho.zero();
     }
+    const EqStage st = eq_stage(free_smem, P.stage_cells, P.tab, P.prof, 1.0f, P.ncell, P.n, begin, end);
     __syncthreads();
     const int64_t gb0 = begin >> 2, gb1 = end >> 2;
     int64_t g0, g1;
     warp_groups(gb0, gb1, &g0, &g1);
     LaneWindow lw;
     lw.reset((c_first - 1) & P.mask);
-    EqCellCache cache;
-    cache.reset();
+    EqCursor cur;
+    cur.reset();
+    BinHint hint{-1, -1, 0, 0, 0.0f};
+    const float ww = __ldg(P.wn);
+    const float4 ww4 = make_float4(ww, ww, ww, ww);
     bool ovf = false;
     int4* cell4 = reinterpret_cast<int4*>(P.cell);
     float4* th4 = reinterpret_cast<float4*>(P.theta);
@@ -990,32 +1024,32 @@ __global__ void __launch_bounds__(256) k_ps_quiet_start_equal(PSEqLoad P)
     float4* w4 = reinterpret_cast<float4*>(P.w);
     for (int64_t g = g0 + (threadIdx.x & 31); g < g1; g += 32) {
         int4 c;
-        float4 t, vv, ww;
+        float4 t, vv;
         const uint32_t s0 = (uint32_t)(g << 2);
         const uint32_t p0 = eq_point_of_slot(s0, P.n), p1 = eq_point_of_slot(s0 + 1, P.n),
                        p2 = eq_point_of_slot(s0 + 2, P.n), p3 = eq_point_of_slot(s0 + 3, P.n);
-        const int cb = eq_cell_of(P.tab, P.ncell, min(min(p0, p1), min(p2, p3)));
-        c.x = c.y = c.z = c.w = cb;
-        ps_eq_one(P, p0, c.x, t.x, vv.x, ww.x, cache);
-        ps_eq_one(P, p1, c.y, t.y, vv.y, ww.y, cache);
-        ps_eq_one(P, p2, c.z, t.z, vv.z, ww.z, cache);
-        ps_eq_one(P, p3, c.w, t.w, vv.w, ww.w, cache);
+        c.x = c.y = c.z = c.w = st.n ? 0 : eq_cell_of(P.tab, P.ncell, min(min(p0, p1), min(p2, p3)));
+        ps_eq_one(P, st, p0, c.x, t.x, vv.x, cur, hint);
+        ps_eq_one(P, st, p1, c.y, t.y, vv.y, cur, hint);
+        ps_eq_one(P, st, p2, c.z, t.z, vv.z, cur, hint);
+        ps_eq_one(P, st, p3, c.w, t.w, vv.w, cur, hint);
         cell4[g] = c;
         th4[g] = t;
         v4[g] = vv;
-        w4[g] = ww;
+        w4[g] = ww4;
         if (dep) {
-            lw.add(c.x, fx_split(fx_weight_q(ww.x, P.wscale, &ovf), t.x), grho);
-            lw.add(c.y, fx_split(fx_weight_q(ww.y, P.wscale, &ovf), t.y), grho);
-            lw.add(c.z, fx_split(fx_weight_q(ww.z, P.wscale, &ovf), t.z), grho);
-            lw.add(c.w, fx_split(fx_weight_q(ww.w, P.wscale, &ovf), t.w), grho);
+            const auto qw = fx_weight_q(ww, P.wscale, &ovf);
+            lw.add(c.x, fx_split(qw, t.x), grho);
+            lw.add(c.y, fx_split(qw, t.y), grho);
+            lw.add(c.z, fx_split(qw, t.z), grho);
+            lw.add(c.w, fx_split(qw, t.w), grho);
         }
     }
     for (int64_t i = (gb1 << 2) + threadIdx.x; i < end; i += blockDim.x) {
         const uint32_t pi = eq_point_of_slot((uint32_t)i, P.n);
-        int c = eq_cell_of(P.tab, P.ncell, pi);
-        float t, vv, ww;
-        ps_eq_one(P, pi, c, t, vv, ww, cache);
+        int c = st.n ? 0 : eq_cell_of(P.tab, P.ncell, pi);
+        float t, vv;
+        ps_eq_one(P, st, pi, c, t, vv, cur, hint);
         P.cell[i] = c;
         P.theta[i] = t;
         P.v[i] = vv;
@@ -1261,11 +1295,12 @@ extern "C" PE_API int pe_ps_quiet_start_equal(int32_t* cell, float* theta, float
     double* C = prof + ncell;                                            // [ncl + 1]
     long long* first = reinterpret_cast<long long*>(C + ncl + 1);        // [ncl + 1]
     double* MoN = reinterpret_cast<double*>(first + ncl + 1);           // [1]
-    double* total = MoN + 1;                                             // [1]
-    float* densf = reinterpret_cast<float*>(total + 1);                  // [nxc]
+    int* mono = reinterpret_cast<int*>(MoN + 1);                         // [1], 8 bytes
+    float* densf = reinterpret_cast<float*>(MoN + 2);                    // [nxc]
     float* wn = densf + nxc;                                             // [1]
-    k_ps_profile<<<1, 1024, 0, s>>>(mass, nxc, bin_shift, ncell, n, prof, total, densf, wn);
-    k_eq_table<double><<<1, kEqThreads, 0, s>>>(prof, ncell, 1.0f, n, C, first, MoN, status);
+    k_ps_profile<<<1 + (ncell + kProfileNodes - 1) / kProfileNodes, 1024, 0, s>>>(mass, nxc, bin_shift, ncell, n, prof,
+                                                                                  densf, wn);
+    k_eq_table<double><<<kEqCluster, kEqBlock, 0, s>>>(prof, ncell, 1.0f, n, C, first, MoN, mono, status);
     PSEqLoad P{};
     P.cell = cell;
     P.theta = theta;
@@ -1286,7 +1321,8 @@ extern "C" PE_API int pe_ps_quiet_start_equal(int32_t* cell, float* theta, float
     P.inv_width = ldexpf(1.0f, -bin_shift);
     P.mid_first = 0.5f * (P.width - 0.5f);
     P.mid_last = (float)(0.5 * ((nxc - 1) * (double)P.width - 0.5 + (double)(ncell - 1)));
-    P.tab = EqTable{C, first, MoN};
+    P.tab = EqTable{C, first, MoN, mono};
+    P.stage_cells = eq_stage_cells(ncell);
     P.table = table;
     P.half = (uint32_t)(2147483648.0 / (double)n);
     uint64_t z = seed + 0x9E3779B97F4A7C15ULL;  // splitmix64 of the seed: the shift is its upper half
@@ -1298,7 +1334,8 @@ extern "C" PE_API int pe_ps_quiet_start_equal(int32_t* cell, float* theta, float
     P.rho = reinterpret_cast<unsigned long long*>(rho_fx);
     P.rho_width = ncell <= kRhoWindowNodes ? ncell : kRhoWindowNodes;
     P.status = status;
-    const size_t smem = rho_fx ? kSmemGridWords * sizeof(uint32_t) * (size_t)P.rho_width : 0;
+    const size_t smem = (rho_fx ? kSmemGridWords * sizeof(uint32_t) * (size_t)P.rho_width : 0) +
+                        eq_stage_bytes(P.stage_cells);
     const void* k = (const void*)k_ps_quiet_start_equal;
     if (ensure_smem(k, smem) != PE_OK) return PE_ECUDA;
     const int grid = particle_grid(k, 256, smem, n, &P.chunk);

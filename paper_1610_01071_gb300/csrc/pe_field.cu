@@ -238,6 +238,7 @@ struct FieldDesc {
     double* phi_prev;
     int extrap;
     int clear;  // zero rho once read (the push that follows accumulates into it)
+    float* Ef0;  // batch: second copy of Ef by the solve that starts a burst (the frozen field), or null
 };
 
 // A unit's (a warp's, a block's) rows as its neighbours see them: its first row and its last
@@ -486,6 +487,7 @@ __device__ __forceinline__ void newton_body(const FieldDesc& d, cg::cluster_grou
         d.phi[j] = p;
         d.E[j] = e;
         d.Ef[j] = f32_of(e);
+        if (d.Ef0) d.Ef0[j] = f32_of(e);
     }
     if (g == 0 && i == 0) {
         if (d.diag) {
@@ -504,12 +506,14 @@ __global__ void __launch_bounds__(kNewtonMaxThreads, 1) k_newton_cluster(FieldDe
     newton_body(d, cluster);
 }
 
-// One cluster per realisation: cluster c solves descs[c]; extrap applies to every realisation.
+// One cluster per realisation: cluster c solves descs[c]; extrap (a solve inside a burst, not the one
+// that starts it) applies to every realisation.
 __global__ void __launch_bounds__(kNewtonMaxThreads, 1) k_newton_batch(const FieldDesc* descs, int extrap)
 {
     cg::cluster_group cluster = cg::this_cluster();
     FieldDesc d = descs[blockIdx.x / cluster.num_blocks()];
     d.extrap = extrap;
+    if (extrap) d.Ef0 = nullptr;
     newton_body(d, cluster);
 }
 
@@ -612,15 +616,17 @@ static FieldDesc field_desc(const int64_t* rho, int ncell, double dx, int s_w, i
                             int extrap, int clear)
 {
     return FieldDesc{reinterpret_cast<long long*>(const_cast<int64_t*>(rho)), phi, E, Ef, diag, status, 1.0 / (dx * dx), 0.5 / dx,
-                     (float)tol, s_w + 24, ncell, mode, maxit, walls ? 1 : 0, phi_prev, extrap ? 1 : 0, clear};
+                     (float)tol, s_w + 24, ncell, mode, maxit, walls ? 1 : 0, phi_prev, extrap ? 1 : 0, clear, nullptr};
 }
 
 size_t field_desc_size() { return sizeof(FieldDesc); }
 
 void make_field_desc(void* out, const int64_t* rho, int ncell, double dx, int s_w, int mode, int walls, double tol,
-                     int maxit, double* phi, double* E, float* Ef, int32_t* diag, uint32_t* status, double* phi_prev)
+                     int maxit, double* phi, double* E, float* Ef, float* Ef0, int32_t* diag, uint32_t* status,
+                     double* phi_prev)
 {
-    const FieldDesc d = field_desc(rho, ncell, dx, s_w, mode, walls, tol, maxit, phi, E, Ef, diag, status, phi_prev, 0, 0);
+    FieldDesc d = field_desc(rho, ncell, dx, s_w, mode, walls, tol, maxit, phi, E, Ef, diag, status, phi_prev, 0, 1);
+    d.Ef0 = Ef0;
     memcpy(out, &d, sizeof(d));
 }
 

@@ -62,7 +62,7 @@ int launch_dependent(void (*kernel)(P...), dim3 grid, int block, size_t smem, cu
 // realisation's solve (0: the grid does not fit), the launch over R realisations of one grid size.
 size_t field_desc_size();
 void make_field_desc(void* out, const int64_t* rho, int ncell, double dx, int s_w, int mode, int walls, double tol,
-                     int maxit, double* phi, double* E, float* Ef, int32_t* diag, uint32_t* status,
+                     int maxit, double* phi, double* E, float* Ef, float* Ef0, int32_t* diag, uint32_t* status,
                      double* phi_prev);
 int newton_batch_cluster_size(int ncell);
 int launch_newton_batch(const void* descs, int R, int ncell, bool extrap, cudaStream_t s);
@@ -103,7 +103,7 @@ void make_push_desc(void* out, int32_t* cell, float* theta, float* v, const floa
                     float inv_dx, float qm, int comoving, int s_p, int bin_shift, int64_t* samp_base,
                     int64_t row_stride, int walls, uint32_t* status);
 void make_work_item(void* out, int r, int64_t begin, int64_t end);
-int launch_particles_batch(int mode, const void* descs, const void* items, int nitems, int p, float kick,
+int launch_particles_batch(bool push, const void* descs, const void* items, int nitems, int p, float kick,
                            unsigned* counter, int max_ncell, int max_nb, int block, int priv, cudaStream_t s);
 
 // Batched restriction + projection of Haar-binned samples (pe_coarse.cu).

@@ -691,9 +691,10 @@ struct WorkItem {
     int r, pad;
 };
 
-// Persistent batched launch over the work items of many realisations: each block takes
-// the next item from a global counter until none are left. Step p and the kick are the
-// same for every realisation; tau and the sample row follow from each descriptor.
+// Persistent batched launch over the work items of many realisations: block b starts with item b and
+// takes further items from a counter (zero before the launch) until none are left, each asked for
+// while the one before it is processed. Step p and the kick are the same for every
+// realisation; tau and the sample row follow from each descriptor.
 // Blocks of 128, 256 or 512 threads (the tuner's choice), at the register budget of 1024 threads
 // per SM; priv = 0 sends every deposit straight to the global grid (no shared-memory window).
 template <int MODE>
@@ -702,12 +703,9 @@ __global__ void __launch_bounds__(512, 2) k_particles_batch(const PushParams* de
 {
     extern __shared__ uint32_t smem[];
     __shared__ int next;
-    for (;;) {
-        if (threadIdx.x == 0) next = (int)atomicAdd(counter, 1u);
-        __syncthreads();
-        const int it = next;
-        __syncthreads();
-        if (it >= nitems) break;
+    for (int it = blockIdx.x; it < nitems; it = next) {
+        __syncthreads();  // the grids are flushed, next is read
+        if (threadIdx.x == 0) next = (int)gridDim.x + (int)atomicAdd(counter, 1u);
         const WorkItem wi = items[it];
         PushParams P = descs[wi.r];
         P.kick = kick;
@@ -723,7 +721,7 @@ __global__ void __launch_bounds__(512, 2) k_particles_batch(const PushParams* de
             particle_chunk<MODE, true>(P, wi.begin, wi.end, smem);
         else
             particle_chunk<MODE, false>(P, wi.begin, wi.end, smem);
-        __syncthreads();
+        __syncthreads();  // next is written
     }
 }
 
@@ -1227,41 +1225,38 @@ void make_work_item(void* out, int r, int64_t begin, int64_t end)
     memcpy(out, &wi, sizeof(wi));
 }
 
-// Shared memory of a batched launch: the field table, the deposit window (priv), the bins.
-static size_t batch_smem(int mode, int max_ncell, int max_nb, int priv, int block)
+// Shared memory of a batched launch: the field table, the deposit window (a push with priv), the bins.
+static size_t batch_smem(bool push, int max_ncell, int max_nb, int priv, int block)
 {
-    const int rw = (mode != 1 && priv) ? (max_ncell <= kRhoWindowNodes ? max_ncell : kRhoWindowNodes) : 0;
-    return with_stage((mode == 2 ? 0 : sizeof(float4) * (size_t)kFieldTabNodes) +
-                          kSmemGridWords * sizeof(uint32_t) * (size_t)rw +
-                          (mode == 2 ? 0 : kBinGridWords * sizeof(uint32_t) * 2 * (size_t)max_nb),
-                      block, mode == 2);
+    const int rw = (push && priv) ? (max_ncell <= kRhoWindowNodes ? max_ncell : kRhoWindowNodes) : 0;
+    return with_stage(sizeof(float4) * (size_t)kFieldTabNodes + kSmemGridWords * sizeof(uint32_t) * (size_t)rw +
+                          kBinGridWords * sizeof(uint32_t) * 2 * (size_t)max_nb,
+                      block, false);
 }
 
 template <int MODE>
-static int launch_batch_mode(const void* descs, const void* items, int nitems, int p, float kick, unsigned* counter,
-                             size_t smem, int block, int priv, cudaStream_t s)
+static int launch_batch_mode(const void* descs, const void* items, int nitems, int p, float kick, size_t smem,
+                             unsigned* counter, int block, int priv, cudaStream_t s)
 {
     const void* k = (const void*)k_particles_batch<MODE>;
     if (ensure_smem(k, smem) != PE_OK) return PE_ECUDA;
-    const int grid = sm_count() * blocks_per_sm(k, block, smem);
+    const int grid = std::min(nitems, sm_count() * blocks_per_sm(k, block, smem));
     k_particles_batch<MODE><<<grid, block, smem, s>>>(static_cast<const PushParams*>(descs),
                                                       static_cast<const WorkItem*>(items), nitems, p, kick, counter,
                                                       priv);
     return launch_status();
 }
 
-// mode 0: fused push + binned sample of step p; mode 1: binned sample only; mode 2: charge
-// deposit only (the tuner's probe of the deposit path). block: 128, 256 or 512 threads.
-int launch_particles_batch(int mode, const void* descs, const void* items, int nitems, int p, float kick,
+// push: fused push + binned sample of step p; otherwise the binned sample alone. counter: this launch's
+// own, zeroed. block: 128, 256 or 512 threads.
+int launch_particles_batch(bool push, const void* descs, const void* items, int nitems, int p, float kick,
                            unsigned* counter, int max_ncell, int max_nb, int block, int priv, cudaStream_t s)
 {
     if (block != 128 && block != 256 && block != 512) return PE_EINVAL;
-    const size_t smem = batch_smem(mode, max_ncell, max_nb, priv, block);
+    const size_t smem = batch_smem(push, max_ncell, max_nb, priv, block);
     if (smem > (size_t)max_smem_optin()) return PE_EINVAL;
-    if (cudaMemsetAsync(counter, 0, sizeof(unsigned), s) != cudaSuccess) return PE_ECUDA;
-    if (mode == 0) return launch_batch_mode<kPushSampleBinned>(descs, items, nitems, p, kick, counter, smem, block, priv, s);
-    if (mode == 1) return launch_batch_mode<kSampleBinned>(descs, items, nitems, p, kick, counter, smem, block, priv, s);
-    return launch_batch_mode<kDeposit>(descs, items, nitems, p, kick, counter, smem, block, priv, s);
+    if (push) return launch_batch_mode<kPushSampleBinned>(descs, items, nitems, p, kick, smem, counter, block, priv, s);
+    return launch_batch_mode<kSampleBinned>(descs, items, nitems, p, kick, smem, counter, block, priv, s);
 }
 
 }  // namespace pe

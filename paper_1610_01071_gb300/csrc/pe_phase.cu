@@ -1007,49 +1007,24 @@ __global__ void __launch_bounds__(256, 4) k_ps_quiet_start_equal(PSEqLoad P)
     }
     const EqStage st = eq_stage(free_smem, P.stage_cells, P.tab, P.prof, 1.0f, P.ncell, P.n, begin, end);
     __syncthreads();
-    const int64_t gb0 = begin >> 2, gb1 = end >> 2;
-    int64_t g0, g1;
-    warp_groups(gb0, gb1, &g0, &g1);
+    // One slot per lane and turn: the 32 lanes' points lie 128 apart and a lane stays within 128
+    // consecutive points for a whole block of 4096 slots, its quantiles ascending.
+    const int nw = blockDim.x >> 5, wid = threadIdx.x >> 5;
+    const int64_t per = (((end - begin + nw - 1) / nw) + 31) & ~int64_t(31);
+    const int64_t a = begin + per * wid, b = a + per < end ? a + per : end;
     LaneWindow lw;
     lw.reset((c_first - 1) & P.mask);
     EqCursor cur;
     cur.reset();
     BinHint hint{-1, -1, 0, 0, 0.0f};
     const float ww = __ldg(P.wn);
-    const float4 ww4 = make_float4(ww, ww, ww, ww);
     bool ovf = false;
-    int4* cell4 = reinterpret_cast<int4*>(P.cell);
-    float4* th4 = reinterpret_cast<float4*>(P.theta);
-    float4* v4 = reinterpret_cast<float4*>(P.v);
-    float4* w4 = reinterpret_cast<float4*>(P.w);
-    for (int64_t g = g0 + (threadIdx.x & 31); g < g1; g += 32) {
-        int4 c;
-        float4 t, vv;
-        const uint32_t s0 = (uint32_t)(g << 2);
-        const uint32_t p0 = eq_point_of_slot(s0, P.n), p1 = eq_point_of_slot(s0 + 1, P.n),
-                       p2 = eq_point_of_slot(s0 + 2, P.n), p3 = eq_point_of_slot(s0 + 3, P.n);
-        c.x = c.y = c.z = c.w = st.n ? 0 : eq_cell_of(P.tab, P.ncell, min(min(p0, p1), min(p2, p3)));
-        ps_eq_one(P, st, p0, c.x, t.x, vv.x, cur, hint);
-        ps_eq_one(P, st, p1, c.y, t.y, vv.y, cur, hint);
-        ps_eq_one(P, st, p2, c.z, t.z, vv.z, cur, hint);
-        ps_eq_one(P, st, p3, c.w, t.w, vv.w, cur, hint);
-        cell4[g] = c;
-        th4[g] = t;
-        v4[g] = vv;
-        w4[g] = ww4;
-        if (dep) {
-            const auto qw = fx_weight_q(ww, P.wscale, &ovf);
-            lw.add(c.x, fx_split(qw, t.x), grho);
-            lw.add(c.y, fx_split(qw, t.y), grho);
-            lw.add(c.z, fx_split(qw, t.z), grho);
-            lw.add(c.w, fx_split(qw, t.w), grho);
-        }
-    }
-    for (int64_t i = (gb1 << 2) + threadIdx.x; i < end; i += blockDim.x) {
-        const uint32_t pi = eq_point_of_slot((uint32_t)i, P.n);
-        int c = st.n ? 0 : eq_cell_of(P.tab, P.ncell, pi);
+#pragma unroll 1
+    for (int64_t i = a + (threadIdx.x & 31); i < b; i += 32) {
+        const uint32_t pt = eq_point_of_slot((uint32_t)i, P.n);
+        int c = st.n ? 0 : eq_cell_of(P.tab, P.ncell, pt);
         float t, vv;
-        ps_eq_one(P, st, pi, c, t, vv, cur, hint);
+        ps_eq_one(P, st, pt, c, t, vv, cur, hint);
         P.cell[i] = c;
         P.theta[i] = t;
         P.v[i] = vv;

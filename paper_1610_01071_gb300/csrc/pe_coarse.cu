@@ -227,7 +227,7 @@ __global__ void __launch_bounds__(256) k_coarsen(const long long* fx, int ncell,
     for (int k = threadIdx.x; k < n_coarse; k += blockDim.x) out[(size_t)row * n_coarse + k] = a[k];
 }
 
-__device__ void synth_level(const Filter& f, const double* a, int nin, double* b);
+__device__ void synth_level(const Filter& f, const double* a, int nin, double* b, int i0, int i1);
 
 // Phase space, wavelet form (Section 3.3): one block per row of nvf fixed-point values (coarse
 // node i of sample p, hat-weighted in x), converted with `scale` and analysed in v by the
@@ -270,7 +270,7 @@ __global__ void __launch_bounds__(256) k_ps_refine_v(const double* coarse, int n
     double* a = x;
     double* b = y;
     for (int len = nvc; len < nvf; len <<= 1) {
-        synth_level(f, a, len, b);
+        synth_level(f, a, len, b, 0, 2 * len);
         __syncthreads();
         double* t = a;
         a = b;
@@ -280,14 +280,38 @@ __global__ void __launch_bounds__(256) k_ps_refine_v(const double* coarse, int n
 }
 
 // Least-squares slope in the paired form of Eq. (leastsquares) and the forward-Euler leap.
-__global__ void k_ls_project(const double* c, int K, int ncoef, double dt, double dT, double* out, double* slope)
+// FP64 issue bounds both forms of this (64 to 76 cycles a warp instruction and scheduler): the pairs'
+// factors, a division each, are formed once per block, and blocks are small, to reach many SMs
+// (512 components, 21 samples: 14.5 us with a division per component and pair, 6.5 us so).
+constexpr int kProjectThreads = 64;
+
+// Factors 6 (K - 2p) / den of the pairs p0 .. p0 + n - 1 into w (all threads of the block).
+__device__ __forceinline__ void pair_factors(int K, double den, int p0, int n, double* w)
 {
+    __syncthreads();
+    for (int k = threadIdx.x; k < n; k += blockDim.x) w[k] = 6.0 * (K - 2 * (p0 + k)) / den;
+    __syncthreads();
+}
+
+__global__ void __launch_bounds__(kProjectThreads) k_ls_project(const double* c, int K, int ncoef, double dt, double dT,
+                                                                double* out, double* slope)
+{
+    __shared__ double w[kProjectThreads];
     const int i = blockIdx.x * blockDim.x + threadIdx.x;
-    if (i >= ncoef) return;
     const double den = (double)K * (K + 1) * (K + 2) * dt;
     double s = 0.0;
-    for (int p = 0; 2 * p <= K; ++p)
-        s += 6.0 * (K - 2 * p) / den * (c[(size_t)(K - p) * ncoef + i] - c[(size_t)p * ncoef + i]);
+    for (int p0 = 0; 2 * p0 <= K; p0 += kProjectThreads) {
+        const int n = min(kProjectThreads, K / 2 + 1 - p0);
+        pair_factors(K, den, p0, n, w);
+        if (i < ncoef) {
+#pragma unroll 4
+            for (int k = 0; k < n; ++k) {
+                const int p = p0 + k;
+                s += w[k] * (c[(size_t)(K - p) * ncoef + i] - c[(size_t)p * ncoef + i]);
+            }
+        }
+    }
+    if (i >= ncoef) return;
     if (slope) slope[i] = s;
     out[i] = c[(size_t)K * ncoef + i] + (dT - K * dt) * s;
 }
@@ -314,41 +338,68 @@ __device__ double block_max_d(double v, double* red)
     return warp_max(lane < nw ? red[lane] : -1e300);
 }
 
-// Periodized synthesis with zero details from nin coefficients in a to 2*nin in b.
-__device__ void synth_level(const Filter& f, const double* a, int nin, double* b)
+__device__ long long block_max_ll(long long v, double* red)
+{
+    auto up = [](long long x) {
+        for (int o = 16; o > 0; o >>= 1) {
+            const long long y = __shfl_xor_sync(0xffffffffu, x, o);
+            x = y > x ? y : x;
+        }
+        return x;
+    };
+    v = up(v);
+    const int lane = threadIdx.x & 31, wid = threadIdx.x >> 5;
+    __syncthreads();
+    if (lane == 0) red[wid] = __longlong_as_double(v);
+    __syncthreads();
+    const int nw = (blockDim.x + 31) >> 5;
+    return up(lane < nw ? __double_as_longlong(red[lane]) : 0ll);
+}
+
+// Periodized synthesis with zero details from nin coefficients in a to the values [i0, i1) of the 2*nin
+// in b.
+__device__ void synth_level(const Filter& f, const double* a, int nin, double* b, int i0, int i1)
 {
     const int n = 2 * nin;
-    for (int i = threadIdx.x; i < n; i += blockDim.x) {
+    for (int i = i0 + threadIdx.x; i < i1; i += blockDim.x) {
         double acc = 0.0;
         for (int m = (i & 1); m < f.len; m += 2) acc += f.h[m] * a[((i - m) & (n - 1)) >> 1];
         b[i] = acc;
     }
 }
 
-// Returns the buffer holding the refined values (one of x, y).
+// Returns the buffer holding the refined values [j0, j1) (one of x, y).
 __device__ double* synthesise(const Filter& f, const double* coarse, int nc, int ncell, double* x, double* y,
-                              double scale)
+                              double scale, int j0, int j1)
 {
     for (int k = threadIdx.x; k < nc; k += blockDim.x) x[k] = coarse[k];
     __syncthreads();
     double* a = x;
     double* b = y;
     for (int len = nc; len < ncell; len <<= 1) {
-        synth_level(f, a, len, b);
+        if (2 * len < ncell) synth_level(f, a, len, b, 0, 2 * len);
+        else synth_level(f, a, len, b, j0, j1);
         __syncthreads();
         double* t = a;
         a = b;
         b = t;
     }
-    for (int j = threadIdx.x; j < ncell; j += blockDim.x) a[j] *= scale;
+    for (int j = j0 + threadIdx.x; j < j1; j += blockDim.x) a[j] *= scale;
     __syncthreads();
     return a;
 }
 
 template <typename P>
 __device__ __forceinline__ void refine_body(const double* coarse, int nc, const Filter& f, int ncell, double scale,
-                                            P* prof_n, P* prof_u, double* buf, double* red,
+                                            P* prof_n, P* prof_u, double* buf, double* red, int part, int parts,
                                             const double** nf_out = nullptr, const double** mf_out = nullptr);
+
+// Blocks of a lifting profile. Each forms the whole density (its maximum and its sign bound the
+// velocities and the clamp) and its own share of the momentum, quotients and outputs. FP64 issue of
+// one SM bounds a block, ~12 of a node's 28 FP64 instructions were the quotient's and 6 sums that only a
+// negative density needs (4096 nodes: 52 us in one block, 16 us in eight; 24 grids of up to 8192
+// nodes: 82 us with a block each, 60 us with four).
+constexpr int kRefineParts = 8, kRefineBatchParts = 4;
 
 template <typename P>
 __global__ void __launch_bounds__(1024) k_refine(const double* coarse, int nc, Filter f, int ncell, double scale,
@@ -356,10 +407,10 @@ __global__ void __launch_bounds__(1024) k_refine(const double* coarse, int nc, F
 {
     extern __shared__ double buf[];
     __shared__ double red[32];
-    refine_body(coarse, nc, f, ncell, scale, prof_n, prof_u, buf, red);
+    refine_body(coarse, nc, f, ncell, scale, prof_n, prof_u, buf, red, (int)blockIdx.x, (int)gridDim.x);
 }
 
-// Lifting profiles of many realisations in one launch (the batched ensemble), block r for
+// Lifting profiles of many realisations in one launch (the batched ensemble), blocks (r, *) for
 // realisation r: the same arithmetic as k_refine.
 struct RefineDesc {
     const double* coarse;
@@ -374,40 +425,53 @@ __global__ void __launch_bounds__(1024) k_refine_batch(const RefineDesc* d, Filt
     extern __shared__ double buf[];
     __shared__ double red[32];
     const RefineDesc r = d[blockIdx.x];
-    refine_body(r.coarse, r.nc, f, r.ncell, r.scale, r.prof_n, r.prof_u, buf, red);
+    refine_body(r.coarse, r.nc, f, r.ncell, r.scale, r.prof_n, r.prof_u, buf, red, (int)blockIdx.y, (int)gridDim.y);
 }
 
 template <typename P>
 __device__ __forceinline__ void refine_body(const double* coarse, int nc, const Filter& f, int ncell, double scale,
-                                            P* prof_n, P* prof_u, double* buf, double* red, const double** nf_out,
-                                            const double** mf_out)
+                                            P* prof_n, P* prof_u, double* buf, double* red, int part, int parts,
+                                            const double** nf_out, const double** mf_out)
 {
+    const int p0 = (int)((int64_t)ncell * part / parts), p1 = (int)((int64_t)ncell * (part + 1) / parts);
     double* X = buf;
     double* Y = buf + ncell;
     double* Z = buf + 2 * ncell;
-    double* nf = synthesise(f, coarse, nc, ncell, X, Y, scale);
+    double* nf = synthesise(f, coarse, nc, ncell, X, Y, scale, 0, ncell);
     double* o1 = (nf == X) ? Y : X;
-    // clamp negative densities and keep the total
-    double s0 = 0.0, s1 = 0.0, neg = 0.0;
+    // clamp negative densities and keep the total; a density whose every value is finite with the sign
+    // clear needs neither, and its largest value is the largest bit pattern
+    long long bits = 0;
+    bool clamp = false;
     for (int j = threadIdx.x; j < ncell; j += blockDim.x) {
-        const double v = nf[j];
-        s0 += v;
-        s1 += fmax(v, 0.0);
-        neg += (v < 0.0) ? 1.0 : 0.0;
+        const long long b = __double_as_longlong(nf[j]);
+        clamp |= (unsigned long long)b >= 0x7ff0000000000000ull;
+        bits = b > bits ? b : bits;
     }
-    s0 = block_sum_d(s0, red);
-    s1 = block_sum_d(s1, red);
-    neg = block_sum_d(neg, red);
-    const double resc = (neg > 0.0 && s1 > 0.0 && s0 > 0.0) ? s0 / s1 : 1.0;
     double nmax = 0.0;
-    for (int j = threadIdx.x; j < ncell; j += blockDim.x) {
-        const double v = fmax(nf[j], 0.0) * resc;
-        nf[j] = v;
-        nmax = fmax(nmax, v);
+    if (__syncthreads_or(clamp)) {
+        double s0 = 0.0, s1 = 0.0, neg = 0.0;
+        for (int j = threadIdx.x; j < ncell; j += blockDim.x) {
+            const double v = nf[j];
+            s0 += v;
+            s1 += fmax(v, 0.0);
+            neg += (v < 0.0) ? 1.0 : 0.0;
+        }
+        s0 = block_sum_d(s0, red);
+        s1 = block_sum_d(s1, red);
+        neg = block_sum_d(neg, red);
+        const double resc = (neg > 0.0 && s1 > 0.0 && s0 > 0.0) ? s0 / s1 : 1.0;
+        for (int j = threadIdx.x; j < ncell; j += blockDim.x) {
+            const double v = fmax(nf[j], 0.0) * resc;
+            nf[j] = v;
+            nmax = fmax(nmax, v);
+        }
+        nmax = block_max_d(nmax, red);
+    } else {
+        nmax = __longlong_as_double(block_max_ll(bits, red));
     }
-    nmax = block_max_d(nmax, red);
-    double* mf = synthesise(f, coarse + nc, nc, ncell, o1, Z, scale);
-    for (int j = threadIdx.x; j < ncell; j += blockDim.x) {
+    double* mf = synthesise(f, coarse + nc, nc, ncell, o1, Z, scale, p0, p1);
+    for (int j = p0 + threadIdx.x; j < p1; j += blockDim.x) {
         const double n = nf[j];
         prof_n[j] = (P)n;
         prof_u[j] = (n > 1e-12 * nmax) ? (P)(mf[j] / n) : P(0);
@@ -426,7 +490,7 @@ __global__ void __launch_bounds__(1024) k_refine_pressure(const double* coarse, 
     __shared__ double red[32];
     const double* nf = nullptr;
     const double* mf = nullptr;
-    refine_body(coarse, nc, f, ncell, scale, prof_n, prof_u, buf, red, &nf, &mf);
+    refine_body(coarse, nc, f, ncell, scale, prof_n, prof_u, buf, red, 0, 1, &nf, &mf);
     double* X = buf;
     double* Y = buf + ncell;
     double* Z = buf + 2 * ncell;
@@ -436,7 +500,7 @@ __global__ void __launch_bounds__(1024) k_refine_pressure(const double* coarse, 
     double nmax = 0.0;
     for (int j = threadIdx.x; j < ncell; j += blockDim.x) nmax = fmax(nmax, nf[j]);
     nmax = block_max_d(nmax, red);
-    const double* sf = synthesise(f, coarse + 2 * nc, nc, ncell, free1, W, scale);
+    const double* sf = synthesise(f, coarse + 2 * nc, nc, ncell, free1, W, scale, 0, ncell);
     for (int j = threadIdx.x; j < ncell; j += blockDim.x) {
         const double n = nf[j];
         double t = 0.0;
@@ -448,8 +512,8 @@ __global__ void __launch_bounds__(1024) k_refine_pressure(const double* coarse, 
     }
 }
 
-// Batched restriction + projection for Haar samples summed over coarse bins (one block per
-// realisation): the same arithmetic, in the same order, as pe_coarsen with bin_shift =
+// Batched restriction + projection for Haar samples summed over coarse bins (blocks (r, *) for
+// realisation r): the same arithmetic, in the same order, as pe_coarsen with bin_shift =
 // log2(ncell / n_coarse) followed by pe_ls_project.
 struct ProjDesc {
     const long long* samp;  // row p of this realisation at samp + p * row_stride: [2][nc]
@@ -461,25 +525,43 @@ struct ProjDesc {
     int nc, pad;
 };
 
-__global__ void __launch_bounds__(256) k_restrict_project_batch(const ProjDesc* descs, int K, double dt, double dT)
+// Each sample is converted once, for its pair and its row of csamples (24 realisations of up to 512
+// components, 21 samples: 37 us in a block per realisation, 12 us so).
+constexpr int kProjectBlocks = 8;
+
+__global__ void __launch_bounds__(kProjectThreads) k_restrict_project_batch(const ProjDesc* descs, int K, double dt,
+                                                                            double dT)
 {
+    __shared__ double w[kProjectThreads];
     const ProjDesc d = descs[blockIdx.x];
     const int ncoef = 2 * d.nc;
     const double den = (double)K * (K + 1) * (K + 2) * dt;
-    for (int i = threadIdx.x; i < ncoef; i += blockDim.x) {
+    for (int i0 = blockIdx.y * kProjectThreads; i0 < ncoef; i0 += gridDim.y * kProjectThreads) {
+        const int i = i0 + threadIdx.x;
         const double scale = (i >= d.nc) ? d.scale_m : d.scale_n;
-        double s = 0.0;
-        for (int p = 0; 2 * p <= K; ++p) {
-            const double cK = (double)d.samp[(int64_t)(K - p) * d.row_stride + i] * scale;
-            const double c0 = (double)d.samp[(int64_t)p * d.row_stride + i] * scale;
-            s += 6.0 * (K - 2 * p) / den * (cK - c0);
+        double s = 0.0, last = 0.0;
+        for (int p0 = 0; 2 * p0 <= K; p0 += kProjectThreads) {
+            const int n = min(kProjectThreads, K / 2 + 1 - p0);
+            pair_factors(K, den, p0, n, w);
+            if (i < ncoef) {
+#pragma unroll 4
+                for (int k = 0; k < n; ++k) {
+                    const int p = p0 + k;
+                    const double cK = (double)d.samp[(int64_t)(K - p) * d.row_stride + i] * scale;
+                    const double c0 = (double)d.samp[(int64_t)p * d.row_stride + i] * scale;
+                    s += w[k] * (cK - c0);
+                    if (p == 0) last = cK;
+                    if (d.csamples) {
+                        d.csamples[(size_t)(K - p) * ncoef + i] = cK;
+                        d.csamples[(size_t)p * ncoef + i] = c0;
+                    }
+                }
+            }
         }
-        const double last = (double)d.samp[(int64_t)K * d.row_stride + i] * scale;
-        d.slope[i] = s;
-        d.coarse[i] = last + (dT - K * dt) * s;
-        if (d.csamples)
-            for (int p = 0; p <= K; ++p)
-                d.csamples[(size_t)p * ncoef + i] = (double)d.samp[(int64_t)p * d.row_stride + i] * scale;
+        if (i < ncoef) {
+            d.slope[i] = s;
+            d.coarse[i] = last + (dT - K * dt) * s;
+        }
     }
 }
 
@@ -497,7 +579,7 @@ void make_proj_desc(void* out, const int64_t* samp, int64_t row_stride, int ncel
 
 int launch_restrict_project_batch(const void* descs, int R, int K, double dt, double dT, cudaStream_t s)
 {
-    k_restrict_project_batch<<<R, 256, 0, s>>>(static_cast<const ProjDesc*>(descs), K, dt, dT);
+    k_restrict_project_batch<<<dim3(R, kProjectBlocks), kProjectThreads, 0, s>>>(static_cast<const ProjDesc*>(descs), K, dt, dT);
     return launch_status();
 }
 
@@ -671,8 +753,8 @@ extern "C" PE_API int pe_ls_project(const double* samples, int32_t K, int32_t nc
                                     double* slope, void* stream)
 {
     if (!samples || !out || K < 1 || ncoef < 1 || !(dt > 0.0)) return PE_EINVAL;
-    const int block = 256;
-    k_ls_project<<<(ncoef + block - 1) / block, block, 0, (cudaStream_t)stream>>>(samples, K, ncoef, dt, dT, out, slope);
+    k_ls_project<<<(ncoef + kProjectThreads - 1) / kProjectThreads, kProjectThreads, 0, (cudaStream_t)stream>>>(
+        samples, K, ncoef, dt, dT, out, slope);
     return launch_status();
 }
 
@@ -691,7 +773,7 @@ int launch_refine_batch(const void* descs, int R, int wavelet, int max_ncell, cu
     const size_t smem = 3 * sizeof(double) * (size_t)max_ncell;
     if (R < 1 || smem > (size_t)max_smem_optin() || !wavelet_ok(wavelet)) return PE_EINVAL;
     if (ensure_smem((const void*)k_refine_batch, smem) != PE_OK) return PE_ECUDA;
-    k_refine_batch<<<R, 1024, smem, s>>>(static_cast<const RefineDesc*>(descs), make_filter(wavelet));
+    k_refine_batch<<<dim3(R, kRefineBatchParts), 1024, smem, s>>>(static_cast<const RefineDesc*>(descs), make_filter(wavelet));
     return launch_status();
 }
 }  // namespace pe
@@ -705,7 +787,7 @@ static int refine_into(const double* coarse, int32_t n_coarse, int32_t wavelet, 
     const size_t smem = 3 * sizeof(double) * (size_t)ncell;
     if (smem > (size_t)max_smem_optin()) return PE_EINVAL;
     if (ensure_smem((const void*)k_refine<P>, smem) != PE_OK) return PE_ECUDA;
-    k_refine<P><<<1, 1024, smem, (cudaStream_t)stream>>>(coarse, n_coarse, make_filter(wavelet), ncell,
+    k_refine<P><<<kRefineParts, 1024, smem, (cudaStream_t)stream>>>(coarse, n_coarse, make_filter(wavelet), ncell,
                                                          pow(2.0, 0.5 * ilog2(ncell)), prof_n, prof_u);
     return launch_status();
 }

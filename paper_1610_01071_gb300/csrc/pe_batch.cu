@@ -9,6 +9,7 @@
 #include <stdlib.h>
 #include <string.h>
 
+#include <algorithm>
 #include <map>
 #include <mutex>
 #include <vector>
@@ -310,6 +311,8 @@ extern "C" PE_API int pe_batch_create(pe_ctx* const* ctxs, int32_t n, void* scra
             }
         if (!placed) b->fgroups.push_back({x->cfg.ncell, {r}});
     }
+    // the largest grids' clusters need the most free SMs together: they start first
+    std::stable_sort(b->fgroups.begin(), b->fgroups.end(), [](const auto& x, const auto& y) { return x.ncell > y.ncell; });
     int rc = PE_OK;
     if (cudaEventCreateWithFlags(&b->ev_fork, cudaEventDisableTiming) != cudaSuccess) rc = PE_ECUDA;
     for (size_t k = 0; rc == PE_OK && k < b->fgroups.size(); ++k) {

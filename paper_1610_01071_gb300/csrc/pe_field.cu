@@ -507,8 +507,11 @@ __global__ void __launch_bounds__(kNewtonMaxThreads, 1) k_newton_cluster(FieldDe
 }
 
 // One cluster per realisation: cluster c solves descs[c]; extrap (a solve inside a burst, not the one
-// that starts it) applies to every realisation.
-__global__ void __launch_bounds__(kNewtonMaxThreads, 1) k_newton_batch(const FieldDesc* descs, int extrap)
+// that starts it) applies to every realisation. Two blocks to an SM: the groups of an ensemble's grid
+// sizes run side by side, and with one block to an SM (128 registers) 24 realisations of 512 to 8192
+// nodes want 169 SMs, which left clusters of 16 waiting for a second wave (20 bytes spill at 64; a
+// macro step of those realisations 8.93 ms, 8.65 ms so).
+__global__ void __launch_bounds__(kNewtonMaxThreads, 2) k_newton_batch(const FieldDesc* descs, int extrap)
 {
     cg::cluster_group cluster = cg::this_cluster();
     FieldDesc d = descs[blockIdx.x / cluster.num_blocks()];

@@ -55,14 +55,14 @@ KERNEL_BYTES = {
 # summarised in profiles/, each valid while the particle kernels' device code
 # (kernel_source_hash) hashes to the value it was taken with.
 NCU_TRAFFIC = {
-    "push_sample": {"source_hash": "173582129c21fd7b", "bytes": 270.715904e6 + 145.457152e6},
-    "push": {"source_hash": "173582129c21fd7b", "bytes": 270.730496e6 + 145.774336e6},
-    "sample": {"source_hash": "173582129c21fd7b", "bytes": 270.679552e6 + 3.367168e6},
-    "deposit": {"source_hash": "173582129c21fd7b", "bytes": 203.015936e6 + 2.963968e6},
-    "push_sample_ps": {"source_hash": "173582129c21fd7b", "bytes": 270.272256e6 + 145.230080e6},
-    "push_sample_psw": {"source_hash": "173582129c21fd7b", "bytes": 270.507520e6 + 145.440768e6},
-    "push_sample_pressure": {"source_hash": "173582129c21fd7b", "bytes": 270.752512e6 + 145.262592e6},
-    "load": {"source_hash": "173582129c21fd7b", "bytes": 0.574720e6 + 207.112192e6},
+    "push_sample": {"source_hash": "1a882e953c11d01d", "bytes": 270.713088e6 + 145.202944e6},
+    "push": {"source_hash": "1a882e953c11d01d", "bytes": 270.704640e6 + 146.609664e6},
+    "sample": {"source_hash": "1a882e953c11d01d", "bytes": 270.663168e6 + 3.001856e6},
+    "deposit": {"source_hash": "1a882e953c11d01d", "bytes": 203.020544e6 + 2.987264e6},
+    "push_sample_ps": {"source_hash": "1a882e953c11d01d", "bytes": 270.277632e6 + 145.245696e6},
+    "push_sample_psw": {"source_hash": "1a882e953c11d01d", "bytes": 270.512128e6 + 145.571840e6},
+    "push_sample_pressure": {"source_hash": "1a882e953c11d01d", "bytes": 270.721280e6 + 145.230848e6},
+    "load": {"source_hash": "1a882e953c11d01d", "bytes": 0.577280e6 + 207.349248e6},
 }
 
 

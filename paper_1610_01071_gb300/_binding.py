@@ -278,7 +278,8 @@ def field(rho, ncell, dx, s_w, phi, mode="boltzmann", tol=1e-11, maxit=50, statu
     dev = rho.device
     E = torch.empty(ncell, dtype=torch.float64, device=dev)
     Ef = torch.empty(ncell, dtype=torch.float32, device=dev)
-    # every solve writes all four words; zeroing them first was one more launch (a call on 4096 nodes: 33 us, 21 us without)
+    # every solve writes all four words; zeroing them first was one more launch (a call on 4096
+    # nodes: 33 us, 21 us without)
     diag = torch.empty(4, dtype=torch.int32, device=dev)
     status = _status(status, dev)
     if boundary == "periodic":

@@ -166,9 +166,13 @@ struct TcEpi {
 // Layer of a small batch (at most kSmallBatch rows; the gated macro step evaluates one): the
 // product with its roles exchanged, C^T[n][b] = sum_k W[n][k] x[b][k], 128 outputs per block as the
 // MMA's rows and the batch as its 32 columns. A thread then finishes one output, where the other
-// form leaves the whole epilogue of a row to two lanes of the block. The weights are loaded before
-// the wait for the previous layer. Same sums as the other form (the accumulation runs over k in
-// the same order).
+// form leaves the whole epilogue of a row to two lanes of the block. Same sums as the other form
+// (the accumulation runs over k in the same order).
+//
+// The weights are loaded before the wait for the previous layer, so whatever writes them (Adam, a
+// parameter upload) must have ended before the first layer starts. k_prep, the first kernel of every
+// evaluation, sees to that: it releases the first layer only after its own wait. The layers
+// themselves may release at once: nothing between k_prep and the last of them writes weights.
 constexpr int kSmallBatch = 32;
 constexpr int kSmallStages = 8;  // K = 512 in flight at once
 constexpr int kSmallABytes = 128 * tc::kBK * 2, kSmallBBytes = kSmallBatch * tc::kBK * 2;
@@ -418,8 +422,10 @@ __global__ void __launch_bounds__(128) k_prep(const T* __restrict__ X, const flo
                                               const float* __restrict__ mu_o, const float* __restrict__ sd_o,
                                               __nv_bfloat16* __restrict__ xz, float* __restrict__ tz)
 {
-    grid_release();
+    // in this order: a small evaluation's layers read the weights before their own wait, and Adam may
+    // be the kernel that this one waits for
     grid_wait();
+    grid_release();
     const int i = blockIdx.x;
     int64_t r = rows ? rows[i] : i;
     int s = 0;

@@ -582,11 +582,11 @@ __device__ __forceinline__ void particle_chunk(const PushParams& P, int64_t begi
         if (kBin && bs.ok) bin_add(q3);
         if (kWrite && bad) {
             const int4 c = cell4[g];
-            const float4 t = th4[g], v = v4[g];
-            if (bad & 1u) co.x = c.x, to.x = t.x, vo.x = v.x, wo.x = wa.x;
-            if (bad & 2u) co.y = c.y, to.y = t.y, vo.y = v.y, wo.y = wa.y;
-            if (bad & 4u) co.z = c.z, to.z = t.z, vo.z = v.z, wo.z = wa.z;
-            if (bad & 8u) co.w = c.w, to.w = t.w, vo.w = v.w, wo.w = wa.w;
+            const float4 t = th4[g], v = v4[g], w = w4[g];
+            if (bad & 1u) co.x = c.x, to.x = t.x, vo.x = v.x, wo.x = wa.x = w.x;
+            if (bad & 2u) co.y = c.y, to.y = t.y, vo.y = v.y, wo.y = wa.y = w.y;
+            if (bad & 4u) co.z = c.z, to.z = t.z, vo.z = v.z, wo.z = wa.z = w.z;
+            if (bad & 8u) co.w = c.w, to.w = t.w, vo.w = v.w, wo.w = wa.w = w.w;
         }
         if (kWrite && act) {
             cell4[g] = co;

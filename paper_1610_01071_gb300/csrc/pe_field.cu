@@ -260,11 +260,16 @@ struct NewtonShared {
                                                      // the residual it leaves
 };
 
-// A unit's first row given the separators around it (the owner and its left neighbour evaluate
-// this same function, so the neighbour's halo stays bit-identical to the owner's node).
+// An interior row y - g s_left - h s_right given the separators around it, its operations spelled out: the
+// owner of a unit's first row and the left neighbour that keeps it as a halo round alike whatever the
+// compiler makes of the code around them, so the halo stays bit-identical to the owner's node.
+__device__ __forceinline__ float interior_row(float y, float g, float h, float s_left, float s_right)
+{
+    return __fmaf_rn(-h, s_right, __fmaf_rn(-g, s_left, y));
+}
 __device__ __forceinline__ float edge_row(const float4& f, float s_left, float s_right)
 {
-    return f.x - f.y * s_left - f.z * s_right;
+    return interior_row(f.x, f.y, f.z, s_left, s_right);
 }
 
 // Solver body for the realisation of this cluster: B = ncell / G nodes per block, one per thread
@@ -416,7 +421,7 @@ __device__ __forceinline__ void newton_body(const FieldDesc& d, cg::cluster_grou
         if (act) {
             if (lane == sep) x = Sw_r;
             else if (i == 0) x = edge_row(own.first, Sl, Sr);  // the form the left neighbour uses for its halo
-            else x = rhs - gc * Sw_l - hc * Sw_r;
+            else x = interior_row(rhs, gc, hc, Sw_l, Sw_r);
         }
         // the updates of the halo nodes: the left neighbour's separator, the right neighbour's first row
         float4 right = wrow[w + 1 < W ? w + 1 : w].first;
@@ -460,9 +465,9 @@ __device__ __forceinline__ void newton_body(const FieldDesc& d, cg::cluster_grou
             double xs = x1;
             if (m > 2.0f) {  // damped
                 const double scale = 2.0 / (double)m;
-                xs = scale * x1;
-                pn = p + xs;
-                hn = halo + scale * xh;
+                xs = __dmul_rn(scale, x1);  // product and sum apart, in the owner and in the halo alike
+                pn = __dadd_rn(p, xs);
+                hn = __dadd_rn(halo, __dmul_rn(scale, xh));
             }
             if (boltz) gn = (fabs(xs) <= 0.03125) ? gj * exp_small(xs) : exp(pn);
             else gn = 1.0 + pn;

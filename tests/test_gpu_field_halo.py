@@ -1,0 +1,34 @@
+"""Field solves: the returned field is the centred difference of the returned potential, to the bit, at
+every node. Warps and blocks difference their edge nodes against copies of the neighbours' potential
+that they advance themselves, so one copy off by a rounding shows here."""
+import pytest
+import torch
+
+import paper_1610_01071_gb300 as pe
+
+pytestmark = pytest.mark.gpu
+DEV = torch.device("cuda:0")
+S_W = 20
+
+
+def _rho(n, kind, g):
+    x = torch.arange(n, dtype=torch.float64, device=DEV) / n
+    noise = 1.0 + 0.05 * torch.randn(n, generator=g, dtype=torch.float64, device=DEV)
+    base = torch.sigmoid((0.0625 - (x - 0.5).abs()) * 200.0) if kind == "absorbing" else 1.0 + 0.5 * torch.sin(6.2831853 * x)
+    return torch.round((base * noise).clamp(min=0.0) * 2.0 ** (S_W + 24)).to(torch.int64)
+
+
+@pytest.mark.parametrize("boundary", ["periodic", "absorbing"])
+@pytest.mark.parametrize("n", [8, 32, 64, 256, 512, 1024, 4096, 8192])
+def test_the_field_is_the_difference_of_the_potential(n, boundary):
+    g = torch.Generator(device=DEV).manual_seed(n)
+    for mode in ("boltzmann", "linearized"):
+        for dx, phi0, maxit in ((0.5, 0.0, 200), (0.3, 0.0, 1), (0.3, -9.0, 3), (0.5, 6.0, 200), (0.37, 0.0, 0)):  # +-: damped steps
+            rho = _rho(n, boundary, g)
+            phi = phi0 * torch.rand(n, generator=g, dtype=torch.float64, device=DEV)
+            E, Ef, _ = pe.field(rho, n, dx, S_W, phi, mode=mode, tol=1e-10, maxit=maxit, boundary=boundary)
+            want = (phi.roll(1) - phi.roll(-1)) * (0.5 / dx)
+            if boundary == "absorbing":
+                want[0] = want[-1] = 0.0
+            assert torch.equal(E, want), (mode, dx, phi0, int((E != want).sum()))
+            assert torch.equal(Ef, want.float())

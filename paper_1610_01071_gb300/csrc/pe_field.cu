@@ -8,6 +8,7 @@
 // control volume is the half cell inside the domain).
 #include <cooperative_groups.h>
 #include <cuda_runtime.h>
+#include <float.h>
 #include <stdint.h>
 #include <string.h>
 
@@ -623,8 +624,10 @@ static FieldDesc field_desc(const int64_t* rho, int ncell, double dx, int s_w, i
                             double* phi, double* E, float* Ef, int32_t* diag, uint32_t* status, double* phi_prev,
                             int extrap, int clear)
 {
+    float ftol = (float)tol;
+    if (tol > 0.0 && ftol < FLT_MIN) ftol = FLT_MIN;  // a positive tolerance stays one: an update of 0 meets it
     return FieldDesc{reinterpret_cast<long long*>(const_cast<int64_t*>(rho)), phi, E, Ef, diag, status, 1.0 / (dx * dx), 0.5 / dx,
-                     (float)tol, s_w + 24, ncell, mode, maxit, walls ? 1 : 0, phi_prev, extrap ? 1 : 0, clear, nullptr};
+                     ftol, s_w + 24, ncell, mode, maxit, walls ? 1 : 0, phi_prev, extrap ? 1 : 0, clear, nullptr};
 }
 
 size_t field_desc_size() { return sizeof(FieldDesc); }

@@ -32,3 +32,13 @@ def test_the_field_is_the_difference_of_the_potential(n, boundary):
                 want[0] = want[-1] = 0.0
             assert torch.equal(E, want), (mode, dx, phi0, int((E != want).sum()))
             assert torch.equal(Ef, want.float())
+
+
+@pytest.mark.parametrize("n", [64, 1024])
+def test_a_tolerance_below_single_precision_still_ends_an_exact_solve(n):
+    rho = torch.full((n,), 1 << (S_W + 24), dtype=torch.int64, device=DEV)  # density 1: phi = 0 is exact
+    phi = torch.zeros(n, dtype=torch.float64, device=DEV)
+    st = torch.zeros(1, dtype=torch.int32, device=DEV)
+    E, _, diag = pe.field(rho, n, 0.5, S_W, phi, mode="linearized", tol=1e-60, maxit=9, status=st)
+    assert diag.tolist()[:2] == [1, 1] and int(st.item()) == 0
+    assert float(E.abs().max()) == 0.0 and float(phi.abs().max()) == 0.0

@@ -704,9 +704,12 @@ __device__ __forceinline__ V block_exclusive_scan(V x, V* total, V* wsum)
     return base + incl - x;
 }
 
-__global__ void __launch_bounds__(kPoissonThreads) k_poisson_periodic(long long* rho_i, long long* rho_e, int clear,
-                                                                      int n, double dx, double nscale, double* phi,
-                                                                      double* E, float* Ef)
+// clear: both deposits are zeroed for the pushes that follow, in coalesced stores behind the block's reads
+// (a store after each node's reads kept the loads from running ahead: 8192 nodes in 86 us, 72 us so, and
+// 69.5 us without the clear).
+__global__ void __launch_bounds__(kPoissonThreads)
+    k_poisson_periodic(long long* __restrict__ rho_i, long long* __restrict__ rho_e, int clear, int n, double dx,
+                       double nscale, double* phi, double* E, float* Ef)
 {
     extern __shared__ double psh[];
     double* F = psh;      // [n]: net charge, then the face fields F_{j+1/2}
@@ -724,12 +727,13 @@ __global__ void __launch_bounds__(kPoissonThreads) k_poisson_periodic(long long*
     if (act)
         for (int k = 0; k < m; ++k) {
             const double q = (double)(rho_i[j0 + k] - rho_e[j0 + k]);
-            if (clear) rho_i[j0 + k] = rho_e[j0 + k] = 0;  // the pushes that follow accumulate
             F[j0 + k] = q;
             s += q;
         }
     double tot;
-    const double off = block_exclusive_scan(s, &tot, wd);
+    const double off = block_exclusive_scan(s, &tot, wd);  // past its barriers every deposit has been read
+    if (clear)
+        for (int j = t; j < n; j += (int)blockDim.x) rho_i[j] = rho_e[j] = 0;
     // face fields before the gauge: F_{j+1/2} - F_{-1/2} = dx nscale (S_j - (j + 1) <S>)
     const double mean = tot / n, c = dx * nscale;
     double fs = 0.0;

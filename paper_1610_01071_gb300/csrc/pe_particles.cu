@@ -355,11 +355,12 @@ __device__ __forceinline__ void deposit_direct(const SmemGrid& g, int c, float t
 // three cells, the window moves (warp-uniformly): to the lowest cell, or (CENTRE) where the cells
 // spread over more than three (velocities without order in the cell, few particles per cell) to
 // the middle of the spread, so that it takes the densest cells and fewer particles go straight to
-// the grid, one lane at a time. The fused passes are bound by issued instructions and gain
-// (wavelet form, 1500 ions per cell in no order: 31 -> 25 us per pass of 1.5e6; batch of mixed sizes
-// 386 -> 360 us); the plain push is bound by the shared reductions there and keeps the lowest cell
-// (electrons crossing a cell per step: 62 us per pass of 2^23, 70 with the middle). Called by all
-// 32 lanes.
+// the grid, one lane at a time. The fused passes with binned or phase-space samples are bound by
+// issued instructions and gain (wavelet form, 1500 ions per cell in no order: 31 -> 25 us per pass of
+// 1.5e6; batch of mixed sizes 386 -> 360 us). The plain push and the passes with nodal samples are
+// bound by the shared reductions and keep the lowest cell (electrons crossing a cell per step: 62 us
+// per push of 2^23, 70 with the middle; nodal push + sample of 2^24 ordered ions: 386 us, 397 with the
+// middle, whose state also spills more registers there). Called by all 32 lanes.
 template <bool CENTRE>
 __device__ __forceinline__ void deposit_group(WarpWindow& win, const SmemGrid& g, int ncell, int mask, const int4& c,
                                               const float4& th, int32_t q0, int32_t q1, int32_t q2, int32_t q3,
@@ -608,7 +609,7 @@ __device__ __forceinline__ void particle_chunk(const PushParams& P, int64_t begi
             bw.end(bsn, bsm, bse);
         else if constexpr (kBin)
             bw.end(bsn, bsm);
-        if (kRho) deposit_group<Tr::sample>(win, grho, P.ncell, P.mask, co, to, q0, q1, q2, q3, e0, e1, e2, e3);
+        if (kRho) deposit_group<Tr::binned || Tr::ps>(win, grho, P.ncell, P.mask, co, to, q0, q1, q2, q3, e0, e1, e2, e3);
     }
     if (kRho) win.flush_first(grho, 4);
     for (int64_t i = (gb1 << 2) + threadIdx.x; i < end; i += blockDim.x) {  // ragged tail (< 4 particles)

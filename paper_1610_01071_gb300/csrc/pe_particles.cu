@@ -102,12 +102,17 @@ struct ModeTraits {
     // passes (three blocks an SM) and the deposit gain from it; the other passes, at four blocks
     // an SM with their loads already in flight, run faster on direct loads and a larger L1
     static constexpr bool stage = ps || MODE == kDeposit;
-    // cell range checked once per group of four (lanes past a slice's end carry weightless
-    // particles) instead of particle by particle: push 2^23 particles 38.6 -> 35.0 us (the memory
-    // bandwidth), sample 2^24 73.3 -> 70.2; the fused passes have no register left for it (263 -> 270
-    // us on the slab)
-    static constexpr bool group_check = !(push && sample);
 };
+
+// Cell range checked once per group of four (lanes past a slice's end carry weightless particles) instead of
+// particle by particle: push of 2^23 particles 38.6 -> 35.0 us (the memory bandwidth), sample of 2^24 73.3 ->
+// 70.2. Not in the fused passes, which have no register left for it (263 -> 270 us on the slab), nor in the
+// nodal sample of three moments, whose fourth block per SM it would cost (64 -> 72 registers; 2^24 unordered
+// particles 122 -> 140 us), nor in the push between walls, which tests every particle's weight anyway
+// (2^24 particles 83.7 us without it, 85.3 with).
+template <int MODE, bool WALLS>
+constexpr bool kGroupCheck = !(ModeTraits<MODE>::push && (ModeTraits<MODE>::sample || WALLS)) &&
+                             !(ModeTraits<MODE>::energy && !ModeTraits<MODE>::binned);
 
 // Fixed-point value rn(x 2^s); records in *ovf whether it left the range |q| <= 2^23.
 __device__ __forceinline__ int32_t fx_weight(float x, float scale, bool* ovf)
@@ -215,7 +220,7 @@ __device__ __forceinline__ bool process(const PushParams& P, const FieldTab& ft,
     if (Tr::energy) bs.eq = 0;
     bs.tq = 0u;
     bs.ok = false;
-    if (!Tr::group_check) {
+    if (!kGroupCheck<MODE, WALLS>) {
         if (!act) return false;  // a lane past the end of its warp's slice
         if ((unsigned)c >= (unsigned)P.ncell) {
             raise_flag(P.status, PE_FLAG_RANGE);
@@ -416,6 +421,7 @@ __device__ __forceinline__ void particle_chunk(const PushParams& P, int64_t begi
     constexpr bool kBin = Tr::binned;
     constexpr bool kWrite = Tr::push;
     constexpr bool kNeedV = (MODE != kDeposit);
+    constexpr bool kGroup = kGroupCheck<MODE, WALLS>;
 
     const int c_first = (begin < end) ? (P.cell[begin] & P.mask) : 0;
 
@@ -531,7 +537,7 @@ __device__ __forceinline__ void particle_chunk(const PushParams& P, int64_t begi
         const int64_t g = gs + lane;
         const bool act = g < g1;
         // a lane past the end of its warp's slice: weightless particles in a cell of the window
-        const int c_idle = Tr::group_check ? (win.base + 1) & P.mask : 0;
+        const int c_idle = kGroup ? (win.base + 1) & P.mask : 0;
         int4 ca = make_int4(c_idle, c_idle, c_idle, c_idle);
         float4 ta = make_float4(0.f, 0.f, 0.f, 0.f), va = ta, wa = ta;
         if (Tr::stage) {
@@ -554,7 +560,7 @@ __device__ __forceinline__ void particle_chunk(const PushParams& P, int64_t begi
         // cells outside [0, ncell) (any bit beyond the mask): flagged, carried as weightless and left
         // as they are in memory
         uint32_t bad = 0u;
-        if (Tr::group_check && __any_sync(0xFFFFFFFFu, ((ca.x | ca.y | ca.z | ca.w) & ~P.mask) != 0)) {
+        if (kGroup && __any_sync(0xFFFFFFFFu, ((ca.x | ca.y | ca.z | ca.w) & ~P.mask) != 0)) {
             bad = ((ca.x & ~P.mask) ? 1u : 0u) | ((ca.y & ~P.mask) ? 2u : 0u) | ((ca.z & ~P.mask) ? 4u : 0u) |
                   ((ca.w & ~P.mask) ? 8u : 0u);
             if (bad) raise_flag(P.status, PE_FLAG_RANGE);
@@ -618,7 +624,7 @@ __device__ __forceinline__ void particle_chunk(const PushParams& P, int64_t begi
         int32_t q;
         const float vi = kNeedV ? P.v[i] : 0.f;
         const float wi = P.w[i];
-        if (Tr::group_check && (P.cell[i] & ~P.mask)) {
+        if (kGroup && (P.cell[i] & ~P.mask)) {
             raise_flag(P.status, PE_FLAG_RANGE);
             continue;
         }

@@ -189,6 +189,17 @@ __device__ __forceinline__ uint32_t eq_point_of_slot(uint32_t s, int64_t n)
                                               : s;
 }
 
+// Cell at which the walk to the cell of slot i's point pt begins, in the global table; the slots from
+// `full` on are the ragged end of a block's chunk. Where the table ascends that is the point's own
+// cell. Where it does not (negative densities) several cells hold a point, and which one the walk ends
+// in depends on its start: there the start belongs to the smallest point of the slot's group of four.
+__device__ __forceinline__ int eq_walk_start(const EqTable& tab, int ncell, int64_t n, int64_t i, int64_t full, uint32_t pt)
+{
+    if (i < full && !__ldg(tab.mono))
+        for (uint32_t k = 0; k < 4u; ++k) pt = min(pt, eq_point_of_slot(((uint32_t)i & ~3u) + k, n));
+    return eq_cell_of(tab, ncell, pt);
+}
+
 // The cells of a thread block's points, in shared memory: constants once per cell and block (the
 // storage order takes a lane back and forth between the cells of 4096 consecutive points, and
 // forming the constants at each change, ~40 FP64 instructions of 64 to 76 cycles, took most of

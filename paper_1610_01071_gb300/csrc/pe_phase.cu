@@ -1026,7 +1026,7 @@ __global__ void __launch_bounds__(256, 4) k_ps_quiet_start_equal(PSEqLoad P)
 #pragma unroll 1
     for (int64_t i = a + (threadIdx.x & 31); i < b; i += 32) {
         const uint32_t pt = eq_point_of_slot((uint32_t)i, P.n);
-        int c = st.n ? 0 : eq_cell_of(P.tab, P.ncell, pt);
+        int c = st.n ? 0 : eq_walk_start(P.tab, P.ncell, P.n, i, end & ~int64_t(3), pt);
         float t, vv;
         ps_eq_one(P, st, pt, c, t, vv, cur, hint);
         P.cell[i] = c;

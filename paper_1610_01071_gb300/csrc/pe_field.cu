@@ -65,7 +65,9 @@ namespace pe {
 // min g' in every component. Before a linear solve |F| is the FP64 residual; after one, the
 // residual that the update leaves is bounded in FP32 as |r - J x| + g x^2 (1/2 + |x|) plus the
 // rounding of that evaluation, which ends the usual solve after its second update without a
-// third residual and reduction only to learn that it has converged.
+// third residual and reduction only to learn that it has converged. Grids below 32 nodes stop by the
+// update alone: their idle lanes count as min g' = 0. One more update costs them little and leaves the
+// potential at rounding instead of at the tolerance.
 
 constexpr int kClusterMinCells = 512;   // grids at least this large use the multi-SM solver
 constexpr int kClusterMax = 16;
@@ -327,7 +329,7 @@ __device__ __forceinline__ void newton_body(const FieldDesc& d, cg::cluster_grou
         const float bd = f32_of(diag0 + (boltz ? gj : 1.0));
         const float gf = boltz ? f32_of(gj) : 1.0f;
         const float fw = warp_max_bits(act ? __float_as_uint(fabsf(r)) : 0u);
-        const float gw = warp_min_bits(act ? gf : 3.0e38f);
+        const float gw = warp_min_bits(act ? gf : 0.0f);  // below 32 nodes: no bound, see above
         // ---- warp interiors: x = rhs - gc S_left - hc S_right
         float a = 0.0f, b = 1.0f, c = 0.0f, rhs = 0.0f, gc = 0.0f, hc = 0.0f;
         if (act && lane != sep) {  // the separator holds an identity row in the warp's reduction

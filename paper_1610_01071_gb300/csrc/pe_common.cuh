@@ -637,7 +637,8 @@ struct BinWindow3 {
                                         const BinGrid& gm, const BinGrid& ge)
     {
         // branches here, unlike BinWindow: with three moments the predicated adds cost more issue slots
-        // than the divergence (pass of 2^24 ions 145 us against 137 us)
+        // than the divergence (push + sample of 2^24 ordered ions on 4096 cells, calls queued back to back:
+        // 112.9 us, 121.0 us predicated)
         const int d = (b - w.K) & (gn.nb - 1);
         if (d == 0) {
             w.n0 += wq;

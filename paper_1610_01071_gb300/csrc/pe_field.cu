@@ -37,8 +37,9 @@ namespace pe {
 //  - one block barrier and one cluster barrier per linear solve: every warp solves the block's
 //    and the cluster's separator systems itself instead of waiting for one warp's result. The
 //    second exchange of an iteration (largest update) runs behind the FP64 update.
-// One solve of a time loop (two updates; the walls' about seven) takes 7.1 us on 128 nodes (15.1
-// us before these points), 10.4 on 1024 (18.0), 12.8 on 4096 (23.3) and 37 on 8192 with walls (60).
+// One solve of a burst (two updates; the walls' about seven), the mean of 40 cold launches under ncu:
+// 8.3 us on 128 nodes (15.2 before these points), 11.0 on 1024 (17.8), 13.8 on 4096 (23.4), 39 on 8192
+// with walls (63).
 //
 // Precision: phi, exp(phi), the Newton residual and the update are FP64; the Jacobian
 // correction J d = -F is solved in FP32. This is Newton's method with an inexact linear solve

@@ -10,10 +10,10 @@
 //
 // What bounds a training step: the chain of its launches. Each product of the usual widths (512,
 // batch 2048) is under 1 us of tensor-core time, so the work around it sets the time: a step
-// of 512-512-512-512-512 at batch 2048 took 266 us in 25 launches (epilogues writing every row
+// of 512-512-512-512-512 at batch 2048 took 259 us in 20 launches (epilogues writing every row
 // in 4-byte pieces and a second time transposed, an Adam kernel finding each weight's place with
-// 64-bit divisions) and takes 95 us in 10, each started under its predecessor's tail
-// (programmatic dependent launch).
+// 64-bit divisions) and takes 91 us in 10, each started under its predecessor's tail
+// (programmatic dependent launch); both as the mean of 200 steps of one call.
 //
 // Storage (caller-owned arena, see pe_mlp_layout_for): FP32 master parameters (the flat
 // vector W_1 [d1][d0], b_1, W_2, ...), their BF16 mirror and its per-layer transposes used by

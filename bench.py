@@ -55,14 +55,14 @@ KERNEL_BYTES = {
 # summarised in profiles/, each valid while the particle kernels' device code
 # (kernel_source_hash) hashes to the value it was taken with.
 NCU_TRAFFIC = {
-    "push_sample": {"source_hash": "1a882e953c11d01d", "bytes": 270.713088e6 + 145.202944e6},
-    "push": {"source_hash": "1a882e953c11d01d", "bytes": 270.704640e6 + 146.609664e6},
-    "sample": {"source_hash": "1a882e953c11d01d", "bytes": 270.663168e6 + 3.001856e6},
-    "deposit": {"source_hash": "1a882e953c11d01d", "bytes": 203.020544e6 + 2.987264e6},
-    "push_sample_ps": {"source_hash": "1a882e953c11d01d", "bytes": 270.277632e6 + 145.245696e6},
-    "push_sample_psw": {"source_hash": "1a882e953c11d01d", "bytes": 270.512128e6 + 145.571840e6},
-    "push_sample_pressure": {"source_hash": "1a882e953c11d01d", "bytes": 270.721280e6 + 145.230848e6},
-    "load": {"source_hash": "1a882e953c11d01d", "bytes": 0.577280e6 + 207.349248e6},
+    "push_sample": {"source_hash": "59ec6722d44334d3", "bytes": 270.713856e6 + 145.255424e6},
+    "push": {"source_hash": "59ec6722d44334d3", "bytes": 270.749440e6 + 146.391552e6},
+    "sample": {"source_hash": "59ec6722d44334d3", "bytes": 270.665472e6 + 3.063040e6},
+    "deposit": {"source_hash": "59ec6722d44334d3", "bytes": 203.020544e6 + 2.969856e6},
+    "push_sample_ps": {"source_hash": "59ec6722d44334d3", "bytes": 270.274816e6 + 145.283584e6},
+    "push_sample_psw": {"source_hash": "59ec6722d44334d3", "bytes": 270.511104e6 + 145.423872e6},
+    "push_sample_pressure": {"source_hash": "59ec6722d44334d3", "bytes": 270.720512e6 + 145.254912e6},
+    "load": {"source_hash": "59ec6722d44334d3", "bytes": 0.581888e6 + 207.336704e6},
 }
 
 
